@@ -110,7 +110,7 @@ class State:
     pass
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed * 7919 + 17)
     cpu = torch.Generator()
@@ -138,20 +138,26 @@ def prepare(case, seed):
     st.kpe_pages = torch.empty(n_pages, page, 64, dtype=torch.bfloat16, device="cuda").normal_(generator=gen)
     lens = lens.to(torch.int32)
 
-    kind = case["kind"]
+    st.table, st.lens = table, lens
+    # the prompts of a tree's branches
+    st.parts = [(_normal(gen, n, 512), _normal(gen, n, 64)) for n in _branch_lengths(case)]
+    return st
+
+
+def prepare(case, seed):
+    st = _inputs(case, seed)
+    H, B, page, kind = case["heads"], case["batch"], case["page"], case["kind"]
+    st.parts, parts_in = [], st.parts
     if kind == "host":
         st.q_nope, st.q_pe = st.q_nope.cpu().pin_memory(), st.q_pe.cpu().pin_memory()
-        st.table, st.lens = table.pin_memory(), lens.pin_memory()
+        st.table, st.lens = st.table.pin_memory(), st.lens.pin_memory()
         st.out = torch.empty(B, H, 128, dtype=torch.bfloat16).pin_memory()
     else:
-        st.table, st.lens = table.cuda(), lens.cuda()
+        st.table, st.lens = st.table.cuda(), st.lens.cuda()
     if kind == "tree":
         dims = b.make_dims(H)
         root = b.typhoon_mla_prepare_shared(dims, st.ckv, st.kpe, st.w_uk, st.w_uv)
-        parts = []
-        for n in _branch_lengths(case):
-            ckv, kpe = _normal(gen, n, 512), _normal(gen, n, 64)
-            parts.append(b.typhoon_mla_prepare_shared(dims, ckv, kpe, st.w_uk, st.w_uv))
+        parts = [b.typhoon_mla_prepare_shared(dims, ckv, kpe, st.w_uk, st.w_uv) for ckv, kpe in parts_in]
         st.levels = [([root], [0, B]), (parts, _groups(case))]
         size = b.typhoon_mla_tree_workspace_bytes(st.levels, B, st.max_pages, page)
         st.workspace = torch.empty(size, dtype=torch.uint8, device="cuda")
@@ -215,6 +221,63 @@ def work(case):
         flops += 262144.0 * H * case["prefix"]
         bytes_ += (512.0 * H + 2 * 1152.0) * case["prefix"] + 262144.0 * H
     return {"bytes": bytes_, "flops": flops}
+
+
+def _e4m3(x):
+    """The values that the 8-bit option keeps: bf16, then E4M3 codes under one power-of-two scale per head."""
+    x = x.to(torch.bfloat16).double()
+    mant, ex = torch.frexp(x.abs().amax() / 448.0)
+    scale = 2.0 ** float(ex - 1 if float(mant) == 0.5 else ex)
+    return (x / scale).float().to(torch.float8_e4m3fn).double() * scale
+
+
+def exact(case, seed):
+    """Attention over prefix, branch and own tokens with one softmax, from the definition, in 64 bits."""
+    st = _inputs(case, seed)
+    H, B, S = case["heads"], case["batch"], case["queries"]
+    qn, qp, w_uk, w_uv = (x.double() for x in (st.q_nope, st.q_pe, st.w_uk, st.w_uv))
+
+    def add(logits, value):
+        """logits [.., rows, tokens], value [.., tokens, d] -> (lse [.., rows], o [.., rows, d])"""
+        lse = torch.logsumexp(logits, -1)
+        return lse, torch.exp(logits - lse[..., None]) @ value
+
+    shared = [(0, B, st.ckv, st.kpe)]
+    if case["kind"] == "tree":
+        begin = _groups(case)
+        shared += [(a, e, ckv, kpe) for a, e, (ckv, kpe) in zip(begin, begin[1:], st.parts) if e > a]
+    rows = B * S
+    total_lse = torch.full((rows, H), -math.inf, dtype=torch.float64, device="cuda")
+    total = torch.zeros(rows, H, 128, dtype=torch.float64, device="cuda")
+
+    def merge(where, lse, o):
+        old = total_lse[where]
+        new = torch.logaddexp(old, lse)
+        total[where] = total[where] * torch.exp(old - new)[..., None] + o * torch.exp(lse - new)[..., None]
+        total_lse[where] = new
+
+    for a, e, ckv, kpe in shared:
+        ckv, kpe = ckv.double(), kpe.double()
+        for h in range(H):
+            k, v = ckv @ w_uk[h].T, ckv @ w_uv[h].T
+            if case["kind"] == "fp8":
+                k, v = _e4m3(k), _e4m3(v)
+            where = (slice(a * S, e * S), h)
+            merge(where, *add((qn[where] @ k.T + qp[where] @ kpe.T) * SCALE, v))
+    q_lat = torch.einsum("rhd,hdc->rhc", qn, w_uk)   # the same logits, from the latent form
+    for r in range(B):
+        ids = st.table[r][st.table[r] >= 0].long().cuda()
+        ckv = st.ckv_pages[ids].reshape(-1, 512).double()
+        kpe = st.kpe_pages[ids].reshape(-1, 64).double()
+        for j in range(S):
+            n = max(int(st.lens[r]) - (S - 1 - j), 0)
+            if n > 0:
+                row = r * S + j
+                lse, o = add((q_lat[row] @ ckv[:n].T + qp[row] @ kpe[:n].T) * SCALE, ckv[:n])
+                merge(row, lse, torch.einsum("hc,hdc->hd", o, w_uv))
+    if case["kind"] in ("host", "tree", "prepare"):
+        return total
+    return total, total_lse
 
 
 def tolerance(case):
