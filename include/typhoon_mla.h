@@ -130,9 +130,32 @@ int typhoon_mla_prepare_shared_fp8(const typhoon_mla_dims_t* dims /* host */,
                                    const void* w_uk, const void* w_uv,
                                    void* stream, typhoon_mla_shared_t** out_handle /* host */);
 
+/*
+ * Both forms above with the handle's buffers in device memory of the caller, for programs that allocate from a pool
+ * of their own (preparing and freeing a prefix with cudaMalloc / cudaFree costs milliseconds).  `fp8` selects the
+ * 8-bit storage.  `storage` is 256-byte aligned, holds at least typhoon_mla_shared_storage_bytes and stays the
+ * handle's until typhoon_mla_free returns; `scratch` (8-bit storage only, same alignment, *scratch_bytes of the
+ * query) is used by the work enqueued here and may be reused on `stream` at once.
+ * Errors as above; too little storage or scratch -> WORKSPACE_TOO_SMALL.
+ */
+int typhoon_mla_prepare_shared_in(const typhoon_mla_dims_t* dims /* host */,
+                                  const void* ckv_shared, const void* kpe_shared,
+                                  int64_t Ls, int64_t ld_ckv, int64_t ld_kpe,
+                                  const void* w_uk, const void* w_uv, int32_t fp8,
+                                  void* storage, size_t storage_bytes, void* scratch, size_t scratch_bytes,
+                                  void* stream, typhoon_mla_shared_t** out_handle /* host */);
+
+/* Bytes of storage (returned; 0 on invalid arguments) and of scratch (through the pointer, which may be NULL)
+ * typhoon_mla_prepare_shared_in needs.  Host, pure. */
+size_t typhoon_mla_shared_storage_bytes(const typhoon_mla_dims_t* dims /* host */, int64_t Ls, int32_t fp8,
+                                        size_t* scratch_bytes /* host */);
+
 /* Release the handle and the device memory it owns (synchronises the device).
- * NULL is accepted. */
+ * NULL is accepted.  With caller storage a failed synchronisation is reported as ERR_CUDA (the handle is gone, work on
+ * the storage may still be pending), else the result is OK.  The side stream and events of up to four freed handles per device are kept for later
+ * handles; typhoon_mla_release_cached destroys the kept ones. */
 int typhoon_mla_free(typhoon_mla_shared_t* shared);
+int typhoon_mla_release_cached(void);
 
 /* Bytes of scratch typhoon_mla_decode needs for this problem size in `mode`
  * (TYPHOON_MLA_MODE_AUTO: the worst case over the modes AUTO may resolve to, so the

@@ -51,6 +51,12 @@ def _load():
     lib.typhoon_mla_prepare_shared.argtypes = [C.POINTER(Dims), vp, vp, i64, i64, i64, vp, vp, vp, C.POINTER(vp)]
     lib.typhoon_mla_prepare_shared_fp8.restype = C.c_int
     lib.typhoon_mla_prepare_shared_fp8.argtypes = [C.POINTER(Dims), vp, vp, i64, i64, i64, vp, vp, vp, C.POINTER(vp)]
+    lib.typhoon_mla_prepare_shared_in.restype = C.c_int
+    lib.typhoon_mla_prepare_shared_in.argtypes = [C.POINTER(Dims), vp, vp, i64, i64, i64, vp, vp, i32, vp, sz, vp, sz, vp,
+                                                  C.POINTER(vp)]
+    lib.typhoon_mla_shared_storage_bytes.restype = sz
+    lib.typhoon_mla_shared_storage_bytes.argtypes = [C.POINTER(Dims), i64, i32, C.POINTER(sz)]
+    lib.typhoon_mla_release_cached.restype = C.c_int
     lib.typhoon_mla_free.restype = C.c_int
     lib.typhoon_mla_free.argtypes = [vp]
     lib.typhoon_mla_workspace_bytes.restype = sz
@@ -142,6 +148,9 @@ def make_dims(H: int, d_nope=128, d_rope=64, d_v=128, kv_lora_rank=512) -> Dims:
     return Dims(H, d_nope, d_rope, d_v, kv_lora_rank)
 
 
+_unsynchronised = []   # storage of prefixes freed where the device cannot be synchronised (during a capture)
+
+
 class SharedPrefix:
     """Owner of the handle returned by typhoon_mla_prepare_shared."""
 
@@ -152,8 +161,10 @@ class SharedPrefix:
 
     def free(self):
         if self.handle:
-            typhoon_mla_free(self.handle)
+            if _lib.typhoon_mla_free(self.handle) != OK:   # it could not synchronise: nobody may reuse the storage
+                _unsynchronised.append(self._keepalive)
             self.handle = None
+            self._keepalive = ()
 
     def __del__(self):
         try:
@@ -162,29 +173,43 @@ class SharedPrefix:
             pass
 
 
-def typhoon_mla_prepare_shared(dims: Dims, ckv_shared: torch.Tensor, kpe_shared: torch.Tensor,
-                               w_uk: torch.Tensor, w_uv: torch.Tensor) -> SharedPrefix:
+def _prepare(dims: Dims, ckv_shared, kpe_shared, w_uk, w_uv, fp8: bool) -> SharedPrefix:
+    """The handle's buffers come from torch's caching allocator, which keeps a freed prefix's memory for the next one
+    (with cudaMalloc / cudaFree a 318 MB prefix takes 3 to 20 ms to prepare and free, 0.5 ms this way) and gives it
+    back when other tensors need it.  Where the allocator has none left, or the stream is being captured, the library
+    allocates for itself."""
+    where = "typhoon_mla_prepare_shared_fp8" if fp8 else "typhoon_mla_prepare_shared"
     Ls = ckv_shared.shape[0]
     h = C.c_void_p()
-    ld_ckv = ckv_shared.stride(0) if Ls > 0 else 512
-    ld_kpe = kpe_shared.stride(0) if Ls > 0 else 64
-    st = _lib.typhoon_mla_prepare_shared(C.byref(dims), _ptr(ckv_shared), _ptr(kpe_shared), Ls, ld_ckv, ld_kpe,
-                                         _ptr(w_uk), _ptr(w_uv), _stream(), C.byref(h))
-    _check(st, "typhoon_mla_prepare_shared")
-    return SharedPrefix(h, dims, (w_uk, w_uv))
+    args = (C.byref(dims), _ptr(ckv_shared), _ptr(kpe_shared), Ls, ckv_shared.stride(0) if Ls > 0 else 512,
+            kpe_shared.stride(0) if Ls > 0 else 64, _ptr(w_uk), _ptr(w_uv))
+    scratch_bytes = C.c_size_t()
+    nbytes = int(_lib.typhoon_mla_shared_storage_bytes(C.byref(dims), Ls, 1 if fp8 else 0, C.byref(scratch_bytes)))
+    storage = scratch = None
+    if nbytes > 0 and not torch.cuda.is_current_stream_capturing():
+        try:
+            storage = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+            scratch = torch.empty(scratch_bytes.value, dtype=torch.uint8, device="cuda") if scratch_bytes.value else None
+        except torch.OutOfMemoryError:
+            storage = None
+    if storage is None:
+        st = getattr(_lib, where)(*args, _stream(), C.byref(h))
+    else:
+        st = _lib.typhoon_mla_prepare_shared_in(*args, 1 if fp8 else 0, _ptr(storage), nbytes, _ptr(scratch),
+                                                scratch_bytes.value, _stream(), C.byref(h))
+    _check(st, where)
+    return SharedPrefix(h, dims, (w_uk, w_uv, storage))
+
+
+def typhoon_mla_prepare_shared(dims: Dims, ckv_shared: torch.Tensor, kpe_shared: torch.Tensor,
+                               w_uk: torch.Tensor, w_uv: torch.Tensor) -> SharedPrefix:
+    return _prepare(dims, ckv_shared, kpe_shared, w_uk, w_uv, False)
 
 
 def typhoon_mla_prepare_shared_fp8(dims: Dims, ckv_shared: torch.Tensor, kpe_shared: torch.Tensor,
                                    w_uk: torch.Tensor, w_uv: torch.Tensor) -> SharedPrefix:
     """The same with the expanded K_nope / V stored as E4M3 codes (one power-of-two scale per head and tensor)."""
-    Ls = ckv_shared.shape[0]
-    h = C.c_void_p()
-    ld_ckv = ckv_shared.stride(0) if Ls > 0 else 512
-    ld_kpe = kpe_shared.stride(0) if Ls > 0 else 64
-    st = _lib.typhoon_mla_prepare_shared_fp8(C.byref(dims), _ptr(ckv_shared), _ptr(kpe_shared), Ls, ld_ckv, ld_kpe,
-                                             _ptr(w_uk), _ptr(w_uv), _stream(), C.byref(h))
-    _check(st, "typhoon_mla_prepare_shared_fp8")
-    return SharedPrefix(h, dims, (w_uk, w_uv))
+    return _prepare(dims, ckv_shared, kpe_shared, w_uk, w_uv, True)
 
 
 def typhoon_mla_free(handle) -> None:

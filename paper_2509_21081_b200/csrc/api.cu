@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "../../include/typhoon_mla.h"
@@ -80,6 +81,56 @@ int cuda_fail(cudaError_t e) {
 int tmla::api_cuda_fail(cudaError_t e) { return cuda_fail(e); }
 void tmla::api_set_last_launches(int n) { g_last_launches = n; }
 namespace {
+
+// ---- side stream and events of a handle -------------------------------------
+// Creating and destroying a stream takes about 55 us each (B200 host), as much as a short decode step, so up to
+// kKeptSides idle sets per device outlive their handle.  A set belongs to one handle at a time; it comes back only
+// after the device has been synchronised (nothing of it is pending) and not while a capture holds it.
+// typhoon_mla_release_cached destroys the kept ones.
+constexpr int kKeptSides = 4, kSideDevices = 64;
+struct Side {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+std::mutex g_side_mu;
+Side g_sides[kSideDevices][kKeptSides];
+int g_n_sides[kSideDevices] = {};
+
+void destroy_side(const Side& x) {
+    if (x.stream) cudaStreamDestroy(x.stream);
+    if (x.fork) cudaEventDestroy(x.fork);
+    if (x.join) cudaEventDestroy(x.join);
+}
+cudaError_t take_side(int dev, Side* out) {
+    if (dev >= 0 && dev < kSideDevices) {
+        std::lock_guard<std::mutex> lock(g_side_mu);
+        if (g_n_sides[dev] > 0) {
+            *out = g_sides[dev][--g_n_sides[dev]];
+            return cudaSuccess;
+        }
+    }
+    Side x;
+    int lo = 0, hi = 0;
+    cudaDeviceGetStreamPriorityRange(&lo, &hi);   // hi is the numerically lowest = highest priority
+    cudaError_t e = cudaStreamCreateWithPriority(&x.stream, cudaStreamNonBlocking, hi);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming);
+    if (e != cudaSuccess) destroy_side(x);
+    else *out = x;
+    return e;
+}
+void give_side(int dev, const Side& x, bool idle) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (idle && x.stream && cudaStreamIsCapturing(x.stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+        dev >= 0 && dev < kSideDevices) {
+        std::lock_guard<std::mutex> lock(g_side_mu);
+        if (g_n_sides[dev] < kKeptSides) {
+            g_sides[dev][g_n_sides[dev]++] = x;
+            return;
+        }
+    }
+    destroy_side(x);
+}
 
 // ---- workspace plan --------------------------------------------------------
 struct Plan {
@@ -324,28 +375,75 @@ int typhoon_mla_free(typhoon_mla_shared_t* sh) {
     // the handle's buffers, stream and events belong to the device it was prepared on, whatever device is current now
     int cur = -1;
     const bool switched = cudaGetDevice(&cur) == cudaSuccess && cur != sh->device && cudaSetDevice(sh->device) == cudaSuccess;
-    cudaDeviceSynchronize();
-    cudaFree(sh->k_nope);
-    cudaFree(sh->v_t);
-    cudaFree(sh->ckv);
-    cudaFree(sh->kpe);
-    cudaFree(sh->w_uk_t);
-    cudaFree(sh->status);
-    cudaFree(sh->k8);
-    cudaFree(sh->v8);
-    cudaFree(sh->fp8_f);
-    if (sh->side_stream) cudaStreamDestroy(sh->side_stream);
-    if (sh->ev_fork) cudaEventDestroy(sh->ev_fork);
-    if (sh->ev_join) cudaEventDestroy(sh->ev_join);
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (!sh->borrowed_storage) {
+        cudaFree(sh->k_nope);
+        cudaFree(sh->v_t);
+        cudaFree(sh->ckv);
+        cudaFree(sh->kpe);
+        cudaFree(sh->w_uk_t);
+        cudaFree(sh->status);
+        cudaFree(sh->k8);
+        cudaFree(sh->v8);
+        cudaFree(sh->fp8_f);
+    }
+    Side side;
+    side.stream = sh->side_stream; side.fork = sh->ev_fork; side.join = sh->ev_join;
+    give_side(sh->device, side, idle);
     if (switched) cudaSetDevice(cur);
     cudaGetLastError();   // a failure while releasing must not surface in the caller's next launch
+    // (a caller that lent the storage has to know when work on it may still be pending)
+    const int st = (sh->borrowed_storage && !idle) ? TYPHOON_MLA_ERR_CUDA : TYPHOON_MLA_OK;
     delete sh;
+    return st;
+}
+
+int typhoon_mla_release_cached(void) {
+    int cur = -1;
+    if (cudaGetDevice(&cur) != cudaSuccess) return cuda_fail(cudaGetLastError());
+    std::lock_guard<std::mutex> lock(g_side_mu);
+    for (int dev = 0; dev < kSideDevices; ++dev) {
+        if (g_n_sides[dev] == 0 || cudaSetDevice(dev) != cudaSuccess) continue;
+        while (g_n_sides[dev] > 0) destroy_side(g_sides[dev][--g_n_sides[dev]]);
+    }
+    cudaSetDevice(cur);
+    cudaGetLastError();
     return TYPHOON_MLA_OK;
 }
 
+// Buffers of a handle, in bytes.  Ls_pad rows; every part starts on a 256-byte boundary of caller-supplied storage.
+struct SharedSizes {
+    size_t ckv, kpe, w_uk_t, status, expanded /* one of K_nope, V^T in 16 bits */, codes /* one of them in 8 bits */, scales;
+    SharedSizes(int H, int64_t Ls, bool fp8) {
+        const size_t Lp = (size_t)round_up(Ls, 128), b_k = (size_t)H * Lp * 128 * 2;
+        ckv = Lp * 512 * 2;
+        kpe = Lp * 64 * 2;
+        w_uk_t = (size_t)H * 512 * 128 * 2;
+        status = 256;
+        expanded = b_k;
+        codes = fp8 ? b_k / 2 : 0;
+        scales = fp8 ? (size_t)H * 3 * sizeof(float) : 0;
+    }
+    static size_t pad(size_t x) { return (size_t)round_up((int64_t)x, 256); }
+    size_t storage(bool fp8) const {
+        return pad(ckv) + pad(kpe) + pad(w_uk_t) + status + (fp8 ? 2 * pad(codes) + pad(scales) : 2 * pad(expanded));
+    }
+};
+
+size_t typhoon_mla_shared_storage_bytes(const typhoon_mla_dims_t* dims, int64_t Ls, int32_t fp8, size_t* scratch_bytes) {
+    if (scratch_bytes) *scratch_bytes = 0;
+    if (!dims || !dims_supported(*dims) || Ls < 0 || Ls > (int64_t)1 << 24) return 0;
+    const bool f = fp8 != 0 && Ls > 0;
+    const SharedSizes sz(dims->num_heads, Ls, f);
+    if (scratch_bytes && f) *scratch_bytes = sz.expanded;
+    return sz.storage(f);
+}
+
+// `storage` / `scratch`: device memory of the caller, or null (the handle then allocates its own).
 static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, const void* kpe_shared,
                         int64_t Ls, int64_t ld_ckv, int64_t ld_kpe, const void* w_uk, const void* w_uv,
-                        void* stream, typhoon_mla_shared_t** out_handle, bool fp8) {
+                        void* stream, typhoon_mla_shared_t** out_handle, bool fp8, void* storage = nullptr,
+                        size_t storage_bytes = 0, void* scratch = nullptr, size_t scratch_bytes = 0) {
     if (!dims || !out_handle || !w_uk || !w_uv || Ls < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
     *out_handle = nullptr;
     if (!dims_supported(*dims)) return TYPHOON_MLA_ERR_UNSUPPORTED_DIMS;
@@ -353,6 +451,12 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
                    !aligned16(ckv_shared) || !aligned16(kpe_shared)))
         return TYPHOON_MLA_ERR_INVALID_ARG;
     if (!aligned16(w_uk) || !aligned16(w_uv) || Ls > (int64_t)1 << 24) return TYPHOON_MLA_ERR_INVALID_ARG;
+    const SharedSizes sz(dims->num_heads, Ls, fp8 && Ls > 0);
+    if (storage) {
+        if ((reinterpret_cast<uintptr_t>(storage) & 255u) || (reinterpret_cast<uintptr_t>(scratch) & 255u)) return TYPHOON_MLA_ERR_INVALID_ARG;
+        if (storage_bytes < sz.storage(fp8 && Ls > 0)) return TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL;
+        if (fp8 && Ls > 0 && (!scratch || scratch_bytes < sz.expanded)) return TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL;
+    }
     int dev = 0, n_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -385,21 +489,27 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     sh->num_sms = n_sm;
     const int H = dims->num_heads;
     const size_t Lp = (size_t)sh->Ls_pad;
-    const size_t b_k = (size_t)H * Lp * 128 * 2, b_ckv = Lp * 512 * 2, b_kpe = Lp * 64 * 2,
-                 b_w = (size_t)H * 512 * 128 * 2;
+    sh->borrowed_storage = storage ? 1 : 0;
+    char* next = reinterpret_cast<char*>(storage);
     auto alloc = [&](void** p, size_t bytes) {
         if (bytes == 0) { *p = nullptr; return true; }
+        if (storage) {
+            *p = next;
+            next += SharedSizes::pad(bytes);
+            sh->owned_bytes += bytes;
+            return true;
+        }
         if (cudaMalloc(p, bytes) != cudaSuccess) { cudaGetLastError(); *p = nullptr; return false; }
         sh->owned_bytes += bytes;
         return true;
     };
     sh->fp8 = (fp8 && Ls > 0) ? 1 : 0;
-    bool ok_alloc = alloc(&sh->ckv, b_ckv) && alloc(&sh->kpe, b_kpe) && alloc(&sh->w_uk_t, b_w) &&
-                    alloc(reinterpret_cast<void**>(&sh->status), 256);
-    if (ok_alloc && !sh->fp8) ok_alloc = alloc(&sh->k_nope, b_k) && alloc(&sh->v_t, b_k);
+    bool ok_alloc = alloc(&sh->ckv, sz.ckv) && alloc(&sh->kpe, sz.kpe) && alloc(&sh->w_uk_t, sz.w_uk_t) &&
+                    alloc(reinterpret_cast<void**>(&sh->status), sz.status);
+    if (ok_alloc && !sh->fp8) ok_alloc = alloc(&sh->k_nope, sz.expanded) && alloc(&sh->v_t, sz.expanded);
     if (ok_alloc && sh->fp8)
-        ok_alloc = alloc(&sh->k8, b_k / 2) && alloc(&sh->v8, b_k / 2) &&
-                   alloc(reinterpret_cast<void**>(&sh->fp8_f), (size_t)H * 3 * sizeof(float));
+        ok_alloc = alloc(&sh->k8, sz.codes) && alloc(&sh->v8, sz.codes) &&
+                   alloc(reinterpret_cast<void**>(&sh->fp8_f), sz.scales);
     if (!ok_alloc) {
         typhoon_mla_free(sh);
         return TYPHOON_MLA_ERR_ALLOC;
@@ -407,22 +517,20 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // 8-bit cache: each tensor is expanded into a 16-bit scratch of the stream's memory pool, encoded from there,
     // and the scratch is handed back in stream order (no synchronisation)
-    void* scratch16 = nullptr;
-    if (sh->fp8 && cudaMallocAsync(&scratch16, b_k, s) != cudaSuccess) {
+    void* scratch16 = nullptr;   // ours (released below); the caller's scratch is used where it gave one
+    if (sh->fp8 && !storage && cudaMallocAsync(&scratch16, sz.expanded, s) != cudaSuccess) {
         cudaGetLastError();
         typhoon_mla_free(sh);
         return TYPHOON_MLA_ERR_ALLOC;
     }
-    void* const k_dst = sh->fp8 ? scratch16 : sh->k_nope;
-    void* const v_dst = sh->fp8 ? scratch16 : sh->v_t;
+    void* const k_dst = sh->fp8 ? (storage ? scratch : scratch16) : sh->k_nope;
+    void* const v_dst = sh->fp8 ? (storage ? scratch : scratch16) : sh->v_t;
     const bool tc = cfg.tc();
     {
-        int lo = 0, hi = 0;
-        cudaDeviceGetStreamPriorityRange(&lo, &hi);   // hi is the numerically lowest = highest priority
-        e = cudaStreamCreateWithPriority(&sh->side_stream, cudaStreamNonBlocking, hi);
+        Side side;
+        e = take_side(dev, &side);
+        sh->side_stream = side.stream; sh->ev_fork = side.fork; sh->ev_join = side.join;
     }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sh->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sh->ev_join, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         if (scratch16) cudaFreeAsync(scratch16, s);
         typhoon_mla_free(sh);
@@ -477,6 +585,15 @@ int typhoon_mla_prepare_shared_fp8(const typhoon_mla_dims_t* dims, const void* c
                                    int64_t Ls, int64_t ld_ckv, int64_t ld_kpe, const void* w_uk, const void* w_uv,
                                    void* stream, typhoon_mla_shared_t** out_handle) {
     return prepare_impl(dims, ckv_shared, kpe_shared, Ls, ld_ckv, ld_kpe, w_uk, w_uv, stream, out_handle, true);
+}
+
+int typhoon_mla_prepare_shared_in(const typhoon_mla_dims_t* dims, const void* ckv_shared, const void* kpe_shared,
+                                  int64_t Ls, int64_t ld_ckv, int64_t ld_kpe, const void* w_uk, const void* w_uv,
+                                  int32_t fp8, void* storage, size_t storage_bytes, void* scratch, size_t scratch_bytes,
+                                  void* stream, typhoon_mla_shared_t** out_handle) {
+    if (!storage) return TYPHOON_MLA_ERR_INVALID_ARG;
+    return prepare_impl(dims, ckv_shared, kpe_shared, Ls, ld_ckv, ld_kpe, w_uk, w_uv, stream, out_handle, fp8 != 0, storage,
+                        storage_bytes, scratch, scratch_bytes);
 }
 
 int typhoon_mla_shared_view(const typhoon_mla_shared_t* sh, const void** k_nope, const void** v_t, int64_t* Ls,

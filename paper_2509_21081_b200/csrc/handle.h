@@ -23,6 +23,7 @@ struct typhoon_mla_shared {
     cudaEvent_t ev_fork, ev_join;
     int* status;    // device word: non-zero after a bounded in-kernel wait expired
     size_t owned_bytes;
+    int borrowed_storage;   // the buffers are slices of the caller's storage (typhoon_mla_prepare_shared_in)
     int device;     // device the handle was prepared on; every call checks that it is the current one
     int num_sms;    // multiprocessors of that device (the work decompositions fill them)
     // 8-bit expanded cache (typhoon_mla_prepare_shared_fp8): k_nope and v_t are null, the codes live here and
