@@ -504,12 +504,12 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
         return true;
     };
     sh->fp8 = (fp8 && Ls > 0) ? 1 : 0;
-    bool ok_alloc = alloc(&sh->ckv, sz.ckv) && alloc(&sh->kpe, sz.kpe) && alloc(&sh->w_uk_t, sz.w_uk_t) &&
-                    alloc(reinterpret_cast<void**>(&sh->status), sz.status);
-    if (ok_alloc && !sh->fp8) ok_alloc = alloc(&sh->k_nope, sz.expanded) && alloc(&sh->v_t, sz.expanded);
-    if (ok_alloc && sh->fp8)
-        ok_alloc = alloc(&sh->k8, sz.codes) && alloc(&sh->v8, sz.codes) &&
-                   alloc(reinterpret_cast<void**>(&sh->fp8_f), sz.scales);
+    // (the streamed buffers first: caller storage that starts on a large-page boundary keeps their 8 KB blocks aligned;
+    // behind the 256-byte status word they cost the shared-prefix kernel 1 to 3 %)
+    bool ok_alloc = sh->fp8 ? alloc(&sh->k8, sz.codes) && alloc(&sh->v8, sz.codes) : alloc(&sh->k_nope, sz.expanded) && alloc(&sh->v_t, sz.expanded);
+    ok_alloc = ok_alloc && alloc(&sh->w_uk_t, sz.w_uk_t) && alloc(&sh->ckv, sz.ckv) && alloc(&sh->kpe, sz.kpe) &&
+               alloc(reinterpret_cast<void**>(&sh->status), sz.status);
+    if (ok_alloc && sh->fp8) ok_alloc = alloc(reinterpret_cast<void**>(&sh->fp8_f), sz.scales);
     if (!ok_alloc) {
         typhoon_mla_free(sh);
         return TYPHOON_MLA_ERR_ALLOC;
@@ -718,6 +718,7 @@ struct NaiveJob {
     int n_ranges;         // tile ranges (tcgen05 path) or KV splits (warp-MMA path)
     int n_slots_level;    // slots of this job's level (the kernel marks the ones it does not fill as empty)
     int slot0;
+    int n_merged = 1;     // first job of a launch: how many consecutive jobs it takes
 };
 // Rows of a level that have no prefix: their slots get weight zero in the combine.
 struct EmptySlots {
@@ -773,21 +774,28 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
     };
 
     // --- naive shared-prefix attention (Algorithm 1 line 4), one launch per (prefix, row range)
-    for (int j = 0; j < n_jobs; ++j) {
+    for (int j = 0; j < n_jobs; j += jobs[j].n_merged) {
         const NaiveJob& jb = jobs[j];
-        const char* qn = reinterpret_cast<const char*>(q_nope) + (size_t)jb.row0 * H * 128 * 2;
-        const char* qp = reinterpret_cast<const char*>(q_pe) + (size_t)jb.row0 * H * 64 * 2;
-        float* op = o_part_n + ((size_t)jb.slot0 * B + jb.row0) * H * 128;
-        float* lp = lse_part_n + ((size_t)jb.slot0 * B + jb.row0) * H;
+        auto sm100_job = [&](const NaiveJob& x) {
+            const char* qn = reinterpret_cast<const char*>(q_nope) + (size_t)x.row0 * H * 128 * 2;
+            const char* qp = reinterpret_cast<const char*>(q_pe) + (size_t)x.row0 * H * 64 * 2;
+            float* op = o_part_n + ((size_t)x.slot0 * B + x.row0) * H * 128;
+            float* lp = lse_part_n + ((size_t)x.slot0 * B + x.row0) * H;
+            NaiveAttnSm100 na{qn, qp, &x.sh->tm_kn, &x.sh->tm_kp, &x.sh->tm_vt, x.rows, H, (int)x.sh->Ls,
+                              x.n_ranges, x.n_slots_level, softmax_scale, op, lp, sh->status, B};
+            if (x.sh->fp8) na.fp8_mult = x.sh->fp8_f;
+            return na;
+        };
         prof_before(TYPHOON_MLA_KERNEL_NAIVE_ATTN, s);
-        if (tc) {
-            NaiveAttnSm100 na{qn, qp, &jb.sh->tm_kn, &jb.sh->tm_kp, &jb.sh->tm_vt, jb.rows, H, (int)jb.sh->Ls,
-                              jb.n_ranges, jb.n_slots_level, softmax_scale, op, lp, sh->status, B};
-            if (jb.sh->fp8) na.fp8_mult = jb.sh->fp8_f;
-            e = launch_naive_attn_sm100(na, s);
+        if (tc && jb.n_merged > 1) {
+            NaiveAttnSm100 na[kNaiveJobsPerLaunch];
+            for (int k = 0; k < jb.n_merged; ++k) na[k] = sm100_job(jobs[j + k]);
+            e = launch_naive_attn_sm100_multi(na, jb.n_merged, s);
+        } else if (tc) {
+            e = launch_naive_attn_sm100(sm100_job(jb), s);
         } else {
-            NaiveAttn na{qn, qp, jb.sh->k_nope, jb.sh->v_t, jb.sh->kpe, B, H, (int)jb.sh->Ls, (int)jb.sh->Ls_pad,
-                         jb.n_ranges, softmax_scale, op, lp};
+            NaiveAttn na{q_nope, q_pe, jb.sh->k_nope, jb.sh->v_t, jb.sh->kpe, B, H, (int)jb.sh->Ls, (int)jb.sh->Ls_pad,
+                         jb.n_ranges, softmax_scale, o_part_n, lse_part_n};
             e = launch_naive_attn_mma(na, s);
         }
         prof_after(TYPHOON_MLA_KERNEL_NAIVE_ATTN, s);
@@ -826,13 +834,15 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                     naive_ctas = std::max(naive_ctas, jobs[j].n_ranges * groups);
                 }
                 const int free_sms = sh->num_sms - naive_ctas;
-                if (n_jobs == 1 && free_sms >= 8 && free_sms < H) {
+                if (jobs[0].n_merged == n_jobs && free_sms >= 8 && free_sms < H) {
                     // ... but only if the shared-prefix kernel lasts about as long as the walk (measured: about 5 us per head
                     // for a walking CTA, 0.7 us per 64-token tile for a shared-prefix CTA; B = 64, H = 128: the walk wins
                     // from 3072 prefix tokens on and loses at 2048); under a short shared-prefix kernel one CTA per head,
                     // which spreads over the whole GPU as soon as that kernel ends, is faster.
                     const int64_t tok = jobs[0].rows <= 128 || jobs[0].sh->fp8 ? 64 : 128;
-                    const int64_t tiles_per_cta = ((jobs[0].sh->Ls + tok - 1) / tok * H + jobs[0].n_ranges - 1) / jobs[0].n_ranges;
+                    int64_t head_tiles = 0;
+                    for (int j = 0; j < n_jobs; ++j) head_tiles += (jobs[j].sh->Ls + tok - 1) / tok;
+                    const int64_t tiles_per_cta = (head_tiles * H + jobs[0].n_ranges - 1) / jobs[0].n_ranges;
                     const int heads_per_cta = (H + free_sms - 1) / free_sms;
                     if ((double)tiles_per_cta * (tok == 64 ? 0.7 : 3.0) >= 4.0 * heads_per_cta) walk_ctas = free_sms;
                 }
@@ -1004,28 +1014,62 @@ int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int
     }
     if (!tp->sh0) return TYPHOON_MLA_ERR_INVALID_ARG;
     const int H = tp->sh0->dims.num_heads;
+    const int n_sm = tp->sh0->num_sms > 0 ? tp->sh0->num_sms : kDefaultNumSM;
+    int level_of[kMaxTreeJobs], slots_of[kMaxTreeJobs], n_merge = 0;
+    // Prefixes that can share a launch come first.  One launch per prefix leaves SMs idle at every launch's end and pays
+    // set-up and pipeline fill once per (prefix, head); in a shared launch a CTA goes on from one prefix's tiles to the
+    // next one's.  (16-bit cache, at most 128 rows: the row groups of larger ones differ in number.)
+    auto mergeable = [](const NaiveJob& j) { return !j.sh->fp8 && j.rows <= 128; };
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int l = 0; l < n_levels; ++l) {
+            const typhoon_mla_prefix_level_t& lv = levels[l];
+            if (!lv.prefixes || !lv.group_begin || lv.n_groups < 1) return TYPHOON_MLA_ERR_INVALID_ARG;
+            if (lv.group_begin[0] != 0 || lv.group_begin[lv.n_groups] != B) return TYPHOON_MLA_ERR_INVALID_ARG;
+            for (int g = 0; g < lv.n_groups; ++g) {
+                const int r0 = lv.group_begin[g], r1 = lv.group_begin[g + 1];
+                if (r1 < r0) return TYPHOON_MLA_ERR_INVALID_ARG;
+                const typhoon_mla_shared* sh = lv.prefixes[g];
+                if (sh && (sh->dims.num_heads != H || sh->device != tp->sh0->device)) return TYPHOON_MLA_ERR_INVALID_ARG;
+                if (!sh || sh->Ls == 0 || r1 == r0) continue;
+                const NaiveJob job{sh, r0, r1 - r0, 0, 0, 0};
+                if (mergeable(job) != (pass == 0)) continue;
+                if (tp->n_jobs == kMaxTreeJobs) return TYPHOON_MLA_ERR_INVALID_ARG;
+                level_of[tp->n_jobs] = l;
+                tp->jobs[tp->n_jobs++] = job;
+            }
+        }
+        if (pass == 0) n_merge = tp->n_jobs;
+    }
+    for (int j = 0; j < tp->n_jobs;) {
+        const int n = j < n_merge ? std::min(kNaiveJobsPerLaunch, n_merge - j) : 1;
+        int ranges = 0;
+        if (n > 1) {
+            int64_t len[kNaiveJobsPerLaunch];
+            int rows = 0;
+            for (int k = 0; k < n; ++k) {
+                len[k] = tp->jobs[j + k].sh->Ls;
+                rows = std::max(rows, tp->jobs[j + k].rows);
+            }
+            naive_sm100_plan_multi(rows, H, len, n, n_sm, schedule, &ranges, &slots_of[j]);
+        } else {
+            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, n_sm, schedule, &ranges, &slots_of[j], tp->jobs[j].sh->fp8 != 0);
+        }
+        for (int k = 0; k < n; ++k) tp->jobs[j + k].n_ranges = ranges;
+        tp->jobs[j].n_merged = n;
+        j += n;
+    }
     int slot0 = 0;
     for (int l = 0; l < n_levels; ++l) {
         const typhoon_mla_prefix_level_t& lv = levels[l];
-        if (!lv.prefixes || !lv.group_begin || lv.n_groups < 1) return TYPHOON_MLA_ERR_INVALID_ARG;
-        if (lv.group_begin[0] != 0 || lv.group_begin[lv.n_groups] != B) return TYPHOON_MLA_ERR_INVALID_ARG;
-        const int first_job = tp->n_jobs;
         int level_slots = 0;
-        for (int g = 0; g < lv.n_groups; ++g) {
-            const int r0 = lv.group_begin[g], r1 = lv.group_begin[g + 1];
-            if (r1 < r0) return TYPHOON_MLA_ERR_INVALID_ARG;
-            const typhoon_mla_shared* sh = lv.prefixes[g];
-            if (sh && (sh->dims.num_heads != H || sh->device != tp->sh0->device)) return TYPHOON_MLA_ERR_INVALID_ARG;
-            if (!sh || sh->Ls == 0 || r1 == r0) continue;
-            if (tp->n_jobs == kMaxTreeJobs) return TYPHOON_MLA_ERR_INVALID_ARG;
-            int ranges = 0, slots = 0;
-            naive_sm100_plan(r1 - r0, H, sh->Ls, sh->num_sms > 0 ? sh->num_sms : kDefaultNumSM, schedule, &ranges, &slots,
-                             sh->fp8 != 0);
-            tp->jobs[tp->n_jobs++] = NaiveJob{sh, r0, r1 - r0, ranges, 0, slot0};
-            level_slots = std::max(level_slots, slots);
-        }
+        for (int j = 0; j < tp->n_jobs; ++j)
+            if (level_of[j] == l) level_slots = std::max(level_slots, slots_of[j]);
         if (level_slots == 0) continue;   // no prefix at this level at all: no slots
-        for (int j = first_job; j < tp->n_jobs; ++j) tp->jobs[j].n_slots_level = level_slots;
+        for (int j = 0; j < tp->n_jobs; ++j)
+            if (level_of[j] == l) {
+                tp->jobs[j].n_slots_level = level_slots;
+                tp->jobs[j].slot0 = slot0;
+            }
         for (int g = 0; g < lv.n_groups; ++g) {
             const int r0 = lv.group_begin[g], r1 = lv.group_begin[g + 1];
             const typhoon_mla_shared* sh = lv.prefixes[g];

@@ -110,6 +110,12 @@ int naive_sm100_tile_tokens(int B, bool fp8 = false);   // KV tile width the ker
 // schedule: 0 = chosen by the plan, 1 = column split, 2 = stream-K
 void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8 = false);
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s);
+// Up to kNaiveJobsPerLaunch prefixes of the 16-bit cache, each with at most 128 query rows, in one launch: ranges and
+// slots (per prefix) come from naive_sm100_plan_multi over the same prefixes in the same order; the jobs' n_ranges is
+// that plan's.
+constexpr int kNaiveJobsPerLaunch = 16;
+void naive_sm100_plan_multi(int max_rows, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots);
+cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaStream_t s);
 cudaError_t make_naive_sm100_tmaps(const void* k_nope, const void* kpe, const void* v_t, int H, int64_t Ls_pad,
                                    CUtensorMap* tm_kn, CUtensorMap* tm_kp, CUtensorMap* tm_vt);
 // Tensor maps of the E4M3 code arrays k8 [H, Ls_pad/64, 64 tokens, 128 dims] and v8 [H, Ls_pad/64, 128 dims,

@@ -45,6 +45,7 @@
 //
 // Every mbarrier wait has a deadline; on expiry all roles fall through to the common teardown
 // and the status word is set.
+#include <algorithm>
 #include <cstddef>
 
 #include "kernels.h"
@@ -67,7 +68,7 @@ struct NaiveSm100Params {
     int B, H, Ls, Ls_pad;
     int part_rows;         // rows of the partial arrays (>= B: a launch may fill a row range of a larger batch)
     int m_groups;          // query-row groups per head
-    int n_tiles;           // KV tiles per head
+    int n_tiles;           // KV tiles per head (of all prefixes of the launch)
     int n_ranges;          // R (grid = R * m_groups CTAs)
     int per, rem;          // T = R * per + rem: ranges [0, rem) hold per + 1 tiles, the others per
     int n_seg_max;         // partial slots per head (one per segment of the head)
@@ -79,6 +80,21 @@ struct NaiveSm100Params {
     float* lse_part;   // [n_slots][part_rows][H]
     int* status;
 };
+// A launch over several prefixes: what differs from one to the next (the members above of the same names do not hold).
+struct alignas(64) NaiveSm100Job {
+    CUtensorMap tm_qn, tm_qp, tm_kn, tm_kp, tm_vt;
+    float* o_part;
+    float* lse_part;
+    int B, Ls, Ls_pad, n_tiles, n_seg_max;
+    int tile0;             // KV tiles of the launch's earlier prefixes, per head
+};
+template <int NJ>
+struct NaiveSm100Jobs {
+    int n;
+    NaiveSm100Job j[NJ];
+};
+template <>
+struct NaiveSm100Jobs<1> {};
 
 struct Barriers {
     uint64_t q_full, q_free;
@@ -106,6 +122,7 @@ struct Barriers {
 struct Segment {
     int t0, cnt;           // first tile, number of tiles
     int h, row0;           // head, first query row
+    int job;               // prefix (0 where a launch holds one)
     int slot_seg;          // index of this segment among the head's segments
     bool last_of_col;      // this segment ends the head
     int n_str0, n_str1;    // tiles per stream
@@ -113,11 +130,30 @@ struct Segment {
 
 // TOK = tokens per KV tile: 64 (mode Y, B <= 128) or 128 (mode X, B > 128).
 // FP8: the expanded cache is stored as E4M3 codes (see the conversion warpgroup below); 64 query rows per CTA.
-template <int TOK, bool M64, bool FP8>
+// NJ: largest number of prefixes per launch (several: 64-token tiles of the 16-bit cache).
+template <int TOK, bool M64, bool FP8, int NJ>
 __global__ void __launch_bounds__(FP8 ? 512 : 384, 1)
 naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_constant__ CUtensorMap tm_qp,
                         const __grid_constant__ CUtensorMap tm_kn, const __grid_constant__ CUtensorMap tm_kp,
-                        const __grid_constant__ CUtensorMap tm_vt, NaiveSm100Params p) {
+                        const __grid_constant__ CUtensorMap tm_vt, NaiveSm100Params p,
+                        const __grid_constant__ NaiveSm100Jobs<NJ> jobs) {
+    // a member of the prefix with index `job`; with one prefix per launch the plain parameter
+#define TMLA_JOB_MEMBER(type, name, one, many) \
+    auto name = [&](int job) -> type { if constexpr (NJ == 1) return one; else return jobs.j[job].many; };
+    TMLA_JOB_MEMBER(int, rows_of, p.B, B)
+    TMLA_JOB_MEMBER(int, tokens_of, p.Ls, Ls)
+    TMLA_JOB_MEMBER(int, tokens_pad_of, p.Ls_pad, Ls_pad)
+    TMLA_JOB_MEMBER(int, n_tiles_of, p.n_tiles, n_tiles)
+    TMLA_JOB_MEMBER(int, n_slots_of, p.n_seg_max, n_seg_max)
+    TMLA_JOB_MEMBER(int, tile0_of, 0, tile0)
+    TMLA_JOB_MEMBER(float*, o_part_of, p.o_part, o_part)
+    TMLA_JOB_MEMBER(float*, lse_part_of, p.lse_part, lse_part)
+    TMLA_JOB_MEMBER(const CUtensorMap&, qn_of, tm_qn, tm_qn)
+    TMLA_JOB_MEMBER(const CUtensorMap&, qp_of, tm_qp, tm_qp)
+    TMLA_JOB_MEMBER(const CUtensorMap&, kn_of, tm_kn, tm_kn)
+    TMLA_JOB_MEMBER(const CUtensorMap&, kp_of, tm_kp, tm_kp)
+    TMLA_JOB_MEMBER(const CUtensorMap&, vt_of, tm_vt, tm_vt)
+#undef TMLA_JOB_MEMBER
     constexpr bool MODE_Y = TOK == 64;
     // 128-token tiles (compute-bound regime): pairs of exponentials computed on the FMA pipe instead of the
     // special-function unit, by position of the pair within a group of eight (bit set = polynomial).  Measured at
@@ -161,19 +197,24 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         Segment s;
         s.h = g / p.n_tiles;
         s.t0 = g - s.h * p.n_tiles;
-        s.cnt = min(p.n_tiles - s.t0, g_end - g);
+        s.job = 0;
+        if constexpr (NJ > 1) {
+            while (s.job + 1 < jobs.n && s.t0 >= jobs.j[s.job + 1].tile0) ++s.job;
+            s.t0 -= jobs.j[s.job].tile0;
+        }
+        s.cnt = min(n_tiles_of(s.job) - s.t0, g_end - g);
         s.row0 = grp * ROWS;
-        // first range that reaches into this head: the one containing the head's first tile
-        const int first_tile = s.h * p.n_tiles, big = p.rem * (p.per + 1);
+        // first range that reaches into this (prefix, head): the one containing its first tile
+        const int first_tile = s.h * p.n_tiles + tile0_of(s.job), big = p.rem * (p.per + 1);
         const int r_first = first_tile < big ? first_tile / (p.per + 1) : p.rem + (first_tile - big) / p.per;
         s.slot_seg = rng - r_first;
-        s.last_of_col = (s.t0 + s.cnt == p.n_tiles);
+        s.last_of_col = (s.t0 + s.cnt == n_tiles_of(s.job));
         if (MODE_Y) {
             s.n_str0 = (s.cnt + 1) >> 1;
             s.n_str1 = s.cnt >> 1;
         } else {
             s.n_str0 = s.cnt;
-            s.n_str1 = (s.row0 + 128 < p.B) ? s.cnt : 0;   // second row tile entirely past B: skip it
+            s.n_str1 = (s.row0 + 128 < rows_of(s.job)) ? s.cnt : 0;   // second row tile entirely past B: skip it
         }
         return s;
     };
@@ -196,9 +237,9 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         mbar_arrive_expect_tx_if(ld0, &bar->q_full, nq * Q_BYTES);
         for (int t = 0; t < nq; ++t) {
             uint8_t* dst = sQ + t * Q_BYTES;
-            tma_load_3d_if(ld0, dst, &tm_qn, &bar->q_full, 0, s.h, s.row0 + t * 128);
-            tma_load_3d_if(ld0, dst + Q_SLAB, &tm_qn, &bar->q_full, 64, s.h, s.row0 + t * 128);
-            tma_load_3d_if(ld0, dst + 2 * Q_SLAB, &tm_qp, &bar->q_full, 0, s.h, s.row0 + t * 128);
+            tma_load_3d_if(ld0, dst, &qn_of(s.job), &bar->q_full, 0, s.h, s.row0 + t * 128);
+            tma_load_3d_if(ld0, dst + Q_SLAB, &qn_of(s.job), &bar->q_full, 64, s.h, s.row0 + t * 128);
+            tma_load_3d_if(ld0, dst + 2 * Q_SLAB, &qp_of(s.job), &bar->q_full, 0, s.h, s.row0 + t * 128);
         }
     };
     auto issue_k = [&](const Segment& s, int e, int ring_pos) {
@@ -207,8 +248,8 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
             uint8_t* dst = sKq + sq * KQ_BYTES;
             const int blk = tile_of(s, e);
             mbar_arrive_expect_tx_if(ld0, &bar->kq_full[sq], KQ_BYTES);
-            tma_load_3d_if(ld0, dst, &tm_kn, &bar->kq_full[sq], 0, blk * 64, s.h);
-            tma_load_2d_if(ld0, dst + 8192, &tm_kp, &bar->kq_full[sq], 0, blk * 64);
+            tma_load_3d_if(ld0, dst, &kn_of(s.job), &bar->kq_full[sq], 0, blk * 64, s.h);
+            tma_load_2d_if(ld0, dst + 8192, &kp_of(s.job), &bar->kq_full[sq], 0, blk * 64);
             return;
         }
         const int st = ring_pos % p.k_stages;
@@ -217,17 +258,17 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         mbar_arrive_expect_tx_if(ld0, &bar->k_full[st], K_TILE_BYTES);
 #pragma unroll
         for (int bi = 0; bi < BLK; ++bi) {
-            const int gb = s.h * (p.Ls_pad / 64) + blk0 + bi;
-            tma_load_3d_if(ld0, dst + bi * 8192, &tm_kn, &bar->k_full[st], 0, 0, gb);
-            tma_load_3d_if(ld0, dst + K_SLAB + bi * 8192, &tm_kn, &bar->k_full[st], 0, 64, gb);
-            tma_load_2d_if(ld0, dst + 2 * K_SLAB + bi * 8192, &tm_kp, &bar->k_full[st], 0, (blk0 + bi) * 64);
+            const int gb = s.h * (tokens_pad_of(s.job) / 64) + blk0 + bi;
+            tma_load_3d_if(ld0, dst + bi * 8192, &kn_of(s.job), &bar->k_full[st], 0, 0, gb);
+            tma_load_3d_if(ld0, dst + K_SLAB + bi * 8192, &kn_of(s.job), &bar->k_full[st], 0, 64, gb);
+            tma_load_2d_if(ld0, dst + 2 * K_SLAB + bi * 8192, &kp_of(s.job), &bar->k_full[st], 0, (blk0 + bi) * 64);
         }
     };
     auto issue_v = [&](const Segment& s, int e, int ring_pos, uint32_t ld) {
         if (FP8) {
             const int sq = ring_pos % p.vq_stages;
             mbar_arrive_expect_tx_if(ld, &bar->vq_full[sq], VQ_BYTES);
-            tma_load_3d_if(ld, sVq + sq * VQ_BYTES, &tm_vt, &bar->vq_full[sq], 0, tile_of(s, e) * 64, s.h);
+            tma_load_3d_if(ld, sVq + sq * VQ_BYTES, &vt_of(s.job), &bar->vq_full[sq], 0, tile_of(s, e) * 64, s.h);
             return;
         }
         const int st = ring_pos % p.v_stages;
@@ -235,7 +276,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         mbar_arrive_expect_tx_if(ld, &bar->v_full[st], V_TILE_BYTES);
 #pragma unroll
         for (int bi = 0; bi < BLK; ++bi)
-            tma_load_4d_if(ld, sV + st * V_TILE_BYTES + bi * 16384, &tm_vt, &bar->v_full[st], 0, 0, blk0 + bi, s.h);
+            tma_load_4d_if(ld, sV + st * V_TILE_BYTES + bi * 16384, &vt_of(s.job), &bar->v_full[st], 0, 0, blk0 + bi, s.h);
     };
 
     // Warp 0 initialises the barriers (one per lane) and at once issues the first segment's Q and
@@ -248,11 +289,11 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         n_pre_k = min(k_depth, s0.cnt);
         n_pre_v = min(v_depth, s0.cnt);
         if (warp == 2) {
-            if (lane == 0) prefetch_tmap(&tm_qn);
-            if (lane == 1) prefetch_tmap(&tm_qp);
-            if (lane == 2) prefetch_tmap(&tm_kn);
-            if (lane == 3) prefetch_tmap(&tm_kp);
-            if (lane == 4) prefetch_tmap(&tm_vt);
+            if (lane == 0) prefetch_tmap(&qn_of(s0.job));
+            if (lane == 1) prefetch_tmap(&qp_of(s0.job));
+            if (lane == 2) prefetch_tmap(&kn_of(s0.job));
+            if (lane == 3) prefetch_tmap(&kp_of(s0.job));
+            if (lane == 4) prefetch_tmap(&vt_of(s0.job));
             asm volatile("bar.sync 1, 64;\n" ::: "memory");   // warp 0 has initialised the barriers
             asm volatile("bar.sync 2, 64;\n" ::: "memory");   // ... and issued Q and the first K tile (needed first)
             for (int e = 0; e < n_pre_v; ++e) issue_v(s0, e, e, ld2);
@@ -460,10 +501,10 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         bool ok = true;
         for (int g = g_begin; g < g_end && ok;) {
             const Segment s = segment_at(g);
-            const int tile_row0 = s.row0 + (MODE_Y ? 0 : i * 128);
+                const int tile_row0 = s.row0 + (MODE_Y ? 0 : i * 128);
             const int b = lane_has_row ? tile_row0 + row : 0x3fffffff;
             const int nt = i == 0 ? s.n_str0 : s.n_str1;
-            const bool warp_has_rows = tile_row0 + (M64 ? (warp & 3) * 16 : lg) < p.B;   // warp-uniform: the warp's first row is a real request
+            const bool warp_has_rows = tile_row0 + (M64 ? (warp & 3) * 16 : lg) < rows_of(s.job);   // warp-uniform: the warp's first row is a real request
             float m_ref = -INFINITY, m_ref_b = -INFINITY;   // (M = 64: reference exponents of this thread's rows A and B)
             uint64_t l_sum2 = pack_f32x2(0.f, 0.f), l_sum2b = pack_f32x2(0.f, 0.f);   // row sum of the probabilities, as four partial sums
             // (8-bit cache: the accumulated logits are the true ones divided by the scale of this head's K, see below)
@@ -485,7 +526,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 }
                 const uint32_t s_addr = tmem_base + ((uint32_t)lg << 16) + s_col(i, u);
                 const int tile = tile_of(s, entry_of(j, i));
-                const int valid = min(TOK, p.Ls - tile * TOK);
+                const int valid = min(TOK, tokens_of(s.job) - tile * TOK);
                 if (M64) {
                     // M = 64 accumulators: the warp's 16 rows sit in the first 16 lanes of its lane group.  They are
                     // read as fragments, so that all 32 threads work: thread t holds 16 of the 64 logits of row
@@ -700,7 +741,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
             // streams worked on the same query rows: stream 1 publishes its softmax state, stream 0 merges both
             // accumulators (same tensor-memory lanes) and writes one partial.
             const int slot = s.slot_seg;
-            const bool owns_rows = MODE_Y ? i == 0 : (i == 0 || s.row0 + 128 < p.B);
+            const bool owns_rows = MODE_Y ? i == 0 : (i == 0 || s.row0 + 128 < rows_of(s.job));
             if (nt > 0) {
                 const int u_last = used + nt - 1;
                 ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_done[i][u_last & 1], (u_last >> 1) & 1, abort_flag));
@@ -740,7 +781,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 }
                 if (nt > 0 && warp_has_rows) {
                     const uint32_t o_addr = tmem_base + ((uint32_t)lg << 16) + 256u + (uint32_t)(MODE_Y ? 0 : i) * 128u;
-                    float* dst = p.o_part + (((int64_t)slot * p.part_rows + b) * p.H + s.h) * 128;
+                    float* dst = o_part_of(s.job) + (((int64_t)slot * p.part_rows + b) * p.H + s.h) * 128;
 #pragma unroll 1
                     for (int c = 0; c < 4; ++c) {
                         uint32_t orr[32];
@@ -755,20 +796,20 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
 #pragma unroll
                             for (int q = 0; q < 32; ++q) v[q] = fmaf(__uint_as_float(orr[q]), a1, v[q]);
                         }
-                        if (b < p.B) {
+                        if (b < rows_of(s.job)) {
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
                                 *reinterpret_cast<float4*>(dst + c * 32 + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                         }
                     }
-                    if (b < p.B) p.lse_part[((int64_t)slot * p.part_rows + b) * p.H + s.h] = lse2 * kLn2;
-                } else if (nt == 0 && owns_rows && b < p.B) {
-                    p.lse_part[((int64_t)slot * p.part_rows + b) * p.H + s.h] = -INFINITY;   // this stream had no tile
+                    if (b < rows_of(s.job)) lse_part_of(s.job)[((int64_t)slot * p.part_rows + b) * p.H + s.h] = lse2 * kLn2;
+                } else if (nt == 0 && owns_rows && b < rows_of(s.job)) {
+                    lse_part_of(s.job)[((int64_t)slot * p.part_rows + b) * p.H + s.h] = -INFINITY;   // this stream had no tile
                 }
                 // the segment that ends a head marks the head's unused slots as empty
-                if (s.last_of_col && owns_rows && b < p.B) {
-                    for (int ss = s.slot_seg + 1; ss < p.n_seg_max; ++ss)
-                        p.lse_part[((int64_t)ss * p.part_rows + b) * p.H + s.h] = -INFINITY;
+                if (s.last_of_col && owns_rows && b < rows_of(s.job)) {
+                    for (int ss = s.slot_seg + 1; ss < n_slots_of(s.job); ++ss)
+                        lse_part_of(s.job)[((int64_t)ss * p.part_rows + b) * p.H + s.h] = -INFINITY;
                 }
                 // the accumulator(s) just read may be overwritten by the next segment
                 tc_fence_before();
@@ -932,26 +973,36 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // pays the fixed cost and a partial slot; with 64-token tiles a further slot per head is also charged
 // the extra read it causes in the combine).  Stream-K is taken when its modelled cost is lower (by at
 // least 5% in the HBM-bound regime of 64-token tiles).
-void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
+//
+// `n` prefixes (their tile counts in `tiles`): the sequence holds all prefixes' tiles of a head, then the next head's;
+// n_slots[i] are the slots of prefix i.
+static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
     // (8-bit cache: always 64-token tiles, row groups of 128 requests)
     const bool mode_y = fp8 || B <= 128;
     const int tok = mode_y ? 64 : 128;
     const int m_groups = fp8 ? (B + 127) / 128 : (mode_y ? 1 : (B + 255) / 256);
-    const int n_tiles = (int)((Ls + tok - 1) / tok);
+    int n_tiles = 0;   // per head, over all prefixes
+    for (int i = 0; i < n; ++i) {
+        n_tiles += (int)((Ls[i] + tok - 1) / tok);
+        n_slots[i] = 0;
+    }
     const long long T = (long long)H * n_tiles;
     if (T <= 0) {
         *n_ranges = 0;
-        *n_slots = 0;
         return;
     }
-    // partial slots a head needs when the T tiles are cut into R ranges (ranges [0, rem) hold per + 1 tiles)
-    auto slots_for = [&](long long R) {
+    // largest number of partial slots a (prefix, head) needs (over the prefixes, or of prefix `only`) when the T tiles are cut into R ranges (ranges [0, rem) hold per + 1 tiles)
+    auto slots_for = [&](long long R, int only = -1) {
         const long long per = T / R, rem = T % R, big = rem * (per + 1);
         auto range_of = [&](long long t) { return t < big ? t / (per + 1) : rem + (t - big) / per; };
         int seg_max = 1;
         for (long long h = 0; h < H; ++h) {
-            const long long first = h * n_tiles, last = first + n_tiles - 1;
-            seg_max = std::max(seg_max, (int)(range_of(last) - range_of(first)) + 1);
+            long long first = h * n_tiles;
+            for (int i = 0; i < n; ++i) {
+                const long long cnt = (Ls[i] + tok - 1) / tok, last = first + cnt - 1;
+                if (cnt > 0 && (only < 0 || only == i)) seg_max = std::max(seg_max, (int)(range_of(last) - range_of(first)) + 1);
+                first += cnt;
+            }
         }
         return seg_max;
     };
@@ -993,73 +1044,136 @@ void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_r
     }
     const int R = stream_k ? r_stream : H * ns_best;
     *n_ranges = R;
-    *n_slots = slots_for(R);   // the kernel uses the same partition
+    for (int i = 0; i < n; ++i)
+        if (Ls[i] > 0) n_slots[i] = slots_for(R, i);   // the kernel uses the same partition
 }
+
+void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
+    plan_sequence(B, H, &Ls, 1, n_sm, schedule, n_ranges, n_slots, fp8);
+}
+
+void naive_sm100_plan_multi(int max_rows, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots) {
+    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false);
+}
+
+
+namespace {
+
+constexpr int kJobs = kNaiveJobsPerLaunch;
+
+// tensor maps of a job's queries
+cudaError_t query_tmaps(const NaiveAttnSm100& a, CUtensorMap* tm_qn, CUtensorMap* tm_qp) {
+    const uint32_t rows = (a.fp8_mult != nullptr && a.B <= 64) ? 64u : 128u;
+    {
+        uint64_t dims[3] = {128, (uint64_t)a.H, (uint64_t)a.B};
+        uint64_t str[2] = {128 * 2, (uint64_t)a.H * 128 * 2};
+        uint32_t box[3] = {64, 1, rows};
+        cudaError_t e = make_tmap_bf16(tm_qn, a.q_nope, 3, dims, str, box);
+        if (e != cudaSuccess) return e;
+    }
+    uint64_t dims[3] = {64, (uint64_t)a.H, (uint64_t)a.B};
+    uint64_t str[2] = {64 * 2, (uint64_t)a.H * 64 * 2};
+    uint32_t box[3] = {64, 1, rows};
+    return make_tmap_bf16(tm_qp, a.q_pe, 3, dims, str, box);
+}
+
+// Launch parameters for `n_tiles` tiles per head and at most `rows` query rows per prefix, and the shared memory.
+cudaError_t fill_params(const NaiveAttnSm100& a, int rows, long long n_tiles, NaiveSm100Params* p, int* smem) {
+    const bool fp8 = a.fp8_mult != nullptr, mode_y = fp8 || rows <= 128;
+    const int tok = mode_y ? 64 : 128;
+    p->B = a.B; p->H = a.H; p->Ls = a.Ls; p->Ls_pad = (a.Ls + 127) / 128 * 128;
+    p->part_rows = a.part_rows > 0 ? a.part_rows : a.B;
+    p->m_groups = fp8 ? (rows + 127) / 128 : (mode_y ? 1 : (rows + 255) / 256);
+    p->n_ranges = a.n_ranges;
+    const long long T = (long long)a.H * n_tiles;
+    if (T >= (1LL << 31) || a.n_ranges > T) return cudaErrorInvalidValue;
+    p->n_tiles = (int)n_tiles;
+    p->per = (int)(T / a.n_ranges);
+    p->rem = (int)(T % a.n_ranges);
+    p->n_seg_max = a.n_slots;
+    p->k_stages = fp8 ? (rows <= 64 ? 3 : 2) : (mode_y ? 4 : 2);   // (8-bit cache: the 128-row query tile takes 24 KB more)
+    p->v_stages = fp8 ? (rows <= 64 ? 3 : 2) : (mode_y ? 4 : 1);
+    p->kq_stages = fp8 ? 4 : 0;
+    p->vq_stages = fp8 ? 4 : 0;
+    p->mult = a.fp8_mult;
+    p->scale_log2 = a.scale * kLog2e;
+    p->o_part = a.o_part; p->lse_part = a.lse_part; p->status = a.status;
+    const int k_tile = fp8 ? 16384 : tok * 384, v_tile = mode_y ? 16384 : 32768;
+    *smem = ((fp8 && rows <= 64) ? Q_TILE_BYTES / 2 : (mode_y ? 1 : 2) * Q_TILE_BYTES) + p->k_stages * k_tile + p->v_stages * v_tile +
+            p->kq_stages * 16384 + p->vq_stages * 8192 + 1024 + (int)sizeof(Barriers) + 64;
+    return *smem > kNaiveSmemMax ? cudaErrorInvalidValue : cudaSuccess;
+}
+
+}  // namespace
 
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s) {
     if (a.B <= 0 || a.Ls <= 0 || a.n_ranges <= 0) return cudaSuccess;
     const bool fp8 = a.fp8_mult != nullptr;
-    CUtensorMap tm_qn, tm_qp;
-    {
-        uint64_t dims[3] = {128, (uint64_t)a.H, (uint64_t)a.B};
-        uint64_t str[2] = {128 * 2, (uint64_t)a.H * 128 * 2};
-        uint32_t box[3] = {64, 1, (fp8 && a.B <= 64) ? 64u : 128u};
-        cudaError_t e = make_tmap_bf16(&tm_qn, a.q_nope, 3, dims, str, box);
-        if (e != cudaSuccess) return e;
-    }
-    {
-        uint64_t dims[3] = {64, (uint64_t)a.H, (uint64_t)a.B};
-        uint64_t str[2] = {64 * 2, (uint64_t)a.H * 64 * 2};
-        uint32_t box[3] = {64, 1, (fp8 && a.B <= 64) ? 64u : 128u};
-        cudaError_t e = make_tmap_bf16(&tm_qp, a.q_pe, 3, dims, str, box);
-        if (e != cudaSuccess) return e;
-    }
-    const bool mode_y = fp8 || a.B <= 128;
-    const int tok = mode_y ? 64 : 128;
+    const int tok = naive_sm100_tile_tokens(a.B, fp8);
     NaiveSm100Params p{};
-    p.B = a.B; p.H = a.H; p.Ls = a.Ls; p.Ls_pad = (a.Ls + 127) / 128 * 128;
-    p.part_rows = a.part_rows > 0 ? a.part_rows : a.B;
-    p.m_groups = fp8 ? (a.B + 127) / 128 : (mode_y ? 1 : (a.B + 255) / 256);
-    p.n_tiles = (a.Ls + tok - 1) / tok;
-    p.n_ranges = a.n_ranges;
-    {
-        const long long T = (long long)a.H * p.n_tiles;
-        if (T >= (1LL << 31) || a.n_ranges > T) return cudaErrorInvalidValue;
-        p.per = (int)(T / a.n_ranges);
-        p.rem = (int)(T % a.n_ranges);
+    CUtensorMap tm_qn, tm_qp;
+    int smem = 0;
+    cudaError_t e = fill_params(a, a.B, (a.Ls + tok - 1) / tok, &p, &smem);
+    if (e == cudaSuccess) e = query_tmaps(a, &tm_qn, &tm_qp);
+    if (e != cudaSuccess) return e;
+    auto launch = [&](auto* kernel, int threads) {
+        return launch_pdl(kernel, dim3(p.n_ranges * p.m_groups), dim3(threads), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p,
+                          NaiveSm100Jobs<1>{});
+    };
+    if (fp8) return a.B <= 64 ? launch(naive_attn_sm100_kernel<64, true, true, 1>, 512) : launch(naive_attn_sm100_kernel<64, false, true, 1>, 512);
+    // (up to 64 rows half-height MMAs: the padding rows 64..127 of the query tile cost tensor-pipe time and power)
+    if (a.B <= 64) return launch(naive_attn_sm100_kernel<64, true, false, 1>, 384);
+    if (a.B <= 128) return launch(naive_attn_sm100_kernel<64, false, false, 1>, 384);
+    return launch(naive_attn_sm100_kernel<128, false, false, 1>, 384);
+}
+
+cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    if (n > kJobs) return cudaErrorInvalidValue;
+    NaiveSm100Jobs<kJobs> jobs{};
+    jobs.n = n;
+    int rows = 0;
+    long long n_tiles = 0;
+    for (int i = 0; i < n; ++i) {
+        if (a[i].B < 1 || a[i].B > 128 || a[i].Ls < 1 || a[i].fp8_mult || a[i].H != a->H || a[i].n_ranges != a->n_ranges)
+            return cudaErrorInvalidValue;
+        rows = std::max(rows, a[i].B);
+        NaiveSm100Job& j = jobs.j[i];
+        const cudaError_t e = query_tmaps(a[i], &j.tm_qn, &j.tm_qp);
+        if (e != cudaSuccess) return e;
+        j.tm_kn = *a[i].tm_kn;
+        j.tm_kp = *a[i].tm_kp;
+        j.tm_vt = *a[i].tm_vt;
+        j.B = a[i].B; j.Ls = a[i].Ls; j.Ls_pad = (a[i].Ls + 127) / 128 * 128;
+        j.n_tiles = (a[i].Ls + 63) / 64;
+        j.tile0 = (int)n_tiles;
+        j.n_seg_max = a[i].n_slots;
+        j.o_part = a[i].o_part; j.lse_part = a[i].lse_part;
+        n_tiles += j.n_tiles;
     }
-    p.n_seg_max = a.n_slots;
-    p.k_stages = fp8 ? (a.B <= 64 ? 3 : 2) : (mode_y ? 4 : 2);   // (8-bit cache: the 128-row query tile takes 24 KB more)
-    p.v_stages = fp8 ? (a.B <= 64 ? 3 : 2) : (mode_y ? 4 : 1);
-    p.kq_stages = fp8 ? 4 : 0;
-    p.vq_stages = fp8 ? 4 : 0;
-    p.mult = a.fp8_mult;
-    p.scale_log2 = a.scale * kLog2e;
-    p.o_part = a.o_part; p.lse_part = a.lse_part; p.status = a.status;
-    const int k_tile = fp8 ? 16384 : tok * 384, v_tile = mode_y ? 16384 : 32768;
-    const int smem = ((fp8 && a.B <= 64) ? Q_TILE_BYTES / 2 : (mode_y ? 1 : 2) * Q_TILE_BYTES) + p.k_stages * k_tile + p.v_stages * v_tile +
-                     p.kq_stages * 16384 + p.vq_stages * 8192 + 1024 + (int)sizeof(Barriers) + 64;
-    dim3 grid(p.n_ranges * p.m_groups, 1, 1);
-    if (smem > kNaiveSmemMax) return cudaErrorInvalidValue;
-    if (fp8) {
-        if (a.B <= 64)
-            return launch_pdl(naive_attn_sm100_kernel<64, true, true>, grid, dim3(512), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p);
-        return launch_pdl(naive_attn_sm100_kernel<64, false, true>, grid, dim3(512), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p);
-    }
-    if (mode_y) {
-        if (a.B <= 64)   // half-height MMAs: the padding rows 64..127 of the query tile cost tensor-pipe time and power
-            return launch_pdl(naive_attn_sm100_kernel<64, true, false>, grid, dim3(384), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p);
-        return launch_pdl(naive_attn_sm100_kernel<64, false, false>, grid, dim3(384), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p);
-    }
-    return launch_pdl(naive_attn_sm100_kernel<128, false, false>, grid, dim3(384), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p);
+    NaiveSm100Params p{};
+    int smem = 0;
+    const cudaError_t e = fill_params(a[0], rows, n_tiles, &p, &smem);
+    if (e != cudaSuccess) return e;
+    const NaiveSm100Job& j0 = jobs.j[0];
+    auto launch = [&](auto* kernel) {
+        return launch_pdl(kernel, dim3(p.n_ranges), dim3(384), smem, s, j0.tm_qn, j0.tm_qp, j0.tm_kn, j0.tm_kp, j0.tm_vt, p, jobs);
+    };
+    return rows <= 64 ? launch(naive_attn_sm100_kernel<64, true, false, kJobs>) : launch(naive_attn_sm100_kernel<64, false, false, kJobs>);
 }
 
 cudaError_t set_attrs_naive_sm100() {
-    cudaError_t e = cudaFuncSetAttribute(naive_attn_sm100_kernel<64, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(naive_attn_sm100_kernel<64, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(naive_attn_sm100_kernel<128, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(naive_attn_sm100_kernel<64, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(naive_attn_sm100_kernel<64, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
+    cudaError_t e = cudaSuccess;
+    auto opt_in = [&](auto* kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
+    };
+    opt_in(naive_attn_sm100_kernel<64, true, false, 1>);
+    opt_in(naive_attn_sm100_kernel<64, false, false, 1>);
+    opt_in(naive_attn_sm100_kernel<128, false, false, 1>);
+    opt_in(naive_attn_sm100_kernel<64, true, true, 1>);
+    opt_in(naive_attn_sm100_kernel<64, false, true, 1>);
+    opt_in(naive_attn_sm100_kernel<64, true, false, kJobs>);
+    opt_in(naive_attn_sm100_kernel<64, false, false, kJobs>);
     return e;
 }
 
