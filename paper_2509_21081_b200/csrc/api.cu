@@ -464,6 +464,7 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     if (e == cudaSuccess) e = set_attrs_naive_sm100();
     if (e == cudaSuccess) e = set_attrs_absorb_sm100();
     if (e == cudaSuccess) e = set_attrs_gemm_sm100();
+    if (e == cudaSuccess) e = set_attrs_project_sm100();
     if (e == cudaSuccess) e = set_attrs_q_absorb_sm100();
     if (e == cudaSuccess) e = set_attrs_attn_mma();
     if (e == cudaSuccess) e = set_attrs_gemm_tn();
@@ -902,12 +903,11 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
         //     LSE combine (line 8)
         prof_before(TYPHOON_MLA_KERNEL_W_UV, s);
         if (tc) {
-            GemmTN g2{o_lat, (int64_t)H * 512, 512, sh->w_uv, 512, 128 * 512, nullptr, 0, 0, B, 128, 512, H, false};
             CombineEpilogue ce;
             ce.o_naive = o_part_n; ce.lse_naive = lse_part_n; ce.n_naive = pl.n_slots_naive;
             ce.lse_abs = lse_a; ce.out = out; ce.lse_out = lse_out; ce.H = H;
             ce.out_fp32 = out_fp32 ? 1 : 0;
-            e = launch_gemm_tn_sm100(g2, sh->status, s, &ce);
+            e = launch_project_sm100(o_lat, sh->w_uv, B, sh->num_sms, sh->status, s, ce);
             combined = true;
         } else {
             GemmTN g2{o_lat, (int64_t)H * 512, 512, sh->w_uv, 512, 128 * 512, o_abs, (int64_t)H * 128, 128,

@@ -27,8 +27,7 @@ struct GemmParams {
     int M, N, K, c_block_n, c_tile64;
     int a_batched, b_batched, a_swap;
     int* status;
-    int out_mode;          // 0: bf16 C, 1: fp32 C, 2: LSE combine epilogue (N == 128, row = request, batch = head)
-    CombineEpilogue ce;
+    int out_fp32;
 };
 
 __global__ void __launch_bounds__(192) gemm_tn_sm100_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -96,79 +95,11 @@ __global__ void __launch_bounds__(192) gemm_tn_sm100_kernel(const __grid_constan
     } else {
         const int lg = (warp & 3) * 32;
         const int row = m0 + lg + lane;
-        // Combine epilogue, first half: while the main loop runs, this thread (one request row) reads the
-        // LSEs of its (request, head), derives the merge weights and accumulates the weighted naive-side
-        // partials in registers, so that their memory latency is hidden behind the GEMM.
-        float accn[128];
-        float wa = 0.f, inv = 0.f, m = -INFINITY, zsum = 0.f;
-        int64_t bh = 0;
-        const bool live = p.out_mode == 2 && row < p.M;
-        if (p.out_mode == 2) {
-            const CombineEpilogue& ce = p.ce;
-            const int64_t BH = (int64_t)p.M * ce.H;
-            bh = (int64_t)row * ce.H + z;
-#pragma unroll
-            for (int q = 0; q < 128; ++q) accn[q] = 0.f;
-            if (live) {
-                const float la = ce.lse_abs[bh];
-                m = la;
-                for (int i = 0; i < ce.n_naive; ++i) m = fmaxf(m, ce.lse_naive[i * BH + bh]);
-                if (m != -INFINITY) {
-                    wa = (la == -INFINITY) ? 0.f : __expf(la - m);
-                    zsum = wa;
-                    for (int i = 0; i < ce.n_naive; ++i) {
-                        const float l = ce.lse_naive[i * BH + bh];
-                        if (l == -INFINITY) continue;          // empty partial: its O slot was never written
-                        const float w = __expf(l - m);
-                        zsum += w;
-                        const float4* src = reinterpret_cast<const float4*>(ce.o_naive + (i * BH + bh) * 128);
-#pragma unroll
-                        for (int q = 0; q < 32; ++q) {
-                            const float4 v = src[q];
-                            accn[4 * q] += w * v.x; accn[4 * q + 1] += w * v.y; accn[4 * q + 2] += w * v.z; accn[4 * q + 3] += w * v.w;
-                        }
-                    }
-                }
-                inv = zsum > 0.f ? 1.f / zsum : 0.f;
-            }
-        }
         const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_full, 0, abort_flag));
         tc_fence_after();
         if (ok) {
-            if (p.out_mode == 2) {
-                // second half: add the absorb-side row (the accumulator, already normalised) with its weight,
-                // normalise (Algorithm 1 line 8) and write the final bf16 row
-                const CombineEpilogue& ce = p.ce;
-#pragma unroll
-                for (int c = 0; c < BN / 32; ++c) {
-                    uint32_t r[32];
-                    tmem_ld32(tmem_base + ((uint32_t)lg << 16) + c * 32, r);
-                    tmem_ld_wait();
-                    if (!live) continue;
-                    __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(ce.out) + bh * 128 + c * 32;
-                    float* dstf = reinterpret_cast<float*>(ce.out) + bh * 128 + c * 32;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float o[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float oa = wa > 0.f ? wa * __uint_as_float(r[j * 8 + e]) : 0.f;
-                            o[e] = (accn[c * 32 + j * 8 + e] + oa) * inv;
-                        }
-                        if (ce.out_fp32) {
-                            *reinterpret_cast<float4*>(dstf + j * 8) = make_float4(o[0], o[1], o[2], o[3]);
-                            *reinterpret_cast<float4*>(dstf + j * 8 + 4) = make_float4(o[4], o[5], o[6], o[7]);
-                        } else {
-                            uint4 v;
-                            v.x = pack_bf16(o[0], o[1]); v.y = pack_bf16(o[2], o[3]);
-                            v.z = pack_bf16(o[4], o[5]); v.w = pack_bf16(o[6], o[7]);
-                            *reinterpret_cast<uint4*>(dst + j * 8) = v;
-                        }
-                    }
-                }
-                if (live && ce.lse_out) ce.lse_out[bh] = (m == -INFINITY) ? -INFINITY : m + __logf(zsum);
-            } else {
-                uint8_t* cbase = reinterpret_cast<uint8_t*>(p.C) + (int64_t)z * p.c_batch * (p.out_mode == 1 ? 4 : 2);
+            {
+                uint8_t* cbase = reinterpret_cast<uint8_t*>(p.C) + (int64_t)z * p.c_batch * (p.out_fp32 ? 4 : 2);
 #pragma unroll 1
                 for (int c = 0; c < BN / 32; ++c) {
                     uint32_t r[32];
@@ -179,7 +110,7 @@ __global__ void __launch_bounds__(192) gemm_tn_sm100_kernel(const __grid_constan
                         const int64_t off = p.c_tile64 ? (((int64_t)(row >> 6) * (p.N >> 6) + (gn >> 6)) << 12) + ((row & 63) << 6) + (gn & 63)
                                             : p.c_block_n ? ((int64_t)(gn >> 6) * p.M + row) * 64 + (gn & 63)
                                                           : (int64_t)row * p.ldc + gn;
-                        if (p.out_mode == 1) {
+                        if (p.out_fp32) {
                             float4* crow = reinterpret_cast<float4*>(cbase + off * 4);
 #pragma unroll
                             for (int j = 0; j < 8; ++j)
@@ -221,10 +152,9 @@ cudaError_t set_attrs_gemm_sm100() {
     return cudaFuncSetAttribute(gemm_tn_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
 }
 
-cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s, const CombineEpilogue* ce) {
+cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s) {
     if (g.M <= 0 || g.batch <= 0) return cudaSuccess;
     if (g.N % BN != 0 || g.K % BK != 0) return cudaErrorInvalidValue;
-    if (ce && g.N != BN) return cudaErrorInvalidValue;
     CUtensorMap tmA, tmB;
     // When the batch stride of A is smaller than its row stride (activations laid out [M, batch, K]) the
     // tensor map is built with the batch dimension in the middle so that strides stay increasing.
@@ -252,7 +182,7 @@ cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s, c
         if (e != cudaSuccess) return e;
     }
     GemmParams p{g.C, g.ldc, g.c_batch, g.M, g.N, g.K, g.c_block_n, g.c_tile64 ? 1 : 0, g.a_batch != 0, g.b_batch != 0, a_swap ? 1 : 0, status,
-                 ce ? 2 : (g.out_fp32 ? 1 : 0), ce ? *ce : CombineEpilogue{}};
+                 g.out_fp32 ? 1 : 0};
     dim3 grid(g.N / BN, (g.M + BM - 1) / BM, g.batch);
     return launch_pdl(gemm_tn_sm100_kernel, grid, dim3(192), SMEM_BYTES, s, tmA, tmB, p);
 }

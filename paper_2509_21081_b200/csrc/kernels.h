@@ -17,6 +17,7 @@ cudaError_t set_attrs_naive_sm100();
 cudaError_t set_attrs_absorb_sm100();
 cudaError_t set_attrs_stacked_sm100();
 cudaError_t set_attrs_gemm_sm100();
+cudaError_t set_attrs_project_sm100();
 cudaError_t set_attrs_q_absorb_sm100();
 cudaError_t set_attrs_attn_mma();
 cudaError_t set_attrs_gemm_tn();
@@ -53,8 +54,9 @@ struct GemmTN {
 cudaError_t launch_gemm_tn(const GemmTN& g, cudaStream_t s);
 // tcgen05/TMEM/TMA version (bf16 output only; N % 128 == 0, K % 64 == 0).  `status` (device int,
 // may be null) is set non-zero if a bounded wait inside the kernel expired.
-// Optional fused epilogue (N must be 128): the accumulator row of (request m, head z) is taken as the
-// normalised absorb-side output and merged with n_naive naive-side partials by their LSEs.
+cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s);
+// Output projection + LSE combine: o_lat [B][H][512] bf16 times w_uv [H][128][512] bf16 is the normalised absorb side of
+// every (request, head), merged with n_naive naive-side partials by their LSEs.
 struct CombineEpilogue {
     const float* o_naive = nullptr;    // [n_naive][B][H][128]
     const float* lse_naive = nullptr;  // [n_naive][B][H]
@@ -65,7 +67,7 @@ struct CombineEpilogue {
     int H = 0;
     int out_fp32 = 0;                  // `out` is fp32 [B][H][128] (a partial result for a later merge)
 };
-cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s, const CombineEpilogue* ce = nullptr);
+cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int n_sm, int* status, cudaStream_t s, const CombineEpilogue& ce);
 
 // Query absorption on tcgen05 (one CTA per head and 128 requests); tm_w from make_q_absorb_tmap.
 cudaError_t make_q_absorb_tmap(const void* w_uk_t, int H, CUtensorMap* tm_w);
