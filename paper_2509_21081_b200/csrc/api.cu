@@ -463,7 +463,7 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     // opt-in shared-memory sizes of every kernel, once per device and off the decode path
     if (e == cudaSuccess) e = set_attrs_naive_sm100();
     if (e == cudaSuccess) e = set_attrs_absorb_sm100();
-    if (e == cudaSuccess) e = set_attrs_gemm_sm100();
+    if (e == cudaSuccess) e = set_attrs_expand_sm100();
     if (e == cudaSuccess) e = set_attrs_project_sm100();
     if (e == cudaSuccess) e = set_attrs_q_absorb_sm100();
     if (e == cudaSuccess) e = set_attrs_attn_mma();
@@ -537,27 +537,24 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
         typhoon_mla_free(sh);
         return cuda_fail(e);
     }
-    e = cudaMemsetAsync(sh->status, 0, 256, s);
-    if (e == cudaSuccess) e = launch_transpose_bf16(w_uk, sh->w_uk_t, 128, 512, H, s);
-    if (e == cudaSuccess && Ls > 0) {
-        e = launch_copy_pad_rows(ckv_shared, ld_ckv, sh->ckv, (int)Ls, (int)Lp, 512, s);
-        if (e == cudaSuccess) e = launch_copy_pad_rows(kpe_shared, ld_kpe, sh->kpe, (int)Ls, (int)Lp, 64, s);
-        if (e == cudaSuccess) {  // K_nope[h] = ckv * W_UK[h]^T
-            GemmTN g{sh->ckv, 512, 0, w_uk, 512, 128 * 512, k_dst, 128, (int64_t)Lp * 128,
-                     (int)Lp, 128, 512, H, false, 0, true};
-            e = tc ? launch_gemm_tn_sm100(g, sh->status, s) : launch_gemm_tn(g, s);
-            if (e == cudaSuccess && sh->fp8)
-                e = launch_quantize_e4m3(k_dst, false, H, (int64_t)Lp, sh->k8, reinterpret_cast<uint32_t*>(sh->fp8_f + 2 * H),
-                                         sh->fp8_f, s);
-        }
-        if (e == cudaSuccess) {  // V^T[h] = W_UV[h] * ckv^T
-            GemmTN g{w_uv, 512, 128 * 512, sh->ckv, 512, 0, v_dst, (int64_t)Lp, (int64_t)(128 * Lp),
-                     128, (int)Lp, 512, H, false, 64};
-            e = tc ? launch_gemm_tn_sm100(g, sh->status, s) : launch_gemm_tn(g, s);
-            if (e == cudaSuccess && sh->fp8)
-                e = launch_quantize_e4m3(v_dst, true, H, (int64_t)Lp, sh->v8, reinterpret_cast<uint32_t*>(sh->fp8_f + 2 * H),
-                                         sh->fp8_f + H, s);
-        }
+    e = launch_prepare_layout(w_uk, sh->w_uk_t, H, ckv_shared, ld_ckv, sh->ckv, kpe_shared, ld_kpe, sh->kpe, Ls, (int64_t)Lp, sh->status, s);
+    // K_nope[h] = ckv * W_UK[h]^T and V^T[h] = W_UV[h] * ckv^T; with 8-bit storage each is encoded before the scratch takes
+    // the next
+    auto expand = [&](bool k, bool v) {
+        if (tc) return launch_expand_sm100(sh->ckv, (int64_t)Lp, w_uk, w_uv, H, k ? k_dst : nullptr, v ? v_dst : nullptr, n_sm, sh->status, s);
+        cudaError_t r = cudaSuccess;
+        if (k) r = launch_gemm_tn(GemmTN{sh->ckv, 512, 0, w_uk, 512, 128 * 512, k_dst, 128, (int64_t)Lp * 128, (int)Lp, 128, 512, H, false, 0, true}, s);
+        if (v && r == cudaSuccess)
+            r = launch_gemm_tn(GemmTN{w_uv, 512, 128 * 512, sh->ckv, 512, 0, v_dst, (int64_t)Lp, (int64_t)(128 * Lp), 128, (int)Lp, 512, H, false, 64}, s);
+        return r;
+    };
+    if (e == cudaSuccess && Ls > 0 && !sh->fp8) e = expand(true, true);
+    if (e == cudaSuccess && Ls > 0 && sh->fp8) {
+        uint32_t* amax = reinterpret_cast<uint32_t*>(sh->fp8_f + 2 * H);
+        e = expand(true, false);
+        if (e == cudaSuccess) e = launch_quantize_e4m3(k_dst, false, H, (int64_t)Lp, sh->k8, amax, sh->fp8_f, s);
+        if (e == cudaSuccess) e = expand(false, true);
+        if (e == cudaSuccess) e = launch_quantize_e4m3(v_dst, true, H, (int64_t)Lp, sh->v8, amax, sh->fp8_f + H, s);
     }
     if (scratch16) {
         const cudaError_t ef = cudaFreeAsync(scratch16, s);

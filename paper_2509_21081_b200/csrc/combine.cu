@@ -278,32 +278,53 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     if (lse_out != nullptr && lane == 0) lse_out[bh] = (m == -INFINITY) ? -INFINITY : m + __logf(z);
 }
 
-__global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in,
-                                                             __nv_bfloat16* __restrict__ out, int R, int C) {
-    __shared__ __nv_bfloat16 tile[32][34];
-    const int64_t off = (int64_t)blockIdx.z * R * C;
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8) {
-        int r = r0 + i, c = c0 + tx;
-        tile[i][tx] = (r < R && c < C) ? in[off + (int64_t)r * C + c] : __float2bfloat16(0.f);
+// What a prepared prefix keeps besides the expansion (see launch_prepare_layout), one launch of three kinds of blocks.  Bound
+// by memory: 16.8 MB of weights each way at 128 heads and 2.3 KB per token.  The transpose moves 16-byte pieces on both
+// sides of a 64 x 64 tile (rows of 33 words, so that the 2-byte column reads spread over the banks).
+struct LayoutParams {
+    const __nv_bfloat16* w; __nv_bfloat16* w_t; int n_w;                         // n_w = H * 16 tiles
+    const __nv_bfloat16* ckv; int64_t ld_ckv; uint4* ckv_out; int n_ckv;         // n_*: blocks of each kind
+    const __nv_bfloat16* kpe; int64_t ld_kpe; uint4* kpe_out;
+    int64_t L, Lp;
+    int* status;
+};
+__global__ void __launch_bounds__(256) prepare_layout_kernel(LayoutParams p) {
+    sm100::pdl_trigger();
+    sm100::pdl_wait();
+    const int tid = threadIdx.x, blk = blockIdx.x;
+    if (blk < p.n_w) {
+        __shared__ uint32_t tile[64 * 33];
+        const int h = blk >> 4, d0 = (blk & 1) * 64, l0 = ((blk >> 1) & 7) * 64;
+        const __nv_bfloat16* in = p.w + (int64_t)h * 65536 + (int64_t)d0 * 512 + l0;
+        __nv_bfloat16* out = p.w_t + (int64_t)h * 65536 + (int64_t)l0 * 128 + d0;
+#pragma unroll
+        for (int i = tid; i < 512; i += 256) {
+            const uint4 v = *reinterpret_cast<const uint4*>(in + (i >> 3) * 512 + (i & 7) * 8);
+            uint32_t* t = tile + (i >> 3) * 33 + (i & 7) * 4;
+            t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = tid; i < 512; i += 256) {   // row l of the output tile, dims 8 j .. 8 j + 7
+            const int l = i >> 3, j = i & 7, sh = (l & 1) * 16;
+            const uint32_t* t = tile + 8 * j * 33 + (l >> 1);
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = ((t[2 * k * 33] >> sh) & 0xffffu) | ((t[(2 * k + 1) * 33] >> sh) << 16);
+            *reinterpret_cast<uint4*>(out + l * 128 + j * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        if (blk == 0 && tid < 64) p.status[tid] = 0;
+        return;
     }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        int c = c0 + i, r = r0 + tx;
-        if (r < R && c < C) out[off + (int64_t)c * R + r] = tile[tx][i];
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    if (blk < p.n_w + p.n_ckv) {                 // 4 latent rows of 64 pieces per pass
+        for (int64_t i = (int64_t)(blk - p.n_w) * 256 + tid; i < p.Lp * 64; i += (int64_t)p.n_ckv * 256)
+            p.ckv_out[i] = (i >> 6) < p.L ? *reinterpret_cast<const uint4*>(p.ckv + (i >> 6) * p.ld_ckv + (i & 63) * 8) : zero;
+    } else {
+        const int n = gridDim.x - p.n_w - p.n_ckv;
+        for (int64_t i = (int64_t)(blk - p.n_w - p.n_ckv) * 256 + tid; i < p.Lp * 8; i += (int64_t)n * 256)
+            p.kpe_out[i] = (i >> 3) < p.L ? *reinterpret_cast<const uint4*>(p.kpe + (i >> 3) * p.ld_kpe + (i & 7) * 8) : zero;
     }
-}
-
-__global__ void __launch_bounds__(256) copy_pad_rows_kernel(const __nv_bfloat16* __restrict__ in, int64_t ld_in,
-                                                            __nv_bfloat16* __restrict__ out, int L, int Lp, int W8) {
-    int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    int64_t total = (int64_t)Lp * W8;
-    if (idx >= total) return;
-    int row = (int)(idx / W8), ch = (int)(idx % W8);
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (row < L) v = *reinterpret_cast<const uint4*>(in + (int64_t)row * ld_in + ch * 8);
-    *reinterpret_cast<uint4*>(out + ((int64_t)row * W8 + ch) * 8) = v;
 }
 
 // Longest-first launch order for ragged suffixes: perm[] = request indices sorted by descending
@@ -416,21 +437,25 @@ cudaError_t launch_combine(const float* o_naive, const float* lse_naive, int n_n
                       out, lse_out, out_fp32 ? 1 : 0);
 }
 
-cudaError_t launch_transpose_bf16(const void* in, void* out, int R, int C, int batch, cudaStream_t s) {
-    if (R <= 0 || C <= 0 || batch <= 0) return cudaSuccess;
-    dim3 grid((C + 31) / 32, (R + 31) / 32, batch);
-    transpose_bf16_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16*>(in),
-                                               reinterpret_cast<__nv_bfloat16*>(out), R, C);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_copy_pad_rows(const void* in, int64_t ld_in, void* out, int L, int Lp, int W, cudaStream_t s) {
-    if (Lp <= 0) return cudaSuccess;
-    int W8 = W / 8;
-    int64_t total = (int64_t)Lp * W8;
-    copy_pad_rows_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-        reinterpret_cast<const __nv_bfloat16*>(in), ld_in, reinterpret_cast<__nv_bfloat16*>(out), L, Lp, W8);
-    return cudaGetLastError();
+cudaError_t launch_prepare_layout(const void* w_uk, void* w_uk_t, int H, const void* ckv, int64_t ld_ckv, void* ckv_out, const void* kpe,
+                                  int64_t ld_kpe, void* kpe_out, int64_t L, int64_t Lp, int* status, cudaStream_t s) {
+    if (H <= 0) return cudaSuccess;
+    LayoutParams p{};
+    p.w = reinterpret_cast<const __nv_bfloat16*>(w_uk);
+    p.w_t = reinterpret_cast<__nv_bfloat16*>(w_uk_t);
+    p.n_w = H * 16;
+    p.ckv = reinterpret_cast<const __nv_bfloat16*>(ckv);
+    p.ld_ckv = ld_ckv;
+    p.ckv_out = reinterpret_cast<uint4*>(ckv_out);
+    p.n_ckv = (int)std::min<int64_t>((Lp * 64 + 1023) / 1024, 2048);   // (four pieces per thread up to 32768 rows)
+    p.kpe = reinterpret_cast<const __nv_bfloat16*>(kpe);
+    p.ld_kpe = ld_kpe;
+    p.kpe_out = reinterpret_cast<uint4*>(kpe_out);
+    p.L = L;
+    p.Lp = Lp;
+    p.status = status;
+    const int n_kpe = (int)std::min<int64_t>((Lp * 8 + 1023) / 1024, 256);
+    return launch_pdl(prepare_layout_kernel, dim3(p.n_w + p.n_ckv + n_kpe), dim3(256), 0, s, p);
 }
 
 }  // namespace tmla

@@ -16,7 +16,7 @@ extern thread_local bool tl_pdl;
 cudaError_t set_attrs_naive_sm100();
 cudaError_t set_attrs_absorb_sm100();
 cudaError_t set_attrs_stacked_sm100();
-cudaError_t set_attrs_gemm_sm100();
+cudaError_t set_attrs_expand_sm100();
 cudaError_t set_attrs_project_sm100();
 cudaError_t set_attrs_q_absorb_sm100();
 cudaError_t set_attrs_attn_mma();
@@ -52,9 +52,11 @@ struct GemmTN {
     bool c_tile64 = false;
 };
 cudaError_t launch_gemm_tn(const GemmTN& g, cudaStream_t s);
-// tcgen05/TMEM/TMA version (bf16 output only; N % 128 == 0, K % 64 == 0).  `status` (device int,
-// may be null) is set non-zero if a bounded wait inside the kernel expired.
-cudaError_t launch_gemm_tn_sm100(const GemmTN& g, int* status, cudaStream_t s);
+// Prefix expansion on tcgen05: ckv [Lp][512] (Lp a multiple of 128) times w_uk / w_uv [H][128][512] -> k_nope
+// [H, Lp/64, 2, 64, 64] and v_t [H, Lp/64, 128, 64]; a null output is not computed.  `status` (device int, may be null) is
+// set non-zero if a bounded wait inside the kernel expired.
+cudaError_t launch_expand_sm100(const void* ckv, int64_t Lp, const void* w_uk, const void* w_uv, int H, void* k_nope, void* v_t,
+                                int n_sm, int* status, cudaStream_t s);
 // Output projection + LSE combine: o_lat [B][H][512] bf16 times w_uv [H][128][512] bf16 is the normalised absorb side of
 // every (request, head), merged with n_naive naive-side partials by their LSEs.
 struct CombineEpilogue {
@@ -194,10 +196,10 @@ int noalloc_resolve_scratch_for_current_device();
 int api_cuda_fail(cudaError_t e);
 void api_set_last_launches(int n);
 
-// out[c][r] = in[r][c] for each of `batch` matrices [R][C] bf16.
-cudaError_t launch_transpose_bf16(const void* in, void* out, int R, int C, int batch, cudaStream_t s);
-
-// rows [L, W] with stride ld_in -> contiguous padded [Lp, W] (padding zero), bf16
-cudaError_t launch_copy_pad_rows(const void* in, int64_t ld_in, void* out, int L, int Lp, int W, cudaStream_t s);
+// Everything a prepared prefix keeps besides the expansion, in one launch: w_uk [H][128][512] transposed to [H][512][128],
+// the latent rows [L][512] and rope keys [L][64] (row strides ld_*, elements, multiples of 8) copied into contiguous
+// zero-padded [Lp] rows, the 256-byte status block cleared.  L = 0: no rows.
+cudaError_t launch_prepare_layout(const void* w_uk, void* w_uk_t, int H, const void* ckv, int64_t ld_ckv, void* ckv_out, const void* kpe,
+                                  int64_t ld_kpe, void* kpe_out, int64_t L, int64_t Lp, int* status, cudaStream_t s);
 
 }  // namespace tmla
