@@ -115,6 +115,29 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
 
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
     pdl_trigger();
+    // Set-up that touches no global memory runs before the wait for the preceding kernel: barriers (the leading uint64_t
+    // members of the struct, one lane each; p_ready counts the 256 softmax threads, all others one arrival), tensor memory
+    // (no other CTA that uses it fits beside this one's shared memory), tensor maps.
+    if (warp == 0) {
+        uint64_t* all = &sh->q_full;
+        constexpr int n_bars = (int)(offsetof(Shared, tmem_base) / sizeof(uint64_t));
+        for (int i = lane; i < n_bars; i += 32) {
+            uint64_t* m = all + i;
+            mbar_init(m, (m >= &sh->p_ready[0] && m < &sh->o_done[0]) ? 256 : 1);
+        }
+        if (lane == 0) sh->abort_flag = 0;
+        fence_mbar_init();
+        __syncwarp();
+    }
+    if (warp == 1) tmem_alloc(&sh->tmem_base, 512);
+    if (warp == 2) {
+        if (lane == 0) prefetch_tmap(&tm_qa);
+        if (lane == 1) prefetch_tmap(&tm_qp);
+        if (lane == 2) prefetch_tmap(&tm_ckv_sh);
+        if (lane == 3) prefetch_tmap(&tm_kpe_sh);
+        if (lane == 4) prefetch_tmap(&tm_ckv_pg);
+        if (lane == 5) prefetch_tmap(&tm_kpe_pg);
+    }
     pdl_wait();   // the descriptors and Q_A read below are written by the preceding kernel
     // Work items in launch order: the shared-prefix items (chunk fastest, then row group), then the suffix items
     // (chunk fastest, then head group, then request position in longest-first order).
@@ -210,24 +233,7 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         for (int sl = 0; sl < 8; ++sl) tma_prefetch_3d_if(ld0, tc, sl * 64, slot, page);
         tma_prefetch_3d_if(ld0, tk, 0, slot, page);
     };
-    if (warp == 2) {   // otherwise idle: fetch the tensor maps while warp 0 sets up the barriers
-        if (lane == 0) prefetch_tmap(&tm_qa);
-        if (lane == 1) prefetch_tmap(&tm_qp);
-        if (lane == 2) prefetch_tmap(tc);
-        if (lane == 3) prefetch_tmap(tk);
-    }
     if (warp == 0) {
-        // the mbarriers are the leading uint64_t members of the struct, one lane each; p_ready counts the
-        // 256 softmax threads, all others one arrival
-        uint64_t* all = &sh->q_full;
-        constexpr int n_bars = (int)(offsetof(Shared, tmem_base) / sizeof(uint64_t));
-        for (int i = lane; i < n_bars; i += 32) {
-            uint64_t* m = all + i;
-            mbar_init(m, (m >= &sh->p_ready[0] && m < &sh->o_done[0]) ? 256 : 1);
-        }
-        if (lane == 0) sh->abort_flag = 0;
-        fence_mbar_init();
-        __syncwarp();
         if (n_tiles > 0) {
             mbar_arrive_expect_tx_if(ld0, &sh->q_full, TILE_BYTES);
 #pragma unroll 1
@@ -242,7 +248,6 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
             for (int j = STAGES; j < 2 * STAGES; ++j) prefetch_tile(j);
         }
     }
-    if (warp == 1) tmem_alloc(&sh->tmem_base, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

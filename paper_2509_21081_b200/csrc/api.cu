@@ -538,6 +538,9 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
         return cuda_fail(e);
     }
     e = launch_prepare_layout(w_uk, sh->w_uk_t, H, ckv_shared, ld_ckv, sh->ckv, kpe_shared, ld_kpe, sh->kpe, Ls, (int64_t)Lp, sh->status, s);
+    // (without an expansion kernel behind it, an operation that is no kernel keeps a decode step's early reads of w_uk_t behind
+    // the layout kernel's completion)
+    if (e == cudaSuccess && Ls == 0) e = cudaMemsetAsync(sh->status, 0, sz.status, s);
     // K_nope[h] = ckv * W_UK[h]^T and V^T[h] = W_UV[h] * ckv^T; with 8-bit storage each is encoded before the scratch takes
     // the next
     auto expand = [&](bool k, bool v) {
@@ -726,7 +729,6 @@ struct EmptySlots {
 // Launch sequence of one step.  `sh` provides the weights, the absorb-side tensor maps, the side stream
 // and the status word; `mode` is resolved (ABSORB, HYBRID or NAIVE); `pl.n_slots_naive` is the total
 // number of naive partial slots.
-constexpr int kMergeProjectMaxB = 2;   // measured: from 3 requests on the GEMM form (weights read once) is faster
 
 static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const NaiveJob* jobs, int n_jobs,
                 const EmptySlots* empties, int n_empties,
@@ -873,8 +875,11 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
         prof_after(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         if (e != cudaSuccess) return fail(e);
         ++launches;
-        if (n_jobs == 0 && n_empties == 0 && n_chunks > 1 && B <= kMergeProjectMaxB) {
-            // absorb-only, a handful of requests: merge + projection + rounding in one launch
+        if (n_jobs == 0 && n_empties == 0 && n_chunks > 1 && (int64_t)B * H <= sh->num_sms) {
+            // Absorb-only with at most one (request, head) row per SM: merge + projection + rounding in one launch, a block
+            // per row (one block fills an SM's registers).  Measured (B200, us per step, this form / merge and GEMM): 16
+            // heads, 8 requests 21.4 / 23.9; 128 heads, 1 request 28.9 / 33; in two waves it loses: 128 heads, 2 requests
+            // 39.4 / 36.8; 16 heads, 16 requests 27.5 / 24.7.
             prof_before(TYPHOON_MLA_KERNEL_MERGE, s);
             e = launch_merge_project(o_part_a, lse_part_a, n_chunks, B, H, sh->w_uv, out, lse_out, out_fp32, s);
             prof_after(TYPHOON_MLA_KERNEL_MERGE, s);

@@ -128,33 +128,58 @@ __global__ void __launch_bounds__(512) merge_latent_few_kernel(const float* __re
     if (col == 0) lse[bh] = (m == -INFINITY) ? -INFINITY : m + __logf(z);
 }
 
-// Absorb-only step at small batch sizes: merge of the chunk partials, output projection O_A W_UV^T (Algorithm 1
-// line 7) and the final rounding in one launch.  One block per (request, head), 512 threads.  The 128 KB of the
-// head's W_UV (16 warps x 8 rows x 1 KB) are requested into L2 first and arrive while the chunk partials are merged
-// as in merge_latent_kernel; the merged latent row stays in fp32 in shared memory; every warp then forms 8 of the 128
-// outputs as dot products over 512 (16 elements per lane, butterfly sum).  Each block re-reads its head's weights,
-// so this form is for one or two requests (the GEMM form reads them once per 128 requests).
-__global__ void __launch_bounds__(512) merge_project_kernel(const float* __restrict__ o_part,
-                                                            const float* __restrict__ lse_part, int n_chunks, int B,
-                                                            int H, const __nv_bfloat16* __restrict__ w_uv,
-                                                            void* __restrict__ out, float* __restrict__ lse_out,
-                                                            int out_fp32) {
-    sm100::pdl_trigger();
-    sm100::pdl_wait();
+// Absorb-only step of few (request, head) rows: merge of the chunk partials, output projection O_A W_UV^T (Algorithm 1
+// line 7) and the final rounding in one launch.  One block per row, 512 threads: group g of 128 threads takes the chunks g,
+// g + 4, ...; the merged latent row stays in fp32 in shared memory; every warp then forms 8 of the 128 outputs as dot
+// products over 512 (16 elements per lane, butterfly sum).  What bounds it is latency, so everything is requested at
+// once: the warp's 8 KB of weights (64 registers per thread) before the wait for the preceding kernel, which does not write
+// them, then the log-sum-exps and the first eight partial rows of the group, before the merge weights are known.
+// Each block re-reads its head's weights, so this is for one wave of rows (the rule and both sides measured: api.cu).
+constexpr int MP_BATCH = 8;
+__device__ __forceinline__ uint4 ldg_nc(const void* p) {   // volatile: stays where it is written
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ldg_f4(const float* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__global__ void __launch_bounds__(512, 1) merge_project_kernel(const float* __restrict__ o_part,
+                                                               const float* __restrict__ lse_part, int n_chunks, int B,
+                                                               int H, const __nv_bfloat16* __restrict__ w_uv,
+                                                               void* __restrict__ out, float* __restrict__ lse_out,
+                                                               int out_fp32) {
     __shared__ float w_s[MERGE_MAX_CHUNKS];
     __shared__ float red[16];
     __shared__ float4 acc_s[4][128];
     const int h = blockIdx.x, b = blockIdx.y, BH = B * H, bh = b * H + h;
     const int tid = threadIdx.x, grp = tid >> 7, col = tid & 127, warp = tid >> 5, lane = tid & 31;
-    // this warp's 8 weight rows (8 KB, contiguous): requested into L2 now, loaded after the merge
-    const __nv_bfloat16* wrow = w_uv + ((int64_t)h * 128 + warp * 8) * 512 + lane * 16;
+    sm100::pdl_trigger();
+    uint4 wv[8][2];   // this warp's 8 weight rows, 16 consecutive elements per lane and row
     {
-        const char* wl = reinterpret_cast<const char*>(w_uv + ((int64_t)h * 128 + warp * 8) * 512);
-        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(wl + lane * 128));
-        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(wl + 4096 + lane * 128));
+        const __nv_bfloat16* wrow = w_uv + ((int64_t)h * 128 + warp * 8) * 512 + lane * 16;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            wv[r][0] = ldg_nc(wrow + r * 512);
+            wv[r][1] = ldg_nc(wrow + r * 512 + 8);
+        }
     }
-    float m = -INFINITY;
-    for (int c = tid; c < n_chunks; c += 512) {
+    sm100::pdl_wait();
+    const float* src = o_part + (int64_t)bh * 512 + col * 4;
+    const int64_t step = (int64_t)BH * 512;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l0 = tid < n_chunks ? lse_part[(int64_t)tid * BH + bh] : -INFINITY;
+    float4 v[MP_BATCH];
+#pragma unroll
+    for (int i = 0; i < MP_BATCH; ++i) {
+        const int c = grp + 4 * i;
+        v[i] = c < n_chunks ? ldg_f4(src + c * step) : zero;   // (an empty chunk's slot was never written: dropped below)
+    }
+    float m = l0;
+    w_s[tid] = l0;
+    for (int c = tid + 512; c < n_chunks; c += 512) {
         const float l = lse_part[(int64_t)c * BH + bh];
         w_s[c] = l;
         m = fmaxf(m, l);
@@ -177,16 +202,22 @@ __global__ void __launch_bounds__(512) merge_project_kernel(const float* __restr
     __syncthreads();
     z = 0.f;
     for (int i = 0; i < 16; ++i) z += red[i];
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 acc = zero;
     if (m != -INFINITY) {
-        const float* src = o_part + (int64_t)bh * 512 + col * 4;
-#pragma unroll 4
-        for (int c = grp; c < n_chunks; c += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(src + (int64_t)c * BH * 512);
-            const float w = w_s[c];
-            const bool live = w != 0.f;   // an empty chunk's slot was never written
-            acc.x += live ? w * v.x : 0.f; acc.y += live ? w * v.y : 0.f;
-            acc.z += live ? w * v.z : 0.f; acc.w += live ? w * v.w : 0.f;
+        for (int c0 = grp; c0 < n_chunks; c0 += 4 * MP_BATCH) {
+#pragma unroll
+            for (int i = 0; i < MP_BATCH; ++i) {
+                const int c = c0 + 4 * i;
+                const float w = c < n_chunks ? w_s[c] : 0.f;
+                const bool live = w != 0.f;
+                acc.x += live ? w * v[i].x : 0.f; acc.y += live ? w * v[i].y : 0.f;
+                acc.z += live ? w * v[i].z : 0.f; acc.w += live ? w * v[i].w : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < MP_BATCH; ++i) {
+                const int c = c0 + 4 * (MP_BATCH + i);
+                if (c < n_chunks) v[i] = ldg_f4(src + c * step);
+            }
         }
     }
     acc_s[grp][col] = acc;
@@ -196,19 +227,13 @@ __global__ void __launch_bounds__(512) merge_project_kernel(const float* __restr
     float o[16];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        float4 v = acc_s[0][lane * 4 + q];
+        float4 t = acc_s[0][lane * 4 + q];
 #pragma unroll
         for (int g = 1; g < 4; ++g) {
             const float4 u = acc_s[g][lane * 4 + q];
-            v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+            t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
         }
-        o[4 * q] = v.x * inv; o[4 * q + 1] = v.y * inv; o[4 * q + 2] = v.z * inv; o[4 * q + 3] = v.w * inv;
-    }
-    uint4 wv[8][2];   // 16 consecutive elements per lane and row (two 16-byte loads)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        wv[r][0] = *reinterpret_cast<const uint4*>(wrow + r * 512);
-        wv[r][1] = *reinterpret_cast<const uint4*>(wrow + r * 512 + 8);
+        o[4 * q] = t.x * inv; o[4 * q + 1] = t.y * inv; o[4 * q + 2] = t.z * inv; o[4 * q + 3] = t.w * inv;
     }
     float res = 0.f;   // lane r < 8 keeps output row warp * 8 + r
 #pragma unroll
@@ -289,8 +314,7 @@ struct LayoutParams {
     int* status;
 };
 __global__ void __launch_bounds__(256) prepare_layout_kernel(LayoutParams p) {
-    sm100::pdl_trigger();
-    sm100::pdl_wait();
+    sm100::pdl_wait();   // (no early trigger: later kernels read the weights written here before their own wait)
     const int tid = threadIdx.x, blk = blockIdx.x;
     if (blk < p.n_w) {
         __shared__ uint32_t tile[64 * 33];

@@ -58,8 +58,10 @@ expand_sm100_kernel(const __grid_constant__ CUtensorMap tm_c, const __grid_const
     volatile int* abort_flag = &abort_word;
 
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
-    pdl_trigger();
+    // (the trigger comes after the wait: what may start now is behind the kernel that wrote w_uk_t, so that the query
+    // absorption may read that before its own wait)
     pdl_wait();
+    pdl_trigger();
     const int c = blockIdx.x;
     const int u0 = c * p.per + min(c, p.rem), u1 = u0 + p.per + (c < p.rem ? 1 : 0);
 

@@ -295,16 +295,18 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
     const int n0 = blockIdx.x * LAT_BN, m0 = blockIdx.y * BM, h = blockIdx.z;
     pdl_trigger();
-    pdl_wait();
 
     const uint32_t ld = elect_one() ? 1u : 0u;
-    auto issue = [&](int kb) {
+    auto issue_weights = [&](int kb) {
         const int s = kb % LAT_STAGES;
-        uint8_t* dst = smem + s * LAT_STAGE_BYTES;
         mbar_arrive_expect_tx_if(ld, &full[s], LAT_STAGE_BYTES);
-        tma_load_3d_if(ld, dst, &tmA, &full[s], kb * BK, h, m0);
-        tma_load_3d_if(ld, dst + SLAB_BYTES, &tmB, &full[s], kb * BK, n0, h);
+        tma_load_3d_if(ld, smem + s * LAT_STAGE_BYTES + SLAB_BYTES, &tmB, &full[s], kb * BK, n0, h);
     };
+    auto issue_rows = [&](int kb) {
+        const int s = kb % LAT_STAGES;
+        tma_load_3d_if(ld, smem + s * LAT_STAGE_BYTES, &tmA, &full[s], kb * BK, h, m0);
+    };
+    // (the weights are the caller's, unchanged while the handle lives: requested before the wait for the preceding kernel)
     if (warp == 0) {
         if (lane < LAT_STAGES) {
             mbar_init(&full[lane], 1);
@@ -317,8 +319,12 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
         fence_mbar_init();
         __syncwarp();
 #pragma unroll 1
-        for (int kb = 0; kb < LAT_STAGES; ++kb) issue(kb);
+        for (int kb = 0; kb < LAT_STAGES; ++kb) issue_weights(kb);
+        pdl_wait();
+#pragma unroll 1
+        for (int kb = 0; kb < LAT_STAGES; ++kb) issue_rows(kb);
     }
+    pdl_wait();
     if (warp == 1) tmem_alloc(&tmem_holder, LAT_BN);
     tc_fence_before();
     __syncthreads();
@@ -330,7 +336,8 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
         for (int kb = LAT_STAGES; kb < KB; ++kb) {
             if (!mbar_wait_warp(&empty[kb % LAT_STAGES], ((kb / LAT_STAGES) & 1) ^ 1, abort_flag)) break;
             kb_issued = kb + 1;
-            issue(kb);
+            issue_weights(kb);
+            issue_rows(kb);
         }
     } else if (warp == 1) {
         constexpr uint32_t idesc = idesc_bf16(BM, LAT_BN, false, false);

@@ -29,6 +29,8 @@ constexpr int A_BYTES = 128 * 128 * 2;        // 2 slabs [128 rows][64]
 constexpr int W_BYTES = 512 * 128 * 2;        // 4 N-tiles x 2 slabs [128 rows][64]
 constexpr int STAGE_BYTES = 128 * 128 * 2;    // one N = 128 block of the result: 2 slabs [128 rows][64]
 constexpr int SMEM_BYTES = A_BYTES + W_BYTES + 2 * STAGE_BYTES + 1024 + 256;
+constexpr int DIRECT_ROWS = 32;                                                   // up to here rows are stored without staging
+constexpr int SMEM_BYTES_DIRECT = A_BYTES + W_BYTES + 1024 + 256;
 
 struct QAbsorbParams {
     void* q_abs;   // bf16 [B, H, 512]
@@ -52,9 +54,9 @@ q_absorb_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     pdl_trigger();
-    pdl_wait();
     const bool walk = p.walk_ctas > 0;
     if (walk ? (int)blockIdx.x == p.walk_ctas : (int)blockIdx.y == p.H) {   // the ordering block (whole block takes this branch)
+        pdl_wait();
         if (walk || blockIdx.x == 0) {
             block_order_by_length(p.seq_lens, p.B, p.order, reinterpret_cast<unsigned long long*>(smem));
             if (p.desc != nullptr) {
@@ -72,7 +74,7 @@ q_absorb_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     uint8_t* sA = smem;
     uint8_t* sW = smem + A_BYTES;
     uint8_t* sOut = sW + W_BYTES;                                  // 2 staging buffers
-    uint64_t* w_full = reinterpret_cast<uint64_t*>(sOut + 2 * STAGE_BYTES);   // [0..3]: weight block n has landed
+    uint64_t* w_full = reinterpret_cast<uint64_t*>(sOut + (p.B <= DIRECT_ROWS ? 0 : 2 * STAGE_BYTES));   // [0..3]: weight block n has landed
     uint64_t* q_full = w_full + 4;      // query tile t has landed (phase t)
     uint64_t* acc_full = w_full + 5;    // the products of tile t are complete (phase t): accumulators ready, query buffer free
     uint64_t* acc_empty = w_full + 6;   // the epilogue has read the accumulators of tile t (128 arrivals, phase t)
@@ -104,13 +106,16 @@ q_absorb_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         __syncwarp();
         if (n_my > 0) {
             const uint32_t ld = elect_one() ? 1u : 0u;
-            // the first query tile and the weights, all at once
+            // The weights (a copy the handle made when the prefix was prepared) do not depend on the preceding kernel:
+            // they are requested before the wait for it, the first query tile after.
+            issue_weights(ld, head_of(0));
+            pdl_wait();
             mbar_arrive_expect_tx_if(ld, q_full, A_BYTES);
             tma_load_3d_if(ld, sA, &tm_q, q_full, 0, head_of(0), tile_of(0) * 128);
             tma_load_3d_if(ld, sA + 16384, &tm_q, q_full, 64, head_of(0), tile_of(0) * 128);
-            issue_weights(ld, head_of(0));
         }
     }
+    pdl_wait();   // (every thread: nothing below may run beside the preceding kernel)
     if (warp == 1) tmem_alloc(tmem_holder, 512);
     tc_fence_before();
     __syncthreads();
@@ -167,7 +172,7 @@ q_absorb_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             tc_fence_after();
             const int b0 = tile_of(k) * 128;
             const int h = head_of(k);
-            if (p.B <= 32) {
+            if (p.B <= DIRECT_ROWS) {
                 // A handful of requests (one warp's rows at most): the staged store's two block-wide barriers per
                 // result block cost more than they save; every thread writes its own row.
                 __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.q_abs) + ((int64_t)(b0 + row) * p.H + h) * 512;
@@ -288,7 +293,7 @@ cudaError_t launch_q_absorb_sm100(const void* q_nope, const CUtensorMap* tm_w, v
     QAbsorbParams p{q_abs, B, H, n_tiles, splits, walk, status, seq_lens, order, block_table, max_pages, page_size,
                     (with_order && block_table != nullptr) ? reinterpret_cast<int4*>(desc) : nullptr};
     const dim3 grid = walk ? dim3(walk + (with_order ? 1 : 0), 1, 1) : dim3(splits, H + (with_order ? 1 : 0), 1);
-    return launch_pdl(q_absorb_sm100_kernel, grid, dim3(192), SMEM_BYTES, s, tm_q, *tm_w, tm_out, p);
+    return launch_pdl(q_absorb_sm100_kernel, grid, dim3(192), B <= DIRECT_ROWS ? SMEM_BYTES_DIRECT : SMEM_BYTES, s, tm_q, *tm_w, tm_out, p);
 }
 
 }  // namespace tmla
