@@ -67,6 +67,8 @@ struct AbsorbSm100Params {
     __nv_bfloat16* o_lat_direct;   // bf16 [B][H][512] or null
     float* lse_direct;             // [B][H]
     int* status;
+    const char* l2_base;           // read by the kernel behind this one: lane l of warp 2 of CTA i requests bytes
+    uint32_t l2_total, l2_bytes;   // [32 i + l, + 1) * l2_bytes of it into L2 (multiples of 16)
 };
 
 struct Shared {
@@ -138,11 +140,13 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         if (lane == 4) prefetch_tmap(&tm_ckv_pg);
         if (lane == 5) prefetch_tmap(&tm_kpe_pg);
     }
-    pdl_wait();   // the descriptors and Q_A read below are written by the preceding kernel
     // Work items in launch order: the shared-prefix items (chunk fastest, then row group), then the suffix items
     // (chunk fastest, then head group, then request position in longest-first order).
     const int n_shared_items = p.n_shared_chunks * p.shared_groups;
     const bool shared_seg = (int)blockIdx.x < n_shared_items;
+    // The preceding kernel writes Q_A and the descriptors, the caller's kernels the page table and the lengths: the wait.  The
+    // handle's latent rows are older: items over the shared prefix request their first tiles before it (below).
+    if (!shared_seg) pdl_wait();
     int chunk, row0, n_rows, b = 0, len_b = -1, pg0 = -1, pg1 = -1;
     if (shared_seg) {
         chunk = blockIdx.x % p.n_shared_chunks;
@@ -233,21 +237,35 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         for (int sl = 0; sl < 8; ++sl) tma_prefetch_3d_if(ld0, tc, sl * 64, slot, page);
         tma_prefetch_3d_if(ld0, tk, 0, slot, page);
     };
-    if (warp == 0) {
-        if (n_tiles > 0) {
-            mbar_arrive_expect_tx_if(ld0, &sh->q_full, TILE_BYTES);
-#pragma unroll 1
-            for (int s = 0; s < 8; ++s) tma_load_2d_if(ld0, sQ + s * SLAB_BYTES, &tm_qa, &sh->q_full, s * 64, row0);
-            tma_load_2d_if(ld0, sQ + 8 * SLAB_BYTES, &tm_qp, &sh->q_full, 0, row0);
+    if (warp == 0 && n_tiles > 0) {
+        auto first_tiles = [&] {
             for (int j = 0; j < min(n_tiles, STAGES); ++j) {
                 int page, slot;
                 page_of(j, page, slot);
 #pragma unroll 1
                 for (int g = 0; g < 4; ++g) issue_group(j, g, page, slot);
             }
-            for (int j = STAGES; j < 2 * STAGES; ++j) prefetch_tile(j);
+        };
+        if (shared_seg) {
+            first_tiles();
+            pdl_wait();
         }
+        mbar_arrive_expect_tx_if(ld0, &sh->q_full, TILE_BYTES);
+#pragma unroll 1
+        for (int s = 0; s < 8; ++s) tma_load_2d_if(ld0, sQ + s * SLAB_BYTES, &tm_qa, &sh->q_full, s * 64, row0);
+        tma_load_2d_if(ld0, sQ + 8 * SLAB_BYTES, &tm_qp, &sh->q_full, 0, row0);
+        if (!shared_seg) first_tiles();
+        for (int j = STAGES; j < 2 * STAGES; ++j) prefetch_tile(j);
     }
+    if (warp == 2) {
+        // The output projection behind this kernel reads W_UV (131 KB per head, cold after a long step): every CTA requests its
+        // share into L2.  (Absorb-only steps: one request, 128 heads 33.5 -> 32.5 us.  Beside a shared-prefix kernel the host
+        // passes no range: there it costs 0.5 %.)
+        const uint64_t at = ((uint64_t)blockIdx.x * 32u + (uint32_t)lane) * p.l2_bytes;
+        if (at < p.l2_total)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p.l2_base + at), "r"(min(p.l2_bytes, p.l2_total - (uint32_t)at)) : "memory");
+    }
+    if (shared_seg) pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -650,6 +668,9 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
     p.lse_direct = lse_direct;
     const int smem = kAbsorbSmem;
     dim3 grid(a.n_shared_chunks * p.shared_groups + a.n_suffix_chunks * head_groups * a.B, 1, 1);
+    p.l2_base = reinterpret_cast<const char*>(a.w_uv);
+    p.l2_total = a.w_uv ? (uint32_t)a.H * 128u * 512u * 2u : 0u;
+    p.l2_bytes = (p.l2_total / (grid.x * 32u) / 16u + 1u) * 16u;
     const CUtensorMap* sh_c = a.n_shared_chunks > 0 ? tm_ckv_sh : &tm_ckv_pg;
     const CUtensorMap* sh_k = a.n_shared_chunks > 0 ? tm_kpe_sh : &tm_kpe_pg;
     return launch_pdl(absorb_attn_sm100_kernel, grid, dim3(384), smem, s, tm_qa, tm_qp, *sh_c, *sh_k, tm_ckv_pg, tm_kpe_pg, p);

@@ -868,7 +868,7 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
         AbsorbAttn ab{q_abs, q_pe, sh->ckv, sh->kpe, mode == TYPHOON_MLA_MODE_ABSORB ? (int)sh->Ls : 0,
                       ckv_pages, kpe_pages, ckv_token_stride, kpe_token_stride, page_size, num_pages, block_table, max_pages,
                       seq_lens, order, desc, B, H, pl.chunk, pl.n_shared_chunks, pl.n_suffix_chunks, softmax_scale,
-                      o_part_a, lse_part_a, sh->status, cfg.stacked_absorb};
+                      o_part_a, lse_part_a, sh->status, forked ? nullptr : sh->w_uv, cfg.stacked_absorb};
         prof_before(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         e = tc ? launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s)
                : launch_absorb_attn_mma(ab, s);
