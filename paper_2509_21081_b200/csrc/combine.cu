@@ -351,6 +351,44 @@ __global__ void __launch_bounds__(256) prepare_layout_kernel(LayoutParams p) {
     }
 }
 
+// Copies of a step whose tensors live in pinned host memory: up to four arrays, each a whole number of 4-byte words, by
+// 16-byte pieces where both ends allow it.  Bound by the host link; eight independent pieces per thread keep it busy.
+struct HostCopies {
+    const void* src[4];
+    void* dst[4];
+    int64_t bytes[4];
+    int first_block[5];   // blocks [first_block[i], first_block[i + 1]) copy array i
+};
+__global__ void __launch_bounds__(256) host_copy_kernel(HostCopies c) {
+    sm100::pdl_trigger();
+    sm100::pdl_wait();
+    int i = 0;
+    while (i < 3 && (int)blockIdx.x >= c.first_block[i + 1]) ++i;
+    const int n_blk = c.first_block[i + 1] - c.first_block[i];
+    const int64_t t = (int64_t)(blockIdx.x - c.first_block[i]) * 256 + threadIdx.x, step = (int64_t)n_blk * 256;
+    const bool vec = ((reinterpret_cast<uintptr_t>(c.src[i]) | reinterpret_cast<uintptr_t>(c.dst[i])) & 15) == 0;
+    int64_t done = 0;   // bytes copied as 16-byte pieces
+    if (vec) {
+        const int64_t n = c.bytes[i] / 16;
+        const char* src = reinterpret_cast<const char*>(c.src[i]);
+        uint4* dst = reinterpret_cast<uint4*>(c.dst[i]);
+        for (int64_t k0 = t; k0 < n; k0 += 8 * step) {
+            uint4 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k0 + u * step < n)
+                    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w) : "l"(src + (k0 + u * step) * 16) : "memory");
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k0 + u * step < n) dst[k0 + u * step] = v[u];
+        }
+        done = n * 16;
+    }
+    const int64_t words = c.bytes[i] / 4;
+    for (int64_t k = done / 4 + t; k < words; k += step)
+        reinterpret_cast<uint32_t*>(c.dst[i])[k] = *(reinterpret_cast<const volatile uint32_t*>(c.src[i]) + k);
+}
+
 // Longest-first launch order for ragged suffixes: perm[] = request indices sorted by descending
 // suffix length (ties by index, so the order is deterministic).  One block, bitonic sort in
 // shared memory of up to 4096 keys.
@@ -459,6 +497,23 @@ cudaError_t launch_combine(const float* o_naive, const float* lse_naive, int n_n
     if (BH <= 0) return cudaSuccess;
     return launch_pdl(combine_kernel, dim3((BH + 7) / 8), dim3(256), 0, s, o_naive, lse_naive, n_naive, o_abs, lse_abs, BH,
                       out, lse_out, out_fp32 ? 1 : 0);
+}
+
+cudaError_t launch_host_copy(const void* const* src, void* const* dst, const int64_t* bytes, int n, cudaStream_t s) {
+    HostCopies c{};
+    int blocks = 0;
+    for (int i = 0; i < 4; ++i) {
+        c.first_block[i] = blocks;
+        if (i >= n || bytes[i] <= 0) continue;
+        if (bytes[i] % 4) return cudaErrorInvalidValue;
+        c.src[i] = src[i];
+        c.dst[i] = dst[i];
+        c.bytes[i] = bytes[i];
+        blocks += (int)std::min<int64_t>((bytes[i] + 32767) / 32768, 64);   // 32 KB per block and pass
+    }
+    c.first_block[4] = blocks;
+    if (blocks == 0) return cudaSuccess;
+    return launch_pdl(host_copy_kernel, dim3(blocks), dim3(256), 0, s, c);
 }
 
 cudaError_t launch_prepare_layout(const void* w_uk, void* w_uk_t, int H, const void* ckv, int64_t ld_ckv, void* ckv_out, const void* kpe,

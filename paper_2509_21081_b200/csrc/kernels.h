@@ -197,6 +197,9 @@ int noalloc_resolve_scratch_for_current_device();
 int api_cuda_fail(cudaError_t e);
 void api_set_last_launches(int n);
 
+// Copies n <= 4 arrays (multiples of 4 bytes, 4-byte aligned) in one launch; either side may be device-visible host memory.
+cudaError_t launch_host_copy(const void* const* src, void* const* dst, const int64_t* bytes, int n, cudaStream_t s);
+
 // Everything a prepared prefix keeps besides the expansion, in one launch: w_uk [H][128][512] transposed to [H][512][128],
 // the latent rows [L][512] and rope keys [L][64] (row strides ld_*, elements, multiples of 8) copied into contiguous
 // zero-padded [Lp] rows, the 256-byte status block cleared.  L = 0: no rows.

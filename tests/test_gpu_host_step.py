@@ -1,0 +1,41 @@
+"""Steps whose tensors live in host memory: the bits of the device call for pinned, pageable and oddly placed buffers, on
+both sides of the size where the copy engines take over (200 requests x 128 heads: 9.8 MB in, 6.6 MB out)."""
+import pytest
+import torch
+
+from paper_2509_21081_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _place(t, kind):
+    """A host copy of `t`: pinned, pageable, or pinned and starting 2, 4 or 16 bytes behind a 256-byte boundary."""
+    if kind == "pageable":
+        return t.clone()
+    shift = {"pinned": 0, "pinned+2": 2, "pinned+4": 4, "pinned+16": 16}[kind]
+    if shift % t.element_size():
+        shift = 0
+    raw = torch.empty(t.numel() * t.element_size() + 256, dtype=torch.uint8).pin_memory()
+    at = (-raw.data_ptr()) % 256 + shift
+    view = raw[at:at + t.numel() * t.element_size()].view(t.dtype).view(t.shape)
+    return view.copy_(t)
+
+
+@pytest.mark.parametrize("kind", ["pinned", "pageable", "pinned+2", "pinned+4", "pinned+16"])
+@pytest.mark.parametrize("H,B,hi", [(16, 1, 64), (16, 3, 0), (48, 17, 130), (128, 33, 64), (128, 200, 64)])
+def test_host_step(kind, H, B, hi):
+    from paper_2509_21081_b200.decoder import TyphoonMLADecoder
+    inp = I.make_inputs(I.MLAConfig("host", B=B, H=H, Ls=300, suffix_lo=min(hi, 1), suffix_hi=hi, seed=B))
+    pc = I.build_pages(inp)
+    dec = TyphoonMLADecoder(H, inp.ckv_shared.cuda(), inp.kpe_shared.cuda(), inp.w_uk.cuda(), inp.w_uv.cuda(), inp.scale, B,
+                            pc.block_table.shape[1])
+    pages = pc.ckv_pages.cuda(), pc.kpe_pages.cuda()
+    ref = dec.decode(inp.q_nope.cuda(), inp.q_pe.cuda(), *pages, pc.block_table.cuda(), pc.seq_lens.cuda()).cpu()
+    args = [_place(t, kind) for t in (inp.q_nope, inp.q_pe, pc.block_table, pc.seq_lens)]
+    out = _place(torch.zeros(B, H, 128, dtype=torch.bfloat16), kind)
+    for _ in range(2):
+        out.zero_()
+        dec.decode_host(args[0], args[1], *pages, args[2], args[3], out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+    dec.close()
