@@ -8,12 +8,13 @@
 // Bound: the weights' way from L2, 64 bytes per clock and SM at the full tensor rate (a [128 x 128] product of a
 // streamed by a streamed operand needs 128).  Two accumulators (all 512 tensor-memory columns): the epilogue of a unit
 // runs under the next unit's products.
-// Measured (B200, 4864 tokens x 128 heads, both tensors): 152 us = 1.07 PFLOP/s; as two
+// Measured (B200, 4864 tokens x 128 heads, both tensors): 125 us = 1.3 PFLOP/s, 93 us without the stores; as two
 // products with [128 x 128] tiles, every tile's operands read anew and its epilogue exposed: 346 us.
 //
 // Output layouts: K_nope [H, L/64, 2 slabs, 64 tokens, 64 dims], V^T [H, L/64, 128 dims, 64 tokens].  An epilogue thread
-// holds one token: its 64 dims of a K slab are 128 contiguous bytes; for V^T the 32 lanes of a warp write 32
-// consecutive tokens of one dim.
+// holds one token: its 64 dims of a K slab are 128 contiguous bytes, written as four whole 32-byte sectors (with 16-byte
+// stores, half sectors, the kernel took 145 us); for V^T the 32 lanes of a warp write 32 consecutive tokens of two dims
+// (8-byte stores of four tokens instead of two made no difference).
 //
 // Warp roles (384 threads): warp 0 = producer of the weight ring, warp 1 = MMA issuer and TMEM owner, warp 2 = producer of
 // the latent rows, warps 4-7 = epilogue of K, warps 8-11 = epilogue of V (thread = one token).
@@ -163,12 +164,13 @@ expand_sm100_kernel(const __grid_constant__ CUtensorMap tm_c, const __grid_const
                 if (!is_v) {
                     __nv_bfloat16* dst = p.k + out0 + (q >> 1) * 4096 + (r & 63) * 64 + (q & 1) * 32;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        *reinterpret_cast<uint4*>(dst + j * 8) =
-                            make_uint4(pack_bf16(__uint_as_float(t[j * 8]), __uint_as_float(t[j * 8 + 1])),
-                                       pack_bf16(__uint_as_float(t[j * 8 + 2]), __uint_as_float(t[j * 8 + 3])),
-                                       pack_bf16(__uint_as_float(t[j * 8 + 4]), __uint_as_float(t[j * 8 + 5])),
-                                       pack_bf16(__uint_as_float(t[j * 8 + 6]), __uint_as_float(t[j * 8 + 7])));
+                    for (int j = 0; j < 2; ++j) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) w[e] = pack_bf16(__uint_as_float(t[j * 16 + 2 * e]), __uint_as_float(t[j * 16 + 2 * e + 1]));
+                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst + j * 16), "r"(w[0]),
+                                     "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+                    }
                 } else {
                     // two lanes exchange halves, so that a lane writes two consecutive tokens of a dim
                     __nv_bfloat16* dst = p.v_t + out0 + q * 32 * 64 + (r & 62);
