@@ -40,7 +40,7 @@
 // V^T [H, L/64, 128, 64], rope keys [L, 64]; every TMA box is a contiguous 8 or 16 KB.
 //
 // With the expanded cache stored as E4M3 codes (template flag FP8; 64-token tiles, row groups of at most 128
-// requests) four more warps (12-15, 512 threads) widen the copied code blocks into half-precision operand
+// requests) four or eight more warps (12-15 or 12-19) widen the copied code blocks into half-precision operand
 // tiles; see the conversion warps below.
 //
 // Every mbarrier wait has a deadline; on expiry all roles fall through to the common teardown
@@ -62,6 +62,13 @@ constexpr int Q_TILE_BYTES = 128 * 192 * 2;   // 3 slabs [128][64] bf16
 
 constexpr int MAX_STAGES = 4;
 constexpr int MAX_Q_STAGES = 8;
+// 8-bit cache: pairs of conversion warps per tensor (template argument PAIRS; 0 = 16-bit cache).  Two with the 64-row
+// query tile (640 threads, 96 registers: 60 bytes spilled) where a CTA has at least kTwoPairTiles tiles; measured (B200, 64
+// requests, 128 heads, us per step, one / two pairs): 3000 tokens 70.1 / 67.9, 2000: 66.9 / 61.8, 1300: 56.5 / 53.6, 700: 47.9 / 50.9;
+// 32 requests, 16384 tokens 246 / 225.  The 128-row softmax has to keep its 126 registers (at 96 it spills 450 bytes), which
+// leaves room for one.
+constexpr int kTwoPairTiles = 16;
+__host__ __device__ constexpr int naive_threads(int pairs) { return 384 + 128 * pairs; }
 constexpr int kNaiveSmemMax = 227 * 1024;   // opt-in limit set once per device; every launch stays below it
 
 struct NaiveSm100Params {
@@ -129,10 +136,10 @@ struct Segment {
 };
 
 // TOK = tokens per KV tile: 64 (mode Y, B <= 128) or 128 (mode X, B > 128).
-// FP8: the expanded cache is stored as E4M3 codes (see the conversion warpgroup below); 64 query rows per CTA.
+// PAIRS > 0 (FP8): the expanded cache is stored as E4M3 codes (see the conversion warps below).
 // NJ: largest number of prefixes per launch (several: 64-token tiles of the 16-bit cache).
-template <int TOK, bool M64, bool FP8, int NJ>
-__global__ void __launch_bounds__(FP8 ? 512 : 384, 1)
+template <int TOK, bool M64, int PAIRS, int NJ>
+__global__ void __launch_bounds__(naive_threads(PAIRS), 1)
 naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_constant__ CUtensorMap tm_qp,
                         const __grid_constant__ CUtensorMap tm_kn, const __grid_constant__ CUtensorMap tm_kp,
                         const __grid_constant__ CUtensorMap tm_vt, NaiveSm100Params p,
@@ -154,7 +161,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
     TMLA_JOB_MEMBER(const CUtensorMap&, kp_of, tm_kp, tm_kp)
     TMLA_JOB_MEMBER(const CUtensorMap&, vt_of, tm_vt, tm_vt)
 #undef TMLA_JOB_MEMBER
-    constexpr bool MODE_Y = TOK == 64;
+    constexpr bool MODE_Y = TOK == 64, FP8 = PAIRS > 0;
     // 128-token tiles (compute-bound regime): pairs of exponentials computed on the FMA pipe instead of the
     // special-function unit, by position of the pair within a group of eight (bit set = polynomial).  Measured at
     // B = 512: one pair in four is the best mix (-4 % kernel time); one in eight and three in eight gain 1-2 %, every
@@ -821,7 +828,8 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
             g += s.cnt;
         }
     } else if (FP8) {
-        // ---------------- conversion warps (8-bit cache only): warps 12-13 for K and the query tile, warps 14-15 for V.
+        // ---------------- conversion warps (8-bit cache only): warps 12-13 (and 16-17) for K, 14-15 (and 18-19) for V, with two
+        // pairs per tensor each pair every second tile; warps 12-13 also convert the query tile.
         // The expanded K_nope and V of the prefix are stored as E4M3 codes with one power-of-two scale per head.
         // Bulk copies bring 8 KB blocks of codes into staging slots; these warps rewrite each block as the
         // half-precision operand tile the MMAs read (same 128-byte-swizzled layouts as the 16-bit path).  Every E4M3
@@ -830,22 +838,17 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         // per segment, here), its rope part is divided by the scale (a power of two: exact), so the accumulated
         // logits are the true ones divided by it, and the softmax scale is multiplied by it.  V: into the final
         // normalisation.
-        const bool is_v = warp >= 14;
-        const int ct = threadIdx.x - (is_v ? 448 : 384);          // 0..63 within the pair of warps
-        auto pair_sync = [&] {
-            if (is_v) asm volatile("bar.sync 4, 64;\n" ::: "memory");
-            else asm volatile("bar.sync 3, 64;\n" ::: "memory");
-        };
+        const bool is_v = (warp & 2) != 0;
+        const int pair = (warp - 12) >> 2;                        // takes the ring positions = pair (mod PAIRS)
+        const int ct = threadIdx.x & 63;                          // 0..63 within the pair of warps
+        const int pair_bar = 3 + 2 * pair + (is_v ? 1 : 0);       // named barriers 3..6
+        auto pair_sync = [&] { asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory"); };
         // The two warps of a pair must take the same decision before either of them goes to the pair's barrier: one
         // may have seen the abort flag in a wait that the other left through its fast path.
         auto pair_vote_or = [&](bool pred) {
             uint32_t r;
-            if (is_v)
-                asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 4, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
-                             : "=r"(r) : "r"(pred ? 1u : 0u) : "memory");
-            else
-                asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 3, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
-                             : "=r"(r) : "r"(pred ? 1u : 0u) : "memory");
+            asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, %2, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
+                         : "=r"(r) : "r"(pred ? 1u : 0u), "r"(pair_bar) : "memory");
             return r != 0;
         };
         auto widen = [](uint32_t w, uint32_t& lo, uint32_t& hi) {
@@ -907,7 +910,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         bool ok = true;
         for (int g = g_begin; g < g_end && ok; ++seg) {
             const Segment s = segment_at(g);
-            if (!is_v) {
+            if (!is_v && pair == 0) {
                 // query tile (three slabs): nope part to half precision, rope part divided by the K scale
                 ok = !pair_vote_or(!__all_sync(0xffffffffu, mbar_wait(&bar->q_full, seg & 1, abort_flag)));
                 if (!ok) break;
@@ -930,7 +933,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 pair_sync();
                 if (ct == 0) mbar_arrive(&bar->q_conv);
             }
-            for (int e = 0; e < s.cnt && ok; ++e) ok = convert_tile(ring_base + e);
+            for (int e = (pair + ring_base * (PAIRS - 1)) % (FP8 ? PAIRS : 1); e < s.cnt && ok; e += PAIRS) ok = convert_tile(ring_base + e);
             ring_base += s.cnt;
             g += s.cnt;
         }
@@ -1120,11 +1123,13 @@ cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s) {
         return launch_pdl(kernel, dim3(p.n_ranges * p.m_groups), dim3(threads), smem, s, tm_qn, tm_qp, *a.tm_kn, *a.tm_kp, *a.tm_vt, p,
                           NaiveSm100Jobs<1>{});
     };
-    if (fp8) return a.B <= 64 ? launch(naive_attn_sm100_kernel<64, true, true, 1>, 512) : launch(naive_attn_sm100_kernel<64, false, true, 1>, 512);
+    if (fp8 && a.B <= 64)
+        return p.per >= kTwoPairTiles ? launch(naive_attn_sm100_kernel<64, true, 2, 1>, naive_threads(2)) : launch(naive_attn_sm100_kernel<64, true, 1, 1>, naive_threads(1));
+    if (fp8) return launch(naive_attn_sm100_kernel<64, false, 1, 1>, naive_threads(1));
     // (up to 64 rows half-height MMAs: the padding rows 64..127 of the query tile cost tensor-pipe time and power)
-    if (a.B <= 64) return launch(naive_attn_sm100_kernel<64, true, false, 1>, 384);
-    if (a.B <= 128) return launch(naive_attn_sm100_kernel<64, false, false, 1>, 384);
-    return launch(naive_attn_sm100_kernel<128, false, false, 1>, 384);
+    if (a.B <= 64) return launch(naive_attn_sm100_kernel<64, true, 0, 1>, 384);
+    if (a.B <= 128) return launch(naive_attn_sm100_kernel<64, false, 0, 1>, 384);
+    return launch(naive_attn_sm100_kernel<128, false, 0, 1>, 384);
 }
 
 cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaStream_t s) {
@@ -1159,7 +1164,7 @@ cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaSt
     auto launch = [&](auto* kernel) {
         return launch_pdl(kernel, dim3(p.n_ranges), dim3(384), smem, s, j0.tm_qn, j0.tm_qp, j0.tm_kn, j0.tm_kp, j0.tm_vt, p, jobs);
     };
-    return rows <= 64 ? launch(naive_attn_sm100_kernel<64, true, false, kJobs>) : launch(naive_attn_sm100_kernel<64, false, false, kJobs>);
+    return rows <= 64 ? launch(naive_attn_sm100_kernel<64, true, 0, kJobs>) : launch(naive_attn_sm100_kernel<64, false, 0, kJobs>);
 }
 
 cudaError_t set_attrs_naive_sm100() {
@@ -1167,13 +1172,14 @@ cudaError_t set_attrs_naive_sm100() {
     auto opt_in = [&](auto* kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
     };
-    opt_in(naive_attn_sm100_kernel<64, true, false, 1>);
-    opt_in(naive_attn_sm100_kernel<64, false, false, 1>);
-    opt_in(naive_attn_sm100_kernel<128, false, false, 1>);
-    opt_in(naive_attn_sm100_kernel<64, true, true, 1>);
-    opt_in(naive_attn_sm100_kernel<64, false, true, 1>);
-    opt_in(naive_attn_sm100_kernel<64, true, false, kJobs>);
-    opt_in(naive_attn_sm100_kernel<64, false, false, kJobs>);
+    opt_in(naive_attn_sm100_kernel<64, true, 0, 1>);
+    opt_in(naive_attn_sm100_kernel<64, false, 0, 1>);
+    opt_in(naive_attn_sm100_kernel<128, false, 0, 1>);
+    opt_in(naive_attn_sm100_kernel<64, true, 1, 1>);
+    opt_in(naive_attn_sm100_kernel<64, true, 2, 1>);
+    opt_in(naive_attn_sm100_kernel<64, false, 1, 1>);
+    opt_in(naive_attn_sm100_kernel<64, true, 0, kJobs>);
+    opt_in(naive_attn_sm100_kernel<64, false, 0, kJobs>);
     return e;
 }
 

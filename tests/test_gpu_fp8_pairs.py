@@ -1,0 +1,41 @@
+"""8-bit cache, 64-row query tile, one and two pairs of conversion warps per tensor: tile counts per CTA below, at and above
+the rule's 16, odd ones, and ranges that cut heads so that segments start at odd ring positions.  Against attention in 64
+bits over the exported codes; what is left are 16-bit queries and probabilities: the 16-bit path's bars."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("schedule", [0, 1, 2])
+@pytest.mark.parametrize("H,B,Ls", [(128, 5, 15 * 64), (128, 64, 16 * 64), (128, 3, 17 * 64 + 1), (16, 33, 151 * 64 + 1), (48, 64, 3400)])
+def test_conversion_pairs(H, B, Ls, schedule):
+    from paper_2509_21081_b200 import binding as b
+    gen = torch.Generator(device="cuda").manual_seed(Ls)
+
+    def rand(*shape, mul=1.0):
+        return (torch.randn(*shape, generator=gen, device="cuda") * mul).to(torch.bfloat16)
+
+    ckv, kpe = rand(Ls, 512), rand(Ls, 64)
+    sh = b.typhoon_mla_prepare_shared_fp8(b.make_dims(H), ckv, kpe, rand(H, 128, 512, mul=512 ** -0.5), rand(H, 128, 512, mul=512 ** -0.5))
+    qn, qp = rand(B, H, 128), rand(B, H, 64)
+    out = torch.full((B, H, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((B, H), float("nan"), device="cuda")
+    try:
+        b.typhoon_mla_set_naive_schedule(schedule)
+        ws = torch.empty(b.typhoon_mla_workspace_bytes(sh, B, 0, 64), dtype=torch.uint8, device="cuda")
+        b.typhoon_mla_decode(sh, qn, qp, None, None, 64, None, None, 192 ** -0.5, out, ws, mode=b.MODE_NAIVE, lse_out=lse)
+    finally:
+        b.typhoon_mla_set_naive_schedule(0)
+    b.typhoon_mla_check_status(sh)
+    kc, vc, sc = b.typhoon_mla_shared_export_fp8(sh)
+    ref, ref_lse = torch.empty(B, H, 128, dtype=torch.float64, device="cuda"), torch.empty(B, H, dtype=torch.float64, device="cuda")
+    for h in range(H):
+        k = kc[h, :Ls].view(torch.float8_e4m3fn).float().double() * sc[0, h].double()
+        v = vc[h].view(torch.float8_e4m3fn).float().double().permute(0, 2, 1).reshape(-1, 128)[:Ls] * sc[1, h].double()
+        logits = (qn[:, h].double() @ k.T + qp[:, h].double() @ kpe.double().T) * 192 ** -0.5
+        ref_lse[:, h] = torch.logsumexp(logits, -1)
+        ref[:, h] = torch.softmax(logits, -1) @ v
+    assert (torch.linalg.norm(out.double() - ref) / torch.linalg.norm(ref)).item() <= 5e-3
+    assert (lse.double() - ref_lse).abs().max().item() <= 2e-2
+    sh.free()
