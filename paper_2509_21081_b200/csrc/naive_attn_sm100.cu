@@ -839,16 +839,29 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         // logits are the true ones divided by it, and the softmax scale is multiplied by it.  V: into the final
         // normalisation.
         const bool is_v = (warp & 2) != 0;
-        const int pair = (warp - 12) >> 2;                        // takes the ring positions = pair (mod PAIRS)
+        const int pair = PAIRS > 1 ? (warp - 12) >> 2 : 0;        // takes the ring positions = pair (mod PAIRS)
         const int ct = threadIdx.x & 63;                          // 0..63 within the pair of warps
-        const int pair_bar = 3 + 2 * pair + (is_v ? 1 : 0);       // named barriers 3..6
-        auto pair_sync = [&] { asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory"); };
+        // named barriers 3..6 (with one pair per tensor as immediates: the register that holds a number costs the 128-row
+        // instance spills, 2 % of its time)
+        const int pair_bar = 3 + 2 * pair + (is_v ? 1 : 0);
+        auto pair_sync = [&] {
+            if (PAIRS > 1) asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory");
+            else if (is_v) asm volatile("bar.sync 4, 64;\n" ::: "memory");
+            else asm volatile("bar.sync 3, 64;\n" ::: "memory");
+        };
         // The two warps of a pair must take the same decision before either of them goes to the pair's barrier: one
         // may have seen the abort flag in a wait that the other left through its fast path.
         auto pair_vote_or = [&](bool pred) {
             uint32_t r;
-            asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, %2, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
-                         : "=r"(r) : "r"(pred ? 1u : 0u), "r"(pair_bar) : "memory");
+            if (PAIRS > 1)
+                asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, %2, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
+                             : "=r"(r) : "r"(pred ? 1u : 0u), "r"(pair_bar) : "memory");
+            else if (is_v)
+                asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 4, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
+                             : "=r"(r) : "r"(pred ? 1u : 0u) : "memory");
+            else
+                asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 3, 64, q;\nselp.u32 %0, 1, 0, p;\n}\n"
+                             : "=r"(r) : "r"(pred ? 1u : 0u) : "memory");
             return r != 0;
         };
         auto widen = [](uint32_t w, uint32_t& lo, uint32_t& hi) {
