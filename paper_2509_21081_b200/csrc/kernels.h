@@ -174,7 +174,7 @@ cudaError_t launch_order_by_length(const int32_t* seq_lens, int B, int32_t* perm
 cudaError_t launch_merge_latent(const float* o_part, const float* lse_part, int n_chunks, int B, int H,
                                 void* o_lat_bf16, float* lse, cudaStream_t s);
 
-// Absorb-only step with one or two requests: merge of the chunk partials + W_UV projection (Algorithm 1 line 7)
+// Absorb-only step of few (request, head) rows: merge of the chunk partials + W_UV projection (Algorithm 1 line 7)
 // + final rounding in one launch; w_uv is [H, 128, 512] bf16; out bf16 (or fp32) [B, H, 128], lse_out optional.
 cudaError_t launch_merge_project(const float* o_part, const float* lse_part, int n_chunks, int B, int H, const void* w_uv,
                                  void* out, float* lse_out, bool out_fp32, cudaStream_t s);
