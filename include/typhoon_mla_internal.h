@@ -97,6 +97,11 @@ enum {
 int typhoon_mla_profile_begin(int32_t kernel_id, int32_t max_launches);
 int typhoon_mla_profile_end(double* total_ms /* host */, int32_t* launches /* host */);
 
+/* 1 if typhoon_mla_decode_host would let a kernel access [p, p + bytes) of host memory in place: all of it lies in one
+ * pinned allocation or registration and starts on a 4-byte boundary.  0 otherwise (the copy engines move it, and
+ * report what cannot be copied).  Host; reads nothing of the range and launches nothing. */
+int typhoon_mla_host_range_mapped(const void* p /* host */, int64_t bytes);
+
 /* Number of kernels the last decode call of this thread launched. */
 int typhoon_mla_last_launch_count(void);
 

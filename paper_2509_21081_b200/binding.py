@@ -56,6 +56,8 @@ def _load():
                                                   C.POINTER(vp)]
     lib.typhoon_mla_shared_storage_bytes.restype = sz
     lib.typhoon_mla_shared_storage_bytes.argtypes = [C.POINTER(Dims), i64, i32, C.POINTER(sz)]
+    lib.typhoon_mla_host_range_mapped.restype = C.c_int
+    lib.typhoon_mla_host_range_mapped.argtypes = [vp, i64]
     lib.typhoon_mla_release_cached.restype = C.c_int
     lib.typhoon_mla_free.restype = C.c_int
     lib.typhoon_mla_free.argtypes = [vp]

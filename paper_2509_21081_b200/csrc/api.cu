@@ -1177,20 +1177,36 @@ int typhoon_mla_profile_end(double* total_ms, int32_t* launches) {
 // 234 / 250, 128 x 128 (6.3 / 4.2 MB) 299 / 308, 512 x 128 (25 / 17 MB) 1121 / 1088.
 constexpr int64_t kKernelCopyMaxBytes = 8 << 20;
 
-// Address under which kernels may access [p, p + bytes) of host memory, or null (pageable memory, a range that is not
-// all of one pinned allocation, an address 4-byte words cannot start at).
+// Address under which kernels may access [p, p + bytes) of host memory, or null: pageable memory, an address 4-byte words
+// cannot start at, or a range that is not shown to lie inside ONE pinned allocation or registration.  (Two pinned ends
+// prove nothing about the middle: pinned memory is mapped at its own address, so the ends of an array that crosses
+// pageable memory are as far apart on the device as on the host.)  One driver query gives type, device address and range.
 static void* device_view(const void* p, int64_t bytes) {
-    cudaPointerAttributes a{}, z{};
-    if ((reinterpret_cast<uintptr_t>(p) & 3) || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&z, reinterpret_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
-        reinterpret_cast<char*>(z.devicePointer) - reinterpret_cast<char*>(a.devicePointer) != bytes - 1)
-        return nullptr;
-    return a.devicePointer;
+    typedef CUresult (*QueryFn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const QueryFn query = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<QueryFn>(fn);
+    }();
+    const uintptr_t host = reinterpret_cast<uintptr_t>(p);
+    if (!query || host == 0 || (host & 3) || bytes <= 0) return nullptr;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr dev = 0, first = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* into[5] = {&type, &managed, &dev, &first, &size};
+    // (what does not apply to `p` comes back as zero)
+    if (query(5, what, into, (CUdeviceptr)host) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed || dev == 0) return nullptr;
+    if (first == 0 || dev < first || dev - first > size || size - (dev - first) < (size_t)bytes) return nullptr;
+    return reinterpret_cast<void*>(dev);
 }
+
+int typhoon_mla_host_range_mapped(const void* p, int64_t bytes) { return device_view(p, bytes) != nullptr ? 1 : 0; }
 
 size_t typhoon_mla_host_staging_bytes(const typhoon_mla_shared_t* sh, int32_t B, int32_t max_pages) {
     if (!sh || B < 1 || max_pages < 0) return 0;

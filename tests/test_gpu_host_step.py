@@ -39,3 +39,33 @@ def test_host_step(kind, H, B, hi):
         torch.cuda.synchronize()
         assert torch.equal(out, ref)
     dec.close()
+
+
+def test_only_one_pinned_block_is_accessed_in_place():
+    """A range that leaves its pinned block is left to the copy engines, also where its last byte lies in another pinned
+    block.  Only the library's check is asked: nothing is copied or launched."""
+    from paper_2509_21081_b200 import binding as b
+    torch.cuda.init()
+    rt = torch.cuda.cudart()
+    raw = torch.zeros(12 * 4096, dtype=torch.uint8)
+    base = (raw.data_ptr() + 4095) // 4096 * 4096
+    blocks = [(base, 8192), (base + 12288, 8192), (base + 20480, 4096)]      # 4096 pageable bytes between the first two
+    mapped = b._lib.typhoon_mla_host_range_mapped
+    assert not mapped(base, 64)
+    for at, size in blocks:
+        assert int(rt.cudaHostRegister(at, size, 0)) == 0
+    try:
+        assert mapped(base, 8192) and mapped(base + 4, 8188) and mapped(base + 12288, 8192)
+        assert not mapped(base, 8196) and not mapped(base + 4096, 4100)      # runs out of its block
+        assert not mapped(base, 20480) and not mapped(base + 8188, 4104)     # both ends pinned, the middle not
+        assert not mapped(base + 8192, 64) and not mapped(base + 4096, 12288)
+        assert not mapped(base + 2, 64) and not mapped(base, 0) and not mapped(None, 64)
+        assert not mapped(base + 12288, 12288)                               # two neighbouring blocks
+    finally:
+        for at, _ in blocks:
+            assert int(rt.cudaHostUnregister(at)) == 0
+    assert not mapped(base, 64)
+    pinned = torch.empty(1 << 20, dtype=torch.uint8).pin_memory()
+    assert mapped(pinned.data_ptr(), 1 << 20) and mapped(pinned.data_ptr() + 1000, 4096)
+    assert not mapped(raw.data_ptr(), 64)
+    assert not mapped(torch.empty(64, dtype=torch.uint8, device="cuda").data_ptr(), 64)
