@@ -261,7 +261,7 @@ size_t typhoon_mla_host_staging_bytes(const typhoon_mla_shared_t* shared, int32_
  * The same step with the per-step tensors in HOST memory (pinned memory makes
  * the copies asynchronous): q_nope, q_pe, block_table, seq_lens are copied to
  * `staging` (device), the step runs, and `out` (host, bf16 [B, H, 128]) is
- * copied back, all on `stream` (pinned arrays of up to 8 MB per direction by a kernel
+ * copied back, all on `stream` (pinned arrays, with at most 512 KB of inputs, by a kernel
  * that accesses them directly, else by the copy engines).  The caches (ckv_pages, kpe_pages) stay device
  * pointers.  The call returns after enqueueing; synchronise the stream before
  * reading `out`.

@@ -1171,11 +1171,14 @@ int typhoon_mla_profile_end(double* total_ms, int32_t* launches) {
     return st;
 }
 
-// Host arrays of a step up to this many bytes per direction are copied by a kernel of ours, larger ones by the copy engines.
-// Every engine copy costs a hand-over of several microseconds between engine and kernels, the kernel moves 46 GB/s
-// against their 50.  Measured (B200, us per step, kernel / engines): 1 request x 16 heads 30 / 48, 32 x 128 (1.5 MB in, 1 MB out)
-// 234 / 250, 128 x 128 (6.3 / 4.2 MB) 299 / 308, 512 x 128 (25 / 17 MB) 1121 / 1088.
-constexpr int64_t kKernelCopyMaxBytes = 8 << 20;
+// Steps whose inputs in host memory are at most this many bytes are copied, in and out, by a kernel of ours, larger ones by
+// the copy engines.  Every engine copy costs a hand-over of several microseconds between engine and kernels, but engines
+// run beside other streams' kernels for nothing, while copying blocks share the SMs with them.  Measured (B200, us per step,
+// engines / kernel): one step at a time 4 requests x 16 heads 51 / 31, 8 x 128 (0.4 MB in, 0.26 MB out) 80 / 59, 32 x 128
+// (1.6 / 1.0 MB) 249 / 233; twelve streams 42 / 36, 42 / 41, 73 / 83 (64 x 128, 3.1 / 2.1 MB: 98 / 140).  The line lies where
+// no number of streams loses (10 x 128: 84 / 64 and 43 / 42; 14 x 128: 101 / 77 and 46 / 48); one direction by either means
+// loses as well (24 x 64, engines in and kernel out, two streams: 48 / 53).
+constexpr int64_t kKernelCopyMaxBytes = 512 << 10;
 
 // Address under which kernels may access [p, p + bytes) of host memory, or null: pageable memory, an address 4-byte words
 // cannot start at, or a range that is not shown to lie inside ONE pinned allocation or registration.  (Two pinned ends
@@ -1241,9 +1244,11 @@ int typhoon_mla_decode_host(const typhoon_mla_shared_t* sh, const void* q_nope_h
     const int64_t out_bytes = (int64_t)BH * 256;
     tmla::tl_pdl = g_pdl.load();
     const void* src[4] = {};
+    void* out_dev = nullptr;
     bool mapped = in_bytes[0] + in_bytes[1] + in_bytes[2] + in_bytes[3] <= kKernelCopyMaxBytes;
     for (int i = 0; i < 4 && mapped; ++i)
         if (in_bytes[i] > 0) mapped = (src[i] = device_view(in_host[i], in_bytes[i])) != nullptr;
+    if (mapped) mapped = (out_dev = device_view(out_host, out_bytes)) != nullptr;
     cudaError_t e = cudaSuccess;
     if (mapped) {
         e = launch_host_copy(src, in_dev, in_bytes, 4, s);
@@ -1257,8 +1262,7 @@ int typhoon_mla_decode_host(const typhoon_mla_shared_t* sh, const void* q_nope_h
                                      reinterpret_cast<const int32_t*>(d_sl), softmax_scale, mode, d_out, nullptr,
                                      workspace, workspace_bytes, stream);
     if (st_code != TYPHOON_MLA_OK) return st_code;
-    void* out_dev = out_bytes <= kKernelCopyMaxBytes ? device_view(out_host, out_bytes) : nullptr;
-    if (out_dev) {
+    if (mapped) {
         const void* out_src = d_out;
         e = launch_host_copy(&out_src, &out_dev, &out_bytes, 1, s);
     } else {

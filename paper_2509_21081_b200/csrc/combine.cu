@@ -353,14 +353,17 @@ __global__ void __launch_bounds__(256) prepare_layout_kernel(LayoutParams p) {
 
 // Copies of a step whose tensors live in pinned host memory: up to four arrays, each a whole number of 4-byte words, by
 // 16-byte pieces where both ends allow it.  Bound by the host link; eight independent pieces per thread keep it busy.
+// Steps on other streams run beside it.  So a block takes no more registers than the attention kernels leave free on an SM
+// (384 threads with 128 each: 64 for 256 threads), the launch has the highest priority (behind other steps' waiting CTAs
+// a copy took as long as they did), and the kernel behind it is not triggered early, whose CTAs would hold their SMs for
+// the length of the transfer.
 struct HostCopies {
     const void* src[4];
     void* dst[4];
     int64_t bytes[4];
     int first_block[5];   // blocks [first_block[i], first_block[i + 1]) copy array i
 };
-__global__ void __launch_bounds__(256) host_copy_kernel(HostCopies c) {
-    sm100::pdl_trigger();
+__global__ void __launch_bounds__(256, 4) host_copy_kernel(const __grid_constant__ HostCopies c) {
     sm100::pdl_wait();
     int i = 0;
     while (i < 3 && (int)blockIdx.x >= c.first_block[i + 1]) ++i;
@@ -513,7 +516,9 @@ cudaError_t launch_host_copy(const void* const* src, void* const* dst, const int
     }
     c.first_block[4] = blocks;
     if (blocks == 0) return cudaSuccess;
-    return launch_pdl(host_copy_kernel, dim3(blocks), dim3(256), 0, s, c);
+    int lowest = 0, highest = 0;
+    const cudaError_t e = cudaDeviceGetStreamPriorityRange(&lowest, &highest);
+    return e != cudaSuccess ? e : launch_pdl_at(highest, host_copy_kernel, dim3(blocks), dim3(256), 0, s, c);
 }
 
 cudaError_t launch_prepare_layout(const void* w_uk, void* w_uk_t, int H, const void* ckv, int64_t ld_ckv, void* ckv_out, const void* kpe,

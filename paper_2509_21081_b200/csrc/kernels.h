@@ -21,19 +21,30 @@ cudaError_t set_attrs_project_sm100();
 cudaError_t set_attrs_q_absorb_sm100();
 cudaError_t set_attrs_attn_mma();
 cudaError_t set_attrs_gemm_tn();
+// launch_pdl_at: the same at a priority of its own, whatever the stream's
+constexpr int kStreamPriority = 1 << 20;   // ... or at the stream's
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+inline cudaError_t launch_pdl_at(int priority, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = tl_pdl ? 1 : 0;
+    if (priority != kStreamPriority) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePriority;
+        attr[cfg.numAttrs].val.priority = priority;
+        ++cfg.numAttrs;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+    return launch_pdl_at(kStreamPriority, kernel, grid, block, smem, s, static_cast<Args&&>(args)...);
 }
 
 
@@ -198,6 +209,7 @@ int api_cuda_fail(cudaError_t e);
 void api_set_last_launches(int n);
 
 // Copies n <= 4 arrays (multiples of 4 bytes, 4-byte aligned) in one launch; either side may be device-visible host memory.
+// At the device's highest priority.
 cudaError_t launch_host_copy(const void* const* src, void* const* dst, const int64_t* bytes, int n, cudaStream_t s);
 
 // Everything a prepared prefix keeps besides the expansion, in one launch: w_uk [H][128][512] transposed to [H][512][128],

@@ -1,5 +1,5 @@
 """Steps whose tensors live in host memory: the bits of the device call for pinned, pageable and oddly placed buffers, on
-both sides of the size where the copy engines take over (200 requests x 128 heads: 9.8 MB in, 6.6 MB out)."""
+both sides of the size where the copy engines take over (512 KB in: 10 and 11 requests x 128 heads)."""
 import pytest
 import torch
 
@@ -22,7 +22,7 @@ def _place(t, kind):
 
 
 @pytest.mark.parametrize("kind", ["pinned", "pageable", "pinned+2", "pinned+4", "pinned+16"])
-@pytest.mark.parametrize("H,B,hi", [(16, 1, 64), (16, 3, 0), (48, 17, 130), (128, 33, 64), (128, 200, 64)])
+@pytest.mark.parametrize("H,B,hi", [(16, 1, 64), (16, 3, 0), (48, 17, 130), (128, 10, 64), (128, 11, 64), (128, 33, 64), (128, 200, 64)])
 def test_host_step(kind, H, B, hi):
     from paper_2509_21081_b200.decoder import TyphoonMLADecoder
     inp = I.make_inputs(I.MLAConfig("host", B=B, H=H, Ls=300, suffix_lo=min(hi, 1), suffix_hi=hi, seed=B))
@@ -69,3 +69,56 @@ def test_only_one_pinned_block_is_accessed_in_place():
     assert mapped(pinned.data_ptr(), 1 << 20) and mapped(pinned.data_ptr() + 1000, 4096)
     assert not mapped(raw.data_ptr(), 64)
     assert not mapped(torch.empty(64, dtype=torch.uint8, device="cuda").data_ptr(), 64)
+
+
+def _captured(b, dec, args, pages, out):
+    """Node types and (kernel name, priority, threads, registers) of the kernels of one captured host step."""
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def call(fn, *a):
+        err, *res = fn(*a)
+        assert int(err) == 0, (fn, err)
+        return res[0] if len(res) == 1 else res
+
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    stream = torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        dec.decode_host(args[0], args[1], *pages, args[2], args[3], out, mode=b.MODE_ABSORB)
+    g = driver.CUgraph(graph.raw_cuda_graph())
+    _, n = call(driver.cuGraphGetNodes, g, 0)
+    nodes, n = call(driver.cuGraphGetNodes, g, n)
+    types, kernels = [], []
+    for node in nodes[:n]:
+        types.append(call(driver.cuGraphNodeGetType, node))
+        if types[-1] != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        prm = call(driver.cuGraphKernelNodeGetParams, node)
+        func = prm.func if int(prm.func) else call(driver.cuKernelGetFunction, prm.kern)
+        attr = call(driver.cuGraphKernelNodeGetAttribute, node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PRIORITY)
+        regs = call(driver.cuFuncGetAttribute, driver.CUfunction_attribute.CU_FUNC_ATTRIBUTE_NUM_REGS, func)
+        kernels.append((call(driver.cuFuncGetName, func).decode(), attr.priority, prm.blockDimX, regs))
+    highest = call(driver.cuCtxGetStreamPriorityRange)[1]
+    return types, kernels, driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_MEMCPY, highest
+
+
+@pytest.mark.parametrize("B,engines", [(8, False), (10, False), (11, True), (64, True)])
+def test_copies_leave_room_for_other_streams(B, engines):
+    """What keeps several host-fed steps in flight from slowing each other down: engines above 512 KB of inputs, for both
+    directions; below it copying blocks that fit on an SM beside an attention kernel (384 threads with 128 of the 65536
+    registers each) and do not queue behind other streams' CTAs."""
+    from paper_2509_21081_b200 import binding as b
+    from paper_2509_21081_b200.decoder import TyphoonMLADecoder
+    H = 128
+    inp = I.make_inputs(I.MLAConfig("host", B=B, H=H, Ls=200, suffix_lo=64, suffix_hi=64, seed=B))
+    pc = I.build_pages(inp)
+    dec = TyphoonMLADecoder(H, inp.ckv_shared.cuda(), inp.kpe_shared.cuda(), inp.w_uk.cuda(), inp.w_uv.cuda(), inp.scale, B,
+                            pc.block_table.shape[1])
+    pages = pc.ckv_pages.cuda(), pc.kpe_pages.cuda()
+    args = [t.pin_memory() for t in (inp.q_nope, inp.q_pe, pc.block_table, pc.seq_lens)]
+    out = torch.empty(B, H, 128, dtype=torch.bfloat16).pin_memory()
+    types, kernels, memcpy, highest = _captured(b, dec, args, pages, out)
+    copies = [k for k in kernels if "host_copy" in k[0]]
+    assert types.count(memcpy) == (5 if engines else 0) and len(copies) == (0 if engines else 2)
+    for _, priority, threads, regs in copies:
+        assert priority == highest and threads * regs + 384 * 128 <= 65536
+    dec.close()
