@@ -295,6 +295,19 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
     return TYPHOON_MLA_OK;
 }
 
+int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t num_sms, int32_t* columns, int32_t* items,
+                             int32_t* ctas, int32_t* early) {
+    if (B < 1 || n_slots < 0 || num_sms < 0 || !columns || !items || !ctas || !early) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
+    const int n_sm = num_sms > 0 ? num_sms : kDefaultNumSM;
+    const ProjectPlan p = project_sm100_plan(B, num_heads, n_slots, n_sm);
+    *columns = p.columns;
+    *items = p.items;
+    *ctas = p.latency ? p.items : std::min(p.items, n_sm);
+    *early = p.early ? 1 : 0;
+    return TYPHOON_MLA_OK;
+}
+
 int typhoon_mla_cost_model(const typhoon_mla_dims_t* d, int32_t kind, int64_t B, int64_t S_q, int64_t L_s,
                            int64_t L_n, int64_t* macs, int64_t* hbm_words) {
     if (!d || B < 0 || S_q < 1 || L_s < 0 || L_n < 0) return TYPHOON_MLA_ERR_INVALID_ARG;

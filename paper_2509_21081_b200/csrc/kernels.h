@@ -80,6 +80,13 @@ struct CombineEpilogue {
     int H = 0;
     int out_fp32 = 0;                  // `out` is fp32 [B][H][128] (a partial result for a later merge)
 };
+struct ProjectPlan {
+    bool latency;    // latency form, else ring form
+    int columns;     // output columns of an item
+    int items;       // (head, 128 requests, columns): one CTA each (latency form), or shared out over at most n_sm CTAs
+    bool early;      // the kernel behind it may start before this one ends
+};
+ProjectPlan project_sm100_plan(int B, int H, int n_slots, int n_sm);
 cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int n_sm, int* status, cudaStream_t s, const CombineEpilogue& ce);
 
 // Query absorption on tcgen05 (one CTA per head and 128 requests); tm_w from make_q_absorb_tmap.

@@ -47,6 +47,7 @@ struct Shape {
 struct ProjectParams {
     int M, H, n_slots;
     int row_tiles, n_items;
+    int early;             // trigger the kernel behind this one at the start (see project_sm100_plan)
     int* status;
     CombineEpilogue ce;
 };
@@ -95,7 +96,7 @@ project_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     volatile int* abort_flag = &bar->abort_flag;
 
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
-    pdl_trigger();
+    if (p.early) pdl_trigger();
     pdl_wait();
 
     const int n_my = (int)blockIdx.x < p.n_items ? (p.n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
@@ -406,7 +407,6 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
 
 template <int BN>
 cudaError_t launch_columns(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmP, ProjectParams p, int n_sm, cudaStream_t s) {
-    p.n_items = 128 / BN * p.row_tiles * p.H;
     return launch_pdl(project_sm100_kernel<BN>, dim3(std::min(p.n_items, n_sm)), dim3(256), Shape<BN>::SMEM, s, tmA, tmB, tmP, p);
 }
 
@@ -419,14 +419,31 @@ cudaError_t set_attrs_project_sm100() {
     return e;
 }
 
+// (the figures at the top of the file: one slot and one wave favour the latency form; with few (head, row tile) pairs the
+// ring form's 32-column items keep four times as many SMs reading)
+//
+// The early trigger lets the next step's shared-prefix kernel start on the SMs this one leaves.  With more (head, row tile)
+// pairs than SMs, CTAs that take several are all resident at once, and the trigger would come at the very start: that kernel
+// then had every SM before the next step's query absorption, which waits on another stream, and the absorb branch ran
+// behind it instead of beside it.  Measured (B200, us per step, with / without the trigger, 128 heads): 198 requests over 5126
+// tokens 179 / 167, 140 over 5126 170 / 154, 300 over 2000 204 / 199, 1024 over 4096 644 / 629; with fewer pairs it is worth it:
+// 200 requests x 64 heads 87 / 93, and 1 % with two 32-column items per CTA (64 x 64).
+ProjectPlan project_sm100_plan(int B, int H, int n_slots, int n_sm) {
+    const int row_tiles = (B + BM - 1) / BM, tiles = row_tiles * H;
+    ProjectPlan p;
+    p.latency = n_slots <= 1 && tiles <= n_sm;
+    p.columns = p.latency ? LAT_BN : (tiles * 2 <= n_sm ? 32 : 128);
+    p.items = 128 / p.columns * tiles;
+    p.early = tiles <= n_sm;
+    return p;
+}
+
 cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int n_sm, int* status, cudaStream_t s, const CombineEpilogue& ce) {
     if (B <= 0 || ce.H <= 0) return cudaSuccess;
     if (n_sm < 1) n_sm = 1;
-    const int row_tiles = (B + BM - 1) / BM, tiles = row_tiles * ce.H;
-    // (the figures at the top of the file: one slot and one wave favour the latency form; with few (head, row tile)
-    // pairs the ring form's 32-column items keep four times as many SMs reading)
-    const bool latency = ce.n_naive <= 1 && tiles <= n_sm;
-    const int bn = latency ? LAT_BN : (tiles * 2 <= n_sm ? 32 : 128);
+    const ProjectPlan pl = project_sm100_plan(B, ce.H, ce.n_naive, n_sm);
+    const bool latency = pl.latency;
+    const int bn = pl.columns, row_tiles = (B + BM - 1) / BM;
     CUtensorMap tmA, tmB, tmP;
     {
         uint64_t dims[3] = {512, (uint64_t)ce.H, (uint64_t)B};
@@ -442,7 +459,7 @@ cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int
         cudaError_t e = make_tmap_bf16(&tmB, w_uv, 3, dims, strides, box);
         if (e != cudaSuccess) return e;
     }
-    const ProjectParams p{B, ce.H, ce.n_naive, row_tiles, 0, status, ce};
+    const ProjectParams p{B, ce.H, ce.n_naive, row_tiles, pl.items, pl.early, status, ce};
     if (latency) return launch_pdl(project_latency_sm100_kernel, dim3(128 / LAT_BN, row_tiles, ce.H), dim3(192), LAT_SMEM, s, tmA, tmB, p);
     if (ce.n_naive > 0) {   // the partials as rows of 256 16-bit elements (the copies move bytes)
         uint64_t dims[4] = {256, (uint64_t)ce.H, (uint64_t)B, (uint64_t)ce.n_naive};

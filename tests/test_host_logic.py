@@ -176,3 +176,12 @@ def test_naive_plan_invariants(b):
     for bad in ((8, 1, 10, 0), (128, 0, 10, 0), (128, 1, 0, 0), (128, 1, 10, 3)):
         with pytest.raises(Exception):
             b.typhoon_mla_naive_plan(*bad)
+
+
+@pytest.mark.parametrize("H,B,slots,early", [(128, 64, 1, 1), (128, 128, 2, 1), (128, 129, 2, 0), (128, 198, 1, 0), (128, 1024, 1, 0),
+                                             (64, 64, 2, 1), (64, 256, 1, 1), (64, 257, 2, 0), (16, 166, 8, 1), (16, 1024, 3, 1), (16, 2048, 1, 0)])
+def test_projection_lets_the_next_kernel_start_early_up_to_one_head_and_row_tile_per_sm(b, H, B, slots, early):
+    columns, items, ctas, got = b.typhoon_mla_project_plan(H, B, slots)
+    assert items * columns == H * ((B + 127) // 128) * 128
+    assert ctas == items or ctas == 148
+    assert got == early == int(H * ((B + 127) // 128) <= 148)
