@@ -838,11 +838,12 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         // per segment, here), its rope part is divided by the scale (a power of two: exact), so the accumulated
         // logits are the true ones divided by it, and the softmax scale is multiplied by it.  V: into the final
         // normalisation.
-        const bool is_v = (warp & 2) != 0;
+        const bool is_v = PAIRS > 1 ? (warp & 2) != 0 : warp >= 14;   // (one pair: see the barrier numbers below)
         const int pair = PAIRS > 1 ? (warp - 12) >> 2 : 0;        // takes the ring positions = pair (mod PAIRS)
-        const int ct = threadIdx.x & 63;                          // 0..63 within the pair of warps
-        // named barriers 3..6 (with one pair per tensor as immediates: the register that holds a number costs the 128-row
-        // instance spills, 2 % of its time)
+        const int ct = PAIRS > 1 ? threadIdx.x & 63 : threadIdx.x - (is_v ? 448 : 384);   // 0..63 within the pair of warps
+        // Named barriers 3..6.  (With one pair per tensor the 128-row instance sits at the edge of its 128 registers: barrier numbers
+        // as immediates and the role from the warp's rank keep it at 126; either left out spilled 48 bytes: 128 requests
+        // x 128 heads over 700 tokens 67.1 us per step instead of 65.4.)
         const int pair_bar = 3 + 2 * pair + (is_v ? 1 : 0);
         auto pair_sync = [&] {
             if (PAIRS > 1) asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory");

@@ -97,3 +97,36 @@ def assert_parity(gpu_out, ref_out, gpu_lse=None, ref_lse=None, mask=None, what=
             tol = LSE_TOL * max(1.0, float(np.max(np.abs(rl[~inf]))) / 10.0)
             assert e <= tol, f"{what}: lse error {e:.3e} > {tol:.3e}"
     return max_abs, rel
+
+
+def captured_step(step):
+    """Captures `step()` as a CUDA graph: (number of copy nodes, its kernels' launch properties); nothing runs."""
+    import pytest
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def call(fn, *a):
+        err, *res = fn(*a)
+        assert int(err) == 0, (fn, err)
+        return res[0] if len(res) == 1 else res
+
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        step()
+    g = driver.CUgraph(graph.raw_cuda_graph())
+    _, n = call(driver.cuGraphGetNodes, g, 0)
+    nodes, n = call(driver.cuGraphGetNodes, g, n)
+    kind, of_func = driver.CUgraphNodeType, driver.CUfunction_attribute
+    copies, kernels = 0, []
+    for node in nodes[:n]:
+        t = call(driver.cuGraphNodeGetType, node)
+        copies += t == kind.CU_GRAPH_NODE_TYPE_MEMCPY
+        if t != kind.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        prm = call(driver.cuGraphKernelNodeGetParams, node)
+        func = prm.func if int(prm.func) else call(driver.cuKernelGetFunction, prm.kern)
+        attr = call(driver.cuGraphKernelNodeGetAttribute, node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PRIORITY)
+        kernels.append(dict(name=call(driver.cuFuncGetName, func).decode(), priority=attr.priority,
+                            highest_priority=call(driver.cuCtxGetStreamPriorityRange)[1], threads=prm.blockDimX,
+                            registers=call(driver.cuFuncGetAttribute, of_func.CU_FUNC_ATTRIBUTE_NUM_REGS, func),
+                            local_bytes=call(driver.cuFuncGetAttribute, of_func.CU_FUNC_ATTRIBUTE_LOCAL_SIZE_BYTES, func)))
+    return copies, kernels

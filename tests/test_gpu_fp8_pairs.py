@@ -39,3 +39,22 @@ def test_conversion_pairs(H, B, Ls, schedule):
     assert (torch.linalg.norm(out.double() - ref) / torch.linalg.norm(ref)).item() <= 5e-3
     assert (lse.double() - ref_lse).abs().max().item() <= 2e-2
     sh.free()
+
+
+@pytest.mark.parametrize("B,Ls,pairs", [(128, 700, 1), (65, 4096, 1), (300, 700, 1), (64, 700, 1), (64, 4096, 2)])
+def test_one_pair_per_tensor_runs_without_spills(B, Ls, pairs):
+    """The instances with one pair of conversion warps per tensor keep everything in registers (at most 128 with 512
+    threads); only the 640-thread one, at 96, does not."""
+    from paper_2509_21081_b200 import binding as b
+    from tests.gpu_harness import captured_step
+    H = 128
+    z = lambda *shape: torch.zeros(*shape, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    sh = b.typhoon_mla_prepare_shared_fp8(b.make_dims(H), z(Ls, 512), z(Ls, 64), z(H, 128, 512), z(H, 128, 512))
+    qn, qp, out = z(B, H, 128), z(B, H, 64), z(B, H, 128)
+    ws = torch.empty(b.typhoon_mla_workspace_bytes(sh, B, 0, 64), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    _, kernels = captured_step(lambda: b.typhoon_mla_decode(sh, qn, qp, None, None, 64, None, None, 192 ** -0.5, out, ws, mode=b.MODE_NAIVE))
+    naive = [k for k in kernels if "naive_attn_sm100" in k["name"]]
+    assert len(naive) == 1 and naive[0]["threads"] == 384 + 128 * pairs
+    assert pairs == 2 or naive[0]["local_bytes"] == 0
+    sh.free()

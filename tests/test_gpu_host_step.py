@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from paper_2509_21081_b200 import inputs as I
+from tests.gpu_harness import captured_step
 
 pytestmark = pytest.mark.gpu
 
@@ -71,36 +72,6 @@ def test_only_one_pinned_block_is_accessed_in_place():
     assert not mapped(torch.empty(64, dtype=torch.uint8, device="cuda").data_ptr(), 64)
 
 
-def _captured(b, dec, args, pages, out):
-    """Node types and (kernel name, priority, threads, registers) of the kernels of one captured host step."""
-    driver = pytest.importorskip("cuda.bindings.driver")
-
-    def call(fn, *a):
-        err, *res = fn(*a)
-        assert int(err) == 0, (fn, err)
-        return res[0] if len(res) == 1 else res
-
-    graph = torch.cuda.CUDAGraph(keep_graph=True)
-    stream = torch.cuda.Stream()
-    with torch.cuda.graph(graph, stream=stream):
-        dec.decode_host(args[0], args[1], *pages, args[2], args[3], out, mode=b.MODE_ABSORB)
-    g = driver.CUgraph(graph.raw_cuda_graph())
-    _, n = call(driver.cuGraphGetNodes, g, 0)
-    nodes, n = call(driver.cuGraphGetNodes, g, n)
-    types, kernels = [], []
-    for node in nodes[:n]:
-        types.append(call(driver.cuGraphNodeGetType, node))
-        if types[-1] != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
-            continue
-        prm = call(driver.cuGraphKernelNodeGetParams, node)
-        func = prm.func if int(prm.func) else call(driver.cuKernelGetFunction, prm.kern)
-        attr = call(driver.cuGraphKernelNodeGetAttribute, node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PRIORITY)
-        regs = call(driver.cuFuncGetAttribute, driver.CUfunction_attribute.CU_FUNC_ATTRIBUTE_NUM_REGS, func)
-        kernels.append((call(driver.cuFuncGetName, func).decode(), attr.priority, prm.blockDimX, regs))
-    highest = call(driver.cuCtxGetStreamPriorityRange)[1]
-    return types, kernels, driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_MEMCPY, highest
-
-
 @pytest.mark.parametrize("B,engines", [(8, False), (10, False), (11, True), (64, True)])
 def test_copies_leave_room_for_other_streams(B, engines):
     """What keeps several host-fed steps in flight from slowing each other down: engines above 512 KB of inputs, for both
@@ -116,9 +87,9 @@ def test_copies_leave_room_for_other_streams(B, engines):
     pages = pc.ckv_pages.cuda(), pc.kpe_pages.cuda()
     args = [t.pin_memory() for t in (inp.q_nope, inp.q_pe, pc.block_table, pc.seq_lens)]
     out = torch.empty(B, H, 128, dtype=torch.bfloat16).pin_memory()
-    types, kernels, memcpy, highest = _captured(b, dec, args, pages, out)
-    copies = [k for k in kernels if "host_copy" in k[0]]
-    assert types.count(memcpy) == (5 if engines else 0) and len(copies) == (0 if engines else 2)
-    for _, priority, threads, regs in copies:
-        assert priority == highest and threads * regs + 384 * 128 <= 65536
+    n_memcpy, kernels = captured_step(lambda: dec.decode_host(args[0], args[1], *pages, args[2], args[3], out, mode=b.MODE_ABSORB))
+    copies = [k for k in kernels if "host_copy" in k["name"]]
+    assert n_memcpy == (5 if engines else 0) and len(copies) == (0 if engines else 2)
+    for k in copies:
+        assert k["priority"] == k["highest_priority"] and k["threads"] * k["registers"] + 384 * 128 <= 65536
     dec.close()
