@@ -29,12 +29,12 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
                            int32_t* tile_tokens /* host */, int32_t* n_ranges /* host */,
                            int32_t* row_groups /* host */, int32_t* n_slots /* host */);
 
-/* How the tcgen05 output projection (Algorithm 1 lines 7 and 8) of B requests with `n_slots` partial slots is cut on a GPU with
- * `num_sms` multiprocessors (0: 148): items of one head, 128 requests and `columns` output columns, the CTAs they run
+/* How the tcgen05 output projection (Algorithm 1 lines 7 and 8) of B requests with `n_slots` partial slots, of which some
+ * come from a prefix with 8-bit storage (or none), is cut on a GPU with `num_sms` multiprocessors (0: 148): items of one head, 128 requests and `columns` output columns, the CTAs they run
  * on, and whether the kernel behind it may be scheduled early (programmatic launch).  Host, pure.  INVALID_ARG for
  * B < 1, unsupported num_heads or n_slots < 0. */
-int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t num_sms, int32_t* columns /* host */,
-                             int32_t* items /* host */, int32_t* ctas /* host */, int32_t* early /* host */);
+int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t prefix_8bit, int32_t num_sms,
+                             int32_t* columns /* host */, int32_t* items /* host */, int32_t* ctas /* host */, int32_t* early /* host */);
 
 /* Read-only views of what the handle owns (for tests and accounting):
  * k_nope bf16 [H, Ls_padded/64, 2, 64, 64]; v_t bf16 [H, Ls_padded/64, 128, 64]. */

@@ -59,7 +59,7 @@ def _load():
     lib.typhoon_mla_host_range_mapped.restype = C.c_int
     lib.typhoon_mla_host_range_mapped.argtypes = [vp, i64]
     lib.typhoon_mla_project_plan.restype = C.c_int
-    lib.typhoon_mla_project_plan.argtypes = [i32, i32, i32, i32] + [C.POINTER(i32)] * 4
+    lib.typhoon_mla_project_plan.argtypes = [i32, i32, i32, i32, i32] + [C.POINTER(i32)] * 4
     lib.typhoon_mla_release_cached.restype = C.c_int
     lib.typhoon_mla_free.restype = C.c_int
     lib.typhoon_mla_free.argtypes = [vp]
@@ -367,10 +367,10 @@ def typhoon_mla_naive_plan(num_heads: int, B: int, L_s: int, schedule: int = 0, 
     return t.value, r.value, g.value, sl.value
 
 
-def typhoon_mla_project_plan(num_heads: int, B: int, n_slots: int, num_sms: int = 0):
+def typhoon_mla_project_plan(num_heads: int, B: int, n_slots: int, prefix_8bit: bool = False, num_sms: int = 0):
     """(columns, items, ctas, early) of the output projection's work decomposition."""
     out = [C.c_int32() for _ in range(4)]
-    _check(_lib.typhoon_mla_project_plan(num_heads, B, n_slots, num_sms, *[C.byref(x) for x in out]), "typhoon_mla_project_plan")
+    _check(_lib.typhoon_mla_project_plan(num_heads, B, n_slots, int(prefix_8bit), num_sms, *[C.byref(x) for x in out]), "typhoon_mla_project_plan")
     return tuple(x.value for x in out)
 
 

@@ -295,12 +295,12 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
     return TYPHOON_MLA_OK;
 }
 
-int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t num_sms, int32_t* columns, int32_t* items,
-                             int32_t* ctas, int32_t* early) {
+int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t prefix_8bit, int32_t num_sms, int32_t* columns,
+                             int32_t* items, int32_t* ctas, int32_t* early) {
     if (B < 1 || n_slots < 0 || num_sms < 0 || !columns || !items || !ctas || !early) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
     const int n_sm = num_sms > 0 ? num_sms : kDefaultNumSM;
-    const ProjectPlan p = project_sm100_plan(B, num_heads, n_slots, n_sm);
+    const ProjectPlan p = project_sm100_plan(B, num_heads, n_slots, prefix_8bit != 0, n_sm);
     *columns = p.columns;
     *items = p.items;
     *ctas = p.latency ? p.items : std::min(p.items, n_sm);
@@ -922,7 +922,9 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
             ce.o_naive = o_part_n; ce.lse_naive = lse_part_n; ce.n_naive = pl.n_slots_naive;
             ce.lse_abs = lse_a; ce.out = out; ce.lse_out = lse_out; ce.H = H;
             ce.out_fp32 = out_fp32 ? 1 : 0;
-            e = launch_project_sm100(o_lat, sh->w_uv, B, sh->num_sms, sh->status, s, ce);
+            bool any_8bit = false;
+            for (int j = 0; j < n_jobs; ++j) any_8bit = any_8bit || jobs[j].sh->fp8 != 0;
+            e = launch_project_sm100(o_lat, sh->w_uv, B, any_8bit, sh->num_sms, sh->status, s, ce);
             combined = true;
         } else {
             GemmTN g2{o_lat, (int64_t)H * 512, 512, sh->w_uv, 512, 128 * 512, o_abs, (int64_t)H * 128, 128,

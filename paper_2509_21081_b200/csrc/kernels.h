@@ -86,8 +86,10 @@ struct ProjectPlan {
     int items;       // (head, 128 requests, columns): one CTA each (latency form), or shared out over at most n_sm CTAs
     bool early;      // the kernel behind it may start before this one ends
 };
-ProjectPlan project_sm100_plan(int B, int H, int n_slots, int n_sm);
-cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int n_sm, int* status, cudaStream_t s, const CombineEpilogue& ce);
+ProjectPlan project_sm100_plan(int B, int H, int n_slots, bool prefix_8bit, int n_sm);
+// `prefix_8bit`: some partial comes from the kernel of an 8-bit prefix (and the next step's will).
+cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, bool prefix_8bit, int n_sm, int* status, cudaStream_t s,
+                                 const CombineEpilogue& ce);
 
 // Query absorption on tcgen05 (one CTA per head and 128 requests); tm_w from make_q_absorb_tmap.
 cudaError_t make_q_absorb_tmap(const void* w_uk_t, int H, CUtensorMap* tm_w);

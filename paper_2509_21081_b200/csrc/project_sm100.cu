@@ -295,7 +295,7 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
 
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
     const int n0 = blockIdx.x * LAT_BN, m0 = blockIdx.y * BM, h = blockIdx.z;
-    pdl_trigger();
+    if (p.early) pdl_trigger();
 
     const uint32_t ld = elect_one() ? 1u : 0u;
     auto issue_weights = [&](int kb) {
@@ -427,21 +427,25 @@ cudaError_t set_attrs_project_sm100() {
 // then had every SM before the next step's query absorption, which waits on another stream, and the absorb branch ran
 // behind it instead of beside it.  Measured (B200, us per step, with / without the trigger, 128 heads): 198 requests over 5126
 // tokens 179 / 167, 140 over 5126 170 / 154, 300 over 2000 204 / 199, 1024 over 4096 644 / 629; with fewer pairs it is worth it:
-// 200 requests x 64 heads 87 / 93, and 1 % with two 32-column items per CTA (64 x 64).
-ProjectPlan project_sm100_plan(int B, int H, int n_slots, int n_sm) {
+// 200 requests x 64 heads 87 / 93, and 1 % with two 32-column items per CTA (64 x 64).  The kernel of an 8-bit prefix lasts
+// longer and leaves the tensor cores more idle, so that the absorb branch is best beside it from the start: without the
+// trigger 128 requests over 700 tokens 67.4 -> 62.0 us, 64 over 4096 93.5 -> 88.5, 40 over 9000 159 -> 130, 200 x 64 heads over
+// 4096 111 -> 100 (one shape of fifteen lost: 48 over 2000, 60.5 -> 64.2).
+ProjectPlan project_sm100_plan(int B, int H, int n_slots, bool prefix_8bit, int n_sm) {
     const int row_tiles = (B + BM - 1) / BM, tiles = row_tiles * H;
     ProjectPlan p;
     p.latency = n_slots <= 1 && tiles <= n_sm;
     p.columns = p.latency ? LAT_BN : (tiles * 2 <= n_sm ? 32 : 128);
     p.items = 128 / p.columns * tiles;
-    p.early = tiles <= n_sm;
+    p.early = tiles <= n_sm && !prefix_8bit;
     return p;
 }
 
-cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, int n_sm, int* status, cudaStream_t s, const CombineEpilogue& ce) {
+cudaError_t launch_project_sm100(const void* o_lat, const void* w_uv, int B, bool prefix_8bit, int n_sm, int* status, cudaStream_t s,
+                                 const CombineEpilogue& ce) {
     if (B <= 0 || ce.H <= 0) return cudaSuccess;
     if (n_sm < 1) n_sm = 1;
-    const ProjectPlan pl = project_sm100_plan(B, ce.H, ce.n_naive, n_sm);
+    const ProjectPlan pl = project_sm100_plan(B, ce.H, ce.n_naive, prefix_8bit, n_sm);
     const bool latency = pl.latency;
     const int bn = pl.columns, row_tiles = (B + BM - 1) / BM;
     CUtensorMap tmA, tmB, tmP;

@@ -185,3 +185,4 @@ def test_projection_lets_the_next_kernel_start_early_up_to_one_head_and_row_tile
     assert items * columns == H * ((B + 127) // 128) * 128
     assert ctas == items or ctas == 148
     assert got == early == int(H * ((B + 127) // 128) <= 148)
+    assert b.typhoon_mla_project_plan(H, B, slots, prefix_8bit=True) == (columns, items, ctas, 0)
