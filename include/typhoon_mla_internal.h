@@ -29,6 +29,11 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
                            int32_t* tile_tokens /* host */, int32_t* n_ranges /* host */,
                            int32_t* row_groups /* host */, int32_t* n_slots /* host */);
 
+/* The same for a launch over `n` (1..16) prefixes of L_s[i] tokens with at most max_rows (<= 128) query rows each: ranges of
+ * the H * (all prefixes' tiles) tiles and partial slots per prefix.  Host, pure. */
+int typhoon_mla_naive_plan_multi(int32_t num_heads, int32_t max_rows, const int64_t* L_s /* host */, int32_t n, int32_t schedule,
+                                 int32_t num_sms, int32_t* n_ranges /* host */, int32_t* n_slots /* host, n */);
+
 /* How the tcgen05 output projection (Algorithm 1 lines 7 and 8) of B requests with `n_slots` partial slots, of which some
  * come from a prefix with 8-bit storage (or none), is cut on a GPU with `num_sms` multiprocessors (0: 148): items of one head, 128 requests and `columns` output columns, the CTAs they run
  * on, and whether the kernel behind it may be scheduled early (programmatic launch).  Host, pure.  INVALID_ARG for

@@ -58,6 +58,8 @@ def _load():
     lib.typhoon_mla_shared_storage_bytes.argtypes = [C.POINTER(Dims), i64, i32, C.POINTER(sz)]
     lib.typhoon_mla_host_range_mapped.restype = C.c_int
     lib.typhoon_mla_host_range_mapped.argtypes = [vp, i64]
+    lib.typhoon_mla_naive_plan_multi.restype = C.c_int
+    lib.typhoon_mla_naive_plan_multi.argtypes = [i32, i32, C.POINTER(i64), i32, i32, i32, C.POINTER(i32), C.POINTER(i32)]
     lib.typhoon_mla_project_plan.restype = C.c_int
     lib.typhoon_mla_project_plan.argtypes = [i32, i32, i32, i32, i32] + [C.POINTER(i32)] * 4
     lib.typhoon_mla_release_cached.restype = C.c_int
@@ -365,6 +367,15 @@ def typhoon_mla_naive_plan(num_heads: int, B: int, L_s: int, schedule: int = 0, 
     _check(_lib.typhoon_mla_naive_plan(num_heads, B, L_s, schedule, num_sms, C.byref(t), C.byref(r), C.byref(g), C.byref(sl)),
            "typhoon_mla_naive_plan")
     return t.value, r.value, g.value, sl.value
+
+
+def typhoon_mla_naive_plan_multi(num_heads: int, max_rows: int, L_s, schedule: int = 0, num_sms: int = 0):
+    """(n_ranges, slots per prefix) of a shared-prefix launch over several prefixes."""
+    n = len(L_s)
+    r, slots = C.c_int32(), (C.c_int32 * n)()
+    _check(_lib.typhoon_mla_naive_plan_multi(num_heads, max_rows, (C.c_int64 * n)(*L_s), n, schedule, num_sms, C.byref(r), slots),
+           "typhoon_mla_naive_plan_multi")
+    return r.value, list(slots)
 
 
 def typhoon_mla_project_plan(num_heads: int, B: int, n_slots: int, prefix_8bit: bool = False, num_sms: int = 0):

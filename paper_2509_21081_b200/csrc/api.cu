@@ -295,6 +295,16 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
     return TYPHOON_MLA_OK;
 }
 
+int typhoon_mla_naive_plan_multi(int32_t num_heads, int32_t max_rows, const int64_t* L_s, int32_t n, int32_t schedule, int32_t num_sms,
+                                 int32_t* n_ranges, int32_t* n_slots) {
+    if (!L_s || !n_ranges || !n_slots || n < 1 || n > kNaiveJobsPerLaunch || max_rows < 1 || max_rows > 128) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (schedule < 0 || schedule > 2 || num_sms < 0 || num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
+    for (int i = 0; i < n; ++i)
+        if (L_s[i] < 1 || L_s[i] > (int64_t)1 << 24) return TYPHOON_MLA_ERR_INVALID_ARG;
+    naive_sm100_plan_multi(max_rows, num_heads, L_s, n, num_sms > 0 ? num_sms : kDefaultNumSM, schedule, n_ranges, n_slots);
+    return TYPHOON_MLA_OK;
+}
+
 int typhoon_mla_project_plan(int32_t num_heads, int32_t B, int32_t n_slots, int32_t prefix_8bit, int32_t num_sms, int32_t* columns,
                              int32_t* items, int32_t* ctas, int32_t* early) {
     if (B < 1 || n_slots < 0 || num_sms < 0 || !columns || !items || !ctas || !early) return TYPHOON_MLA_ERR_INVALID_ARG;

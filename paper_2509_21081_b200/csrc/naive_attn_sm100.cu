@@ -991,16 +991,20 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // the extra read it causes in the combine).  Stream-K is taken when its modelled cost is lower (by at
 // least 5% in the HBM-bound regime of 64-token tiles).
 //
-// `n` prefixes (their tile counts in `tiles`): the sequence holds all prefixes' tiles of a head, then the next head's;
-// n_slots[i] are the slots of prefix i.
+// `n` prefixes (at most kNaiveJobsPerLaunch, of Ls[i] tokens): the sequence holds all prefixes' tiles of a head, then the next
+// head's; n_slots[i] are the slots of prefix i.  Runs on every call of a step, so the slots of all prefixes come from one walk
+// along the sequence without divisions (16 prefixes x 128 heads: 8 us; a pass per prefix with a division per tile
+// count and range took 159).
 static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
     // (8-bit cache: always 64-token tiles, row groups of 128 requests)
     const bool mode_y = fp8 || B <= 128;
     const int tok = mode_y ? 64 : 128;
     const int m_groups = fp8 ? (B + 127) / 128 : (mode_y ? 1 : (B + 255) / 256);
+    long long tiles[kNaiveJobsPerLaunch];
     int n_tiles = 0;   // per head, over all prefixes
     for (int i = 0; i < n; ++i) {
-        n_tiles += (int)((Ls[i] + tok - 1) / tok);
+        tiles[i] = (Ls[i] + tok - 1) / tok;
+        n_tiles += (int)tiles[i];
         n_slots[i] = 0;
     }
     const long long T = (long long)H * n_tiles;
@@ -1008,20 +1012,26 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
         *n_ranges = 0;
         return;
     }
-    // largest number of partial slots a (prefix, head) needs (over the prefixes, or of prefix `only`) when the T tiles are cut into R ranges (ranges [0, rem) hold per + 1 tiles)
-    auto slots_for = [&](long long R, int only = -1) {
-        const long long per = T / R, rem = T % R, big = rem * (per + 1);
-        auto range_of = [&](long long t) { return t < big ? t / (per + 1) : rem + (t - big) / per; };
-        int seg_max = 1;
-        for (long long h = 0; h < H; ++h) {
-            long long first = h * n_tiles;
+    // Partial slots when the T tiles are cut into R ranges (ranges [0, rem) hold per + 1 tiles): per prefix the largest number
+    // of ranges that meet one of its (head) pieces; the largest of all is returned.
+    auto fill_slots = [&](long long R) {
+        const long long per = T / R, rem = T % R;
+        long long rng = 0, end = per + (rem > 0 ? 1 : 0), t = 0;   // tiles below `end` belong to range rng or an earlier one
+        auto range_of = [&](long long tile) {                     // (of ascending tiles)
+            while (tile >= end) end += per + (++rng < rem ? 1 : 0);
+            return rng;
+        };
+        int most = 1;
+        for (int i = 0; i < n; ++i) n_slots[i] = 0;
+        for (int h = 0; h < H; ++h)
             for (int i = 0; i < n; ++i) {
-                const long long cnt = (Ls[i] + tok - 1) / tok, last = first + cnt - 1;
-                if (cnt > 0 && (only < 0 || only == i)) seg_max = std::max(seg_max, (int)(range_of(last) - range_of(first)) + 1);
-                first += cnt;
+                if (tiles[i] == 0) continue;
+                const long long first = range_of(t);
+                t += tiles[i];
+                n_slots[i] = std::max(n_slots[i], (int)(range_of(t - 1) - first) + 1);
+                most = std::max(most, n_slots[i]);
             }
-        }
-        return seg_max;
+        return most;
     };
     // column split
     const long long base = (long long)H * m_groups;
@@ -1047,7 +1057,7 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     const long long per_stream = (T + r_stream - 1) / r_stream;
     const long long waves_stream = ((long long)r_stream * m_groups + n_sm - 1) / n_sm;
     const double segs_stream = (per_stream >= n_tiles) ? (double)per_stream / n_tiles + 1.0 : 2.0;
-    const double cost_stream = (double)waves_stream * (per_stream + segs_stream * fixed) + slot_cost * (slots_for(r_stream) - 1);
+    const double cost_stream = (double)waves_stream * (per_stream + segs_stream * fixed) + slot_cost * (fill_slots(r_stream) - 1);
     bool stream_k;
     if (schedule == 1) stream_k = false;
     else if (schedule == 2) stream_k = true;
@@ -1061,8 +1071,7 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     }
     const int R = stream_k ? r_stream : H * ns_best;
     *n_ranges = R;
-    for (int i = 0; i < n; ++i)
-        if (Ls[i] > 0) n_slots[i] = slots_for(R, i);   // the kernel uses the same partition
+    if (R != r_stream) fill_slots(R);   // the kernel uses the same partition
 }
 
 void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {

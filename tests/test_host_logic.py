@@ -186,3 +186,47 @@ def test_projection_lets_the_next_kernel_start_early_up_to_one_head_and_row_tile
     assert ctas == items or ctas == 148
     assert got == early == int(H * ((B + 127) // 128) <= 148)
     assert b.typhoon_mla_project_plan(H, B, slots, prefix_8bit=True) == (columns, items, ctas, 0)
+
+
+def _slots(H, tiles, n_ranges):
+    """From the definition: range of every tile, then the ranges each (head, prefix) meets."""
+    T = H * sum(tiles)
+    per, rem = divmod(T, n_ranges)
+    owner = [r for r in range(n_ranges) for _ in range(per + (r < rem))]
+    out, t = [0] * len(tiles), 0
+    for _ in range(H):
+        for i, n in enumerate(tiles):
+            out[i] = max(out[i], owner[t + n - 1] - owner[t] + 1)
+            t += n
+    return out
+
+
+@pytest.mark.parametrize("schedule", [0, 1, 2])
+@pytest.mark.parametrize("H,rows,L_s", [(16, 1, [1]), (128, 64, [4096]), (128, 65, [129]), (16, 128, [64, 1]), (48, 7, [1, 1, 5000]),
+                                        (128, 30, [1000, 900, 1500, 64]), (16, 20, [1 + 97 * i for i in range(16)])])
+def test_partial_slots_of_every_prefix_of_a_launch(b, H, rows, L_s, schedule):
+    tiles = [(n + 63) // 64 for n in L_s]
+    for sms in (1, 20, 148):
+        n_ranges, slots = b.typhoon_mla_naive_plan_multi(H, rows, L_s, schedule, sms)
+        assert 1 <= n_ranges <= H * sum(tiles)
+        assert slots == _slots(H, tiles, n_ranges)
+        if len(L_s) == 1:
+            assert b.typhoon_mla_naive_plan(H, rows, L_s[0], schedule, sms) == (64, n_ranges, 1, slots[0])
+
+
+def test_planning_a_launch_of_many_prefixes_costs_no_more_than_planning_each(b):
+    import time
+    lib = b._lib
+
+    def best(L_s):   # (the call alone: marshalling is done)
+        n = len(L_s)
+        args = (128, 8, (ctypes.c_int64 * n)(*L_s), n, 2, 148, ctypes.byref(ctypes.c_int32()), (ctypes.c_int32 * n)())
+        times = []
+        for _ in range(40):
+            t = time.perf_counter()
+            for _ in range(20):
+                lib.typhoon_mla_naive_plan_multi(*args)
+            times.append((time.perf_counter() - t) / 20)
+        return min(times)
+
+    assert best([256 + 64 * i for i in range(16)]) < 16 * best([736])
