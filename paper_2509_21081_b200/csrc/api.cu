@@ -358,8 +358,13 @@ int typhoon_mla_set_absorb_efficiency(double fraction) {
     return TYPHOON_MLA_OK;
 }
 
-// `naive_time_factor`: how much longer the shared-prefix kernel takes than the model says (1 for the 16-bit cache; the
-// 8-bit cache's kernel is bound by its widening step: measured 1.4-1.7 times the 16-bit kernel's time)
+// `naive_time_factor`: how much longer the shared-prefix part takes than the model says (1 for the 16-bit cache).  The 8-bit
+// cache's kernel is bound by its widening step: 1.13 to 1.4 times the 16-bit kernel's time up to 64 query rows (two conversion
+// pairs from 16 tiles per CTA on), 1.3 to 1.8 up to 128, 1.5 to 2 above.  The forms cross at 24 to 64 rows (16 heads: up to 128).
+// Over 16 and 128 heads, 512 to 32768 tokens, 1 to 512 requests the chosen form is on average 0.35 % behind the better one
+// at 1.25 and 1.3, 0.5 % at 1.5 and 1.2, 0.8 % at 1 and 1.6 (128 heads, 24 requests over 32768 tokens 326 us latent against 417;
+// 48 over 512 tokens 49.9 against 45.7).
+constexpr double kNaiveTime8Bit = 1.3;
 static int choose_mode_impl(const typhoon_mla_dims_t* dims, int64_t Ls, int32_t B, int64_t total_suffix_tokens,
                             double naive_time_factor) {
     if (!dims || B < 1 || Ls <= 0) return TYPHOON_MLA_MODE_ABSORB;
@@ -390,7 +395,7 @@ int typhoon_mla_choose_mode_for(const typhoon_mla_dims_t* dims, int64_t Ls, int3
 
 int typhoon_mla_choose_mode(const typhoon_mla_shared_t* sh, int32_t B, int64_t total_suffix_tokens) {
     if (!sh) return TYPHOON_MLA_MODE_ABSORB;
-    return choose_mode_impl(&sh->dims, sh->Ls, B, total_suffix_tokens, sh->fp8 ? 1.5 : 1.0);
+    return choose_mode_impl(&sh->dims, sh->Ls, B, total_suffix_tokens, sh->fp8 ? kNaiveTime8Bit : 1.0);
 }
 
 int typhoon_mla_free(typhoon_mla_shared_t* sh) {

@@ -208,3 +208,14 @@ def test_random_shapes(seed):
         G.assert_parity(out, ref, lse, ref_lse, what=f"fp8 random {seed}: B={B} H={H} Ls={Ls} hi={hi} ps={page_size}")
     finally:
         b.typhoon_mla_set_naive_schedule(0)
+
+
+@pytest.mark.parametrize("H,Ls,B,hybrid", [(128, 512, 48, True), (128, 512, 32, False), (128, 2048, 32, True), (128, 8192, 32, True),
+                                           (128, 8192, 24, False), (128, 32768, 24, False), (16, 32768, 24, False), (16, 32768, 48, True)])
+def test_formulation_chosen_for_an_8bit_prefix(H, Ls, B, hybrid):
+    """The faster of the two by measurement, at sizes around where they cross (the others differ by 5 % or less)."""
+    from paper_2509_21081_b200 import binding as b
+    z = lambda *shape: torch.zeros(*shape, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    sh = b.typhoon_mla_prepare_shared_fp8(b.make_dims(H), z(Ls, 512), z(Ls, 64), z(H, 128, 512), z(H, 128, 512))
+    assert b.typhoon_mla_choose_mode(sh, B) == (b.MODE_HYBRID if hybrid else b.MODE_ABSORB)
+    sh.free()
