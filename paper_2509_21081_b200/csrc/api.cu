@@ -866,13 +866,16 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                     // ... but only if the shared-prefix kernel lasts about as long as the walk (measured: about 5 us per head
                     // for a walking CTA, 0.7 us per 64-token tile for a shared-prefix CTA; B = 64, H = 128: the walk wins
                     // from 3072 prefix tokens on and loses at 2048); under a short shared-prefix kernel one CTA per head,
-                    // which spreads over the whole GPU as soon as that kernel ends, is faster.
+                    // which spreads over the whole GPU as soon as that kernel ends, is faster.  A 64-token tile of the 8-bit
+                    // cache takes 1.0 us, with more than 64 rows 1.3 (H = 128, us per step, one CTA per head / walk: 64
+                    // requests over 1900 tokens 65.4 / 53.2, over 2400 69.7 / 59.6, 100 over 1500 74.3 / 65.5).
                     const int64_t tok = jobs[0].rows <= 128 || jobs[0].sh->fp8 ? 64 : 128;
                     int64_t head_tiles = 0;
                     for (int j = 0; j < n_jobs; ++j) head_tiles += (jobs[j].sh->Ls + tok - 1) / tok;
                     const int64_t tiles_per_cta = (head_tiles * H + jobs[0].n_ranges - 1) / jobs[0].n_ranges;
                     const int heads_per_cta = (H + free_sms - 1) / free_sms;
-                    if ((double)tiles_per_cta * (tok == 64 ? 0.7 : 3.0) >= 4.0 * heads_per_cta) walk_ctas = free_sms;
+                    const double tile_us = jobs[0].sh->fp8 ? (jobs[0].rows <= 64 ? 1.0 : 1.3) : tok == 64 ? 0.7 : 3.0;
+                    if ((double)tiles_per_cta * tile_us >= 4.0 * heads_per_cta) walk_ctas = free_sms;
                 }
             }
             e = launch_q_absorb_sm100(q_nope, &sh->tm_wuk_t, q_abs, B, H, sh->num_sms, walk_ctas, sh->status, order ? seq_lens : nullptr, order,

@@ -126,7 +126,7 @@ def captured_step(step):
         func = prm.func if int(prm.func) else call(driver.cuKernelGetFunction, prm.kern)
         attr = call(driver.cuGraphKernelNodeGetAttribute, node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PRIORITY)
         kernels.append(dict(name=call(driver.cuFuncGetName, func).decode(), priority=attr.priority,
-                            highest_priority=call(driver.cuCtxGetStreamPriorityRange)[1], threads=prm.blockDimX,
+                            highest_priority=call(driver.cuCtxGetStreamPriorityRange)[1], threads=prm.blockDimX, grid=(prm.gridDimX, prm.gridDimY),
                             registers=call(driver.cuFuncGetAttribute, of_func.CU_FUNC_ATTRIBUTE_NUM_REGS, func),
                             local_bytes=call(driver.cuFuncGetAttribute, of_func.CU_FUNC_ATTRIBUTE_LOCAL_SIZE_BYTES, func)))
     return copies, kernels

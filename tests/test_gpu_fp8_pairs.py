@@ -58,3 +58,39 @@ def test_one_pair_per_tensor_runs_without_spills(B, Ls, pairs):
     assert len(naive) == 1 and naive[0]["threads"] == 384 + 128 * pairs
     assert pairs == 2 or naive[0]["local_bytes"] == 0
     sh.free()
+
+
+@pytest.mark.parametrize("B,Ls,walks", [(64, 1600, False), (64, 1900, True), (40, 2500, True), (65, 1200, False), (100, 1500, True)])
+def test_absorb_branch_beside_an_8bit_prefix(B, Ls, walks):
+    """Beside a shared-prefix kernel on 128 of 148 SMs that lasts long enough the query absorption walks through the heads on
+    the other 20 (the 8-bit kernel's tiles are slower than the 16-bit one's); with one stream it takes a CTA per head.
+    Same products either way: same bits."""
+    from paper_2509_21081_b200 import binding as b
+    from tests.gpu_harness import captured_step
+    H, pages = 128, 2
+    gen = torch.Generator(device="cuda").manual_seed(B)
+
+    def rand(*shape, mul=1.0):
+        return (torch.randn(*shape, generator=gen, device="cuda") * mul).to(torch.bfloat16)
+
+    sh = b.typhoon_mla_prepare_shared_fp8(b.make_dims(H), rand(Ls, 512), rand(Ls, 64), rand(H, 128, 512, mul=0.044),
+                                          rand(H, 128, 512, mul=0.044))
+    table = torch.arange(B * pages, dtype=torch.int32, device="cuda").view(B, pages)
+    lens = (torch.arange(B, dtype=torch.int32, device="cuda") * 37) % (64 * pages + 1)
+    args = (rand(B, H, 128), rand(B, H, 64), rand(B * pages, 64, 512), rand(B * pages, 64, 64), 64, table, lens, 192 ** -0.5)
+    ws = torch.empty(b.typhoon_mla_workspace_bytes(sh, B, pages, 64), dtype=torch.uint8, device="cuda")
+    got = {}
+    for overlap in (True, False):
+        out = torch.full((B, H, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        try:
+            b.typhoon_mla_set_overlap(overlap)
+            b.typhoon_mla_decode(sh, *args, out, ws, mode=b.MODE_HYBRID)
+            b.typhoon_mla_check_status(sh)
+            got[overlap] = out
+            _, kernels = captured_step(lambda: b.typhoon_mla_decode(sh, *args, out, ws, mode=b.MODE_HYBRID))
+        finally:
+            b.typhoon_mla_set_overlap(True)
+        grid = [k["grid"] for k in kernels if "q_absorb" in k["name"]]
+        assert grid == [(21, 1) if walks and overlap else (1, 129)]   # (with the block that orders the requests)
+    assert torch.isfinite(got[True]).all() and torch.equal(got[True], got[False])
+    sh.free()
