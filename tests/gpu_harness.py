@@ -54,6 +54,40 @@ def run_oracle_fp8(inp, pairs=None, drop_suffix=False):
                                    f(inp.w_uk), f(inp.w_uv), inp.scale, pairs=pairs)
 
 
+def reference64(inp):
+    """The step from its definition in 64 bits on the GPU (one softmax over shared prefix and own tokens): numpy (out, lse)."""
+    B, H = inp.cfg.B, inp.cfg.H
+    qn, qp, w_uk, w_uv, ckv, kpe = (x.cuda().double() for x in (inp.q_nope, inp.q_pe, inp.w_uk, inp.w_uv, inp.ckv_shared,
+                                                                inp.kpe_shared))
+    lse = torch.full((B, H), -math.inf, dtype=torch.float64, device="cuda")
+    out = torch.zeros(B, H, 128, dtype=torch.float64, device="cuda")
+
+    def merge(where, l, o):
+        old = lse[where]
+        new = torch.logaddexp(old, l)
+        out[where] = out[where] * torch.exp(old - new)[..., None] + o * torch.exp(l - new)[..., None]
+        lse[where] = new
+
+    if ckv.shape[0]:
+        for h in range(H):
+            logits = (qn[:, h] @ (ckv @ w_uk[h].T).T + qp[:, h] @ kpe.T) * inp.scale
+            merge((slice(None), h), torch.logsumexp(logits, -1), torch.softmax(logits, -1) @ (ckv @ w_uv[h].T))
+    q_lat = torch.einsum("bhd,hdc->bhc", qn, w_uk)
+    for r in range(B):
+        c, k = inp.ckv_suffix[r].cuda().double(), inp.kpe_suffix[r].cuda().double()
+        if c.shape[0]:
+            logits = (q_lat[r] @ c.T + qp[r] @ k.T) * inp.scale
+            merge(r, torch.logsumexp(logits, -1), torch.einsum("hc,hdc->hd", torch.softmax(logits, -1) @ c, w_uv))
+    return out.cpu().numpy(), lse.cpu().numpy()
+
+
+def worst_row(got, ref):
+    """Largest relative error (2-norm) of a (request, head) row: an error in one row cannot hide in the whole tensor's norm
+    (385 x 128 rows, one of them wrong: 4.5e-3)."""
+    got, ref = got.reshape(-1, got.shape[-1]).double(), ref.reshape(-1, ref.shape[-1]).double()
+    return (torch.linalg.norm(got - ref, dim=1) / torch.linalg.norm(ref, dim=1)).max().item()
+
+
 def errors(gpu, ref, mask=None):
     if mask is not None:
         gpu, ref = gpu[mask], ref[mask]

@@ -1,12 +1,13 @@
 """The projection + combine kernel in its forms, at the edges of its rule: one wave of (head, 128-row tile) pairs and one
 more, half a wave (32-column items), no slot, one slot and several slots, row tiles that end in one row.
 
-Reference: the same step with the suffix part absorbed by the warp-MMA kernels (an implementation that shares no kernel
-with it).  Both sides round probabilities, latent output and result to 16 bits: the bars of two runs of the library."""
+Reference: the definition in 64 bits, with the parity bars (per row, so that no column item or slot chunk of one row can hide);
+the warp-MMA kernels, an implementation that shares no kernel with these, are held against it as well."""
 import pytest
 import torch
 
 from paper_2509_21081_b200 import inputs as I
+from tests import gpu_harness as G
 
 pytestmark = pytest.mark.gpu
 
@@ -44,12 +45,11 @@ def test_projection_forms(H, B, Ls, hi, schedule, fp32):
         b.typhoon_mla_set_naive_schedule(schedule)
         got = {m: step(m) for m in (b.MODE_HYBRID, b.MODE_ABSORB)}
         b.typhoon_mla_set_kernel_path(b.PATH_WARP_MMA)
-        ref, ref_lse = step(b.MODE_HYBRID)
+        got["warp MMA"] = step(b.MODE_HYBRID)
     finally:
         b.typhoon_mla_set_kernel_path(b.PATH_TCGEN05)
         b.typhoon_mla_set_naive_schedule(0)
-    for out, lse in got.values():
-        assert torch.isfinite(out).all()
-        assert (torch.linalg.norm(out - ref) / torch.linalg.norm(ref)).item() <= 5e-3
-        assert (lse - ref_lse).abs().max().item() <= 2e-2
+    ref, ref_lse = G.reference64(inp)
+    for what, (out, lse) in got.items():
+        G.assert_parity(out.double().cpu().numpy(), ref, lse.double().cpu().numpy(), ref_lse, what=str(what))
     sh.free()

@@ -7,6 +7,8 @@ are those of two runs of the library (relative Frobenius 5e-3, log-sum-exp 2e-2)
 import pytest
 import torch
 
+from tests.gpu_harness import worst_row
+
 pytestmark = pytest.mark.gpu
 
 CASES = {
@@ -60,6 +62,7 @@ def test_prefixes_that_share_a_launch(case, schedule):
         for a, c, la, lc in ((flat[r0:r1], o1, flat_lse[r0:r1], l1), (got[r0:r1], o, got_lse[r0:r1], l)):
             assert torch.isfinite(a).all()
             assert (torch.linalg.norm(a - c) / torch.linalg.norm(c)).item() <= 5e-3
+            assert worst_row(a, c) <= 2e-2                 # (the row bar of the parity tests)
             assert (la - lc).abs().max().item() <= 2e-2
     for h in parts + [root]:
         h.free()
