@@ -71,7 +71,7 @@ int typhoon_mla_set_overlap(int32_t enable);
 
 /* The kernels of a step are launched with the programmatic-stream-serialization attribute (default):
  * a kernel may be scheduled while its predecessor in the stream is still running and waits, before its
- * first access to global memory, until that predecessor has completed.  0 gives ordinary stream-ordered
+ * first access to global memory that a step may have written, until that predecessor has completed.  0 gives ordinary stream-ordered
  * launches. */
 int typhoon_mla_set_programmatic_launch(int32_t enable);
 

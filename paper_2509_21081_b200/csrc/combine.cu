@@ -314,7 +314,7 @@ struct LayoutParams {
     int* status;
 };
 __global__ void __launch_bounds__(256) prepare_layout_kernel(LayoutParams p) {
-    sm100::pdl_wait();   // (no early trigger: later kernels read the weights written here before their own wait)
+    sm100::pdl_wait();   // (must not trigger early: later kernels read what is written here before their own wait, see kernels.h)
     const int tid = threadIdx.x, blk = blockIdx.x;
     if (blk < p.n_w) {
         __shared__ uint32_t tile[64 * 33];

@@ -59,8 +59,8 @@ expand_sm100_kernel(const __grid_constant__ CUtensorMap tm_c, const __grid_const
     volatile int* abort_flag = &abort_word;
 
     const int warp = warp_index_uniform(), lane = threadIdx.x & 31;
-    // (the trigger comes after the wait: what may start now is behind the kernel that wrote w_uk_t, so that the query
-    // absorption may read that before its own wait)
+    // (the trigger must stay behind the wait: what may start now is behind the kernel that wrote w_uk_t and the latent rows, so
+    // that a step may read them before its own wait, see kernels.h)
     pdl_wait();
     pdl_trigger();
     const int c = blockIdx.x;

@@ -6,16 +6,24 @@
 
 namespace tmla {
 
-// Launch with the programmatic-stream-serialization attribute when enabled (see sm100::pdl_wait): the
-// kernel must call pdl_wait() before its first access to global memory.  The switch is per thread: an API
-// call copies its snapshot of the process-wide setting here before it launches anything.
+// Launch with the programmatic-stream-serialization attribute when enabled (see sm100::pdl_wait).  The switch is per
+// thread: an API call copies its snapshot of the process-wide setting here before it launches anything.
+//
+// What a kernel launched this way may do before its pdl_wait(), which every thread of it executes:
+//  - write nothing to global memory;
+//  - read only what is older than any step: the handle's copies (w_uk_t: query absorption; ckv, kpe: the absorb kernel's
+//    shared-prefix items) and the borrowed w_uv, which the caller keeps unchanged (projection, merge + projection).
+// A kernel may be scheduled as soon as all CTAs of its predecessor have triggered, and then its successor in turn, so the
+// second point holds only because no kernel that prepares a prefix lets a later one start before those copies are
+// complete: prepare_layout_kernel, which writes them, never calls pdl_trigger(); expand_sm100_kernel behind it calls it
+// after its own wait; a prefix of no tokens has a memset there instead.  A trigger moved forward in either would let a step
+// read unwritten weights.
 extern thread_local bool tl_pdl;
 
 // Opt-in shared-memory sizes of the kernels, set once per device (by typhoon_mla_prepare_shared, with that
 // device current) instead of before every launch.
 cudaError_t set_attrs_naive_sm100();
 cudaError_t set_attrs_absorb_sm100();
-cudaError_t set_attrs_stacked_sm100();
 cudaError_t set_attrs_expand_sm100();
 cudaError_t set_attrs_project_sm100();
 cudaError_t set_attrs_q_absorb_sm100();

@@ -508,7 +508,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         bool ok = true;
         for (int g = g_begin; g < g_end && ok;) {
             const Segment s = segment_at(g);
-                const int tile_row0 = s.row0 + (MODE_Y ? 0 : i * 128);
+            const int tile_row0 = s.row0 + (MODE_Y ? 0 : i * 128);
             const int b = lane_has_row ? tile_row0 + row : 0x3fffffff;
             const int nt = i == 0 ? s.n_str0 : s.n_str1;
             const bool warp_has_rows = tile_row0 + (M64 ? (warp & 3) * 16 : lg) < rows_of(s.job);   // warp-uniform: the warp's first row is a real request

@@ -16,8 +16,7 @@
 //
 // Latency form (at most one slot, one wave): CTA = (head, 128 requests, 64 columns), two CTAs per SM, the first
 // operand tiles requested before the CTA's set-up is complete, the one slot read from global memory meanwhile.
-// 64 requests, 128 heads: step 82.9 -> 78.8 us where the ring form gives 81.5 (8 requests without slots: 71.4 -> 69.6,
-// ring form 72.2).
+// 64 requests, 128 heads, 4096 tokens: step 84.1 -> 82.1 us; 8 requests without slots: 71.4 -> 69.6 (ring form 72.2).
 #include <algorithm>
 #include <cstddef>
 
@@ -307,7 +306,7 @@ project_latency_sm100_kernel(const __grid_constant__ CUtensorMap tmA, const __gr
         const int s = kb % LAT_STAGES;
         tma_load_3d_if(ld, smem + s * LAT_STAGE_BYTES, &tmA, &full[s], kb * BK, h, m0);
     };
-    // (the weights are the caller's, unchanged while the handle lives: requested before the wait for the preceding kernel)
+    // (the weights are the caller's, unchanged while the handle lives: requested before the wait, see kernels.h)
     if (warp == 0) {
         if (lane < LAT_STAGES) {
             mbar_init(&full[lane], 1);

@@ -107,7 +107,7 @@ q_absorb_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if (n_my > 0) {
             const uint32_t ld = elect_one() ? 1u : 0u;
             // The weights (a copy the handle made when the prefix was prepared) do not depend on the preceding kernel:
-            // they are requested before the wait for it, the first query tile after.
+            // they are requested before the wait for it (see kernels.h), the first query tile after.
             issue_weights(ld, head_of(0));
             pdl_wait();
             mbar_arrive_expect_tx_if(ld, q_full, A_BYTES);
