@@ -157,32 +157,32 @@ int naive_splits(int B, int H, int64_t Ls, int n_sm) {
 
 void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int* chunk, int* n_sh,
                    int* n_sf) {
-    const int units = B * ((H + 63) / 64);
-    // CTAs per shared-prefix chunk: 64-row groups of the stacked [B * H] query matrix, or of each request
-    const int units_sh = (tc && stacked) ? (int)(((int64_t)B * H + 63) / 64) : units;
+    const bool pair = tc && absorb_uses_pairs(H);
+    const int row_tile = pair ? 128 : 64;
+    const int units = B * ((H + row_tile - 1) / row_tile);
+    // work items per shared-prefix chunk: row groups of the stacked [B * H] query matrix, or of each request
+    const int units_sh = (tc && stacked) ? (int)(((int64_t)B * H + row_tile - 1) / row_tile) : units;
     const int64_t longest = std::max<int64_t>(std::max(Ls_absorb, cap_suffix), 1);
     int64_t c;
     if (tc) {
-        // One CTA per SM: minimise waves x (tiles per chunk + fixed cost in tile units) over the number of
-        // chunks the longest segment is cut into.
-        const double fixed = 3.0;
+        // One CTA (pair) per SM (pair of SMs): minimise waves x (tiles per chunk + fixed cost in tile units) over the number of
+        // chunks the longest segment is cut into.  A split segment writes and re-reads fp32 partials, 2 KB per row both ways.
+        const int tile = pair ? 128 : 64, slots = pair ? n_sm / 2 : n_sm;
+        const double fixed = pair ? 4.0 : 3.0, split = pair ? 3.0 : 3.5;
         double best_cost = 1e30;
-        c = round_up(longest, 64);
+        c = round_up(longest, tile);
         for (int parts = 1; parts <= 512; ++parts) {
-            const int64_t ch = round_up((longest + parts - 1) / parts, 64);
+            const int64_t ch = round_up((longest + parts - 1) / parts, tile);
             const int64_t per_req = (Ls_absorb + ch - 1) / ch + (cap_suffix + ch - 1) / ch;
-            const int64_t ctas = (int64_t)units_sh * ((Ls_absorb + ch - 1) / ch) + (int64_t)units * ((cap_suffix + ch - 1) / ch);
+            const int64_t items = (int64_t)units_sh * ((Ls_absorb + ch - 1) / ch) + (int64_t)units * ((cap_suffix + ch - 1) / ch);
             if (per_req > kMaxAbsorbChunks) continue;   // limit of the merge kernel
-            const int64_t waves = (ctas + n_sm - 1) / n_sm;
-            // a split segment writes and re-reads fp32 partials (64 heads x 2 KB, both ways): about 3.5 tiles
-            // worth of traffic per chunk
-            const double split_cost = (per_req > 1) ? 3.5 : 0.0;
-            const double cost = (double)waves * ((double)ch / 64.0 + fixed + split_cost);
+            const int64_t waves = (items + slots - 1) / slots;
+            const double cost = (double)waves * ((double)ch / tile + fixed + (per_req > 1 ? split : 0.0));
             if (cost < best_cost - 1e-9) {
                 best_cost = cost;
                 c = ch;
             }
-            if (ch <= 64) break;
+            if (ch <= tile) break;
         }
     } else {
         const int target = std::max(1, (2 * n_sm + units - 1) / units);
@@ -491,6 +491,7 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     // opt-in shared-memory sizes of every kernel, once per device and off the decode path
     if (e == cudaSuccess) e = set_attrs_naive_sm100();
     if (e == cudaSuccess) e = set_attrs_absorb_sm100();
+    if (e == cudaSuccess) e = set_attrs_absorb_pair_sm100();
     if (e == cudaSuccess) e = set_attrs_expand_sm100();
     if (e == cudaSuccess) e = set_attrs_project_sm100();
     if (e == cudaSuccess) e = set_attrs_q_absorb_sm100();
@@ -901,8 +902,9 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                       seq_lens, order, desc, B, H, pl.chunk, pl.n_shared_chunks, pl.n_suffix_chunks, softmax_scale,
                       o_part_a, lse_part_a, sh->status, forked ? nullptr : sh->w_uv, cfg.stacked_absorb};
         prof_before(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
-        e = tc ? launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s)
-               : launch_absorb_attn_mma(ab, s);
+        e = !tc ? launch_absorb_attn_mma(ab, s)
+            : absorb_uses_pairs(H) ? launch_absorb_pair_sm100(ab, sh->Ls_pad, o_lat, lse_a, sh->status, s)
+                                   : launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s);
         prof_after(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         if (e != cudaSuccess) return fail(e);
         ++launches;

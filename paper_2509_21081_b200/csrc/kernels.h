@@ -24,6 +24,7 @@ extern thread_local bool tl_pdl;
 // device current) instead of before every launch.
 cudaError_t set_attrs_naive_sm100();
 cudaError_t set_attrs_absorb_sm100();
+cudaError_t set_attrs_absorb_pair_sm100();
 cudaError_t set_attrs_expand_sm100();
 cudaError_t set_attrs_project_sm100();
 cudaError_t set_attrs_q_absorb_sm100();
@@ -189,6 +190,11 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
                                      void* o_lat_direct, float* lse_direct, int* status, cudaStream_t s);
 cudaError_t make_absorb_shared_tmaps(const void* ckv, const void* kpe, int64_t Ls_pad, CUtensorMap* tm_ckv,
                                      CUtensorMap* tm_kpe);
+
+// The same for 128 query rows per pair of CTAs (chunk must be a multiple of 128).
+inline bool absorb_uses_pairs(int H) { return H > 64; }
+cudaError_t launch_absorb_pair_sm100(const AbsorbAttn& a, int64_t Ls_pad, void* o_lat_direct, float* lse_direct, int* status,
+                                     cudaStream_t s);
 
 // perm[0..B) = request indices by descending suffix length (B <= 4096).
 // -inf into n_slots segments of `count` floats, `stride` floats apart.

@@ -315,6 +315,101 @@ __device__ __forceinline__ void tma_load_4d_if(uint32_t issue, void* dst, const 
         : "memory");
 }
 
+// ---------------------------------------------------------------- CTA pairs (cta_group::2)
+// Two CTAs of a cluster on neighbouring SMs work on one product: the even one issues the MMAs (one thread), each supplies its
+// half of A's rows and of B's columns from the same offsets of its shared memory and gets its half of the rows of D in its tensor
+// memory.  A kernel uses one cta_group for all its tcgen05 instructions.
+__device__ __forceinline__ uint32_t cluster_cta_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+    return __shfl_sync(0xffffffffu, r, 0);   // (known to be uniform, like the warp index)
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// Address (shared::cluster window) of the same variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_map(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+// Arrival on a barrier of the other CTA (an address from cluster_map).  What it announces here is in the arriving CTA's own shared
+// or tensor memory, already ordered for the tensor core of that SM by the caller's proxy / tcgen05 fence, and is read only by the
+// pair's MMA, never by threads of the other CTA: the default scope will do.  (With .release.cluster the arriving warp stood still for
+// about 1100 clocks per arrival.)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_dst, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(smem_dst)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void umma_pair_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc),
+        "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void umma_pair_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc),
+        "r"(accumulate)
+        : "memory");
+}
+// All previously issued MMAs of this thread arrive on `bar` of both CTAs when complete.
+__device__ __forceinline__ void umma_pair_commit(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+// Tiled loads into this CTA's shared memory whose bytes are counted by a barrier of either CTA of the pair (`bar`: an address
+// from cluster_map).
+__device__ __forceinline__ void tma_load_2d_pair_if(uint32_t issue, void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], "
+        "[%2];\n}\n" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair_if(uint32_t issue, void* dst, const CUtensorMap* m, uint32_t bar, int x, int y,
+                                                    int z) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5}], "
+        "[%2];\n}\n" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair_if(uint32_t issue, void* dst, const CUtensorMap* m, uint32_t bar, int x, int y,
+                                                    int z, int w) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %7, 0;\n"
+        "@q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, "
+        "%6}], [%2];\n}\n" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_4d_if(uint32_t issue, const CUtensorMap* m, int x, int y, int z, int w) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];\n}\n" ::"l"(reinterpret_cast<uint64_t>(m)),
+        "r"(x), "r"(y), "r"(z), "r"(w), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* m, const void* ssrc, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n" ::
+                     "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(ssrc)), "r"(x), "r"(y), "r"(z), "r"(w)
+                 : "memory");
+}
+
 // ---------------------------------------------------------------- packed fp32 arithmetic
 // Two fp32 lanes per instruction (sm_100): the softmax loops do their scale-and-subtract and their row sums
 // on pairs, which halves the issue slots those take next to the exponentials.
