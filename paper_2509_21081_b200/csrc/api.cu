@@ -208,7 +208,7 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
         p.n_split_naive = naive_slots_override > 0 ? 1 : 0;
         p.n_slots_naive = naive_slots_override;
     } else if (use_naive && tc) {
-        naive_sm100_plan(B, H, sh->Ls, n_sm, schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0);   // n_split_naive = tile ranges
+        naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0);   // n_split_naive = tile ranges
     } else {
         p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm) : 0;
         p.n_slots_naive = p.n_split_naive;
@@ -490,6 +490,7 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     // opt-in shared-memory sizes of every kernel, once per device and off the decode path
     if (e == cudaSuccess) e = set_attrs_naive_sm100();
+    if (e == cudaSuccess) e = set_attrs_naive_pair_sm100();
     if (e == cudaSuccess) e = set_attrs_absorb_sm100();
     if (e == cudaSuccess) e = set_attrs_absorb_pair_sm100();
     if (e == cudaSuccess) e = set_attrs_expand_sm100();
@@ -595,6 +596,7 @@ static int prepare_impl(const typhoon_mla_dims_t* dims, const void* ckv_shared, 
     if (e == cudaSuccess && Ls > 0)
         e = sh->fp8 ? make_naive_fp8_tmaps(sh->k8, sh->kpe, sh->v8, H, sh->Ls_pad, &sh->tm_kn, &sh->tm_kp, &sh->tm_vt)
                     : make_naive_sm100_tmaps(sh->k_nope, sh->kpe, sh->v_t, H, sh->Ls_pad, &sh->tm_kn, &sh->tm_kp, &sh->tm_vt);
+    if (e == cudaSuccess && Ls > 0 && !sh->fp8) e = make_naive_pair_tmap(sh->v_t, H, sh->Ls_pad, &sh->tm_vt_half);
     if (e == cudaSuccess) e = make_q_absorb_tmap(sh->w_uk_t, H, &sh->tm_wuk_t);
     if (e == cudaSuccess && Ls > 0) e = make_absorb_shared_tmaps(sh->ckv, sh->kpe, sh->Ls_pad, &sh->tm_ckv, &sh->tm_kpe_tok);
     if (e != cudaSuccess) {
@@ -813,6 +815,7 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
             NaiveAttnSm100 na{qn, qp, &x.sh->tm_kn, &x.sh->tm_kp, &x.sh->tm_vt, x.rows, H, (int)x.sh->Ls,
                               x.n_ranges, x.n_slots_level, softmax_scale, op, lp, sh->status, B};
             if (x.sh->fp8) na.fp8_mult = x.sh->fp8_f;
+            na.tm_vt_half = &x.sh->tm_vt_half;
             return na;
         };
         prof_before(TYPHOON_MLA_KERNEL_NAIVE_ATTN, s);
@@ -859,7 +862,7 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                 int naive_ctas = 0;
                 for (int j = 0; j < n_jobs; ++j) {
                     const int rows = jobs[j].rows;
-                    const int groups = jobs[j].sh->fp8 ? (rows + 127) / 128 : (rows <= 128 ? 1 : (rows + 255) / 256);
+                    const int groups = jobs[j].sh->fp8 ? (rows + 127) / 128 : (rows <= 128 ? 1 : 2 * ((rows + 255) / 256));   // CTAs per range
                     naive_ctas = std::max(naive_ctas, jobs[j].n_ranges * groups);
                 }
                 const int free_sms = sh->num_sms - naive_ctas;
@@ -1090,7 +1093,7 @@ int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int
             }
             naive_sm100_plan_multi(rows, H, len, n, n_sm, schedule, &ranges, &slots_of[j]);
         } else {
-            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, n_sm, schedule, &ranges, &slots_of[j], tp->jobs[j].sh->fp8 != 0);
+            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, naive_places(tp->jobs[j].rows, n_sm, tp->jobs[j].sh->fp8 != 0), schedule, &ranges, &slots_of[j], tp->jobs[j].sh->fp8 != 0);
         }
         for (int k = 0; k < n; ++k) tp->jobs[j + k].n_ranges = ranges;
         tp->jobs[j].n_merged = n;

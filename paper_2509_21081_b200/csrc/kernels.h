@@ -23,6 +23,7 @@ extern thread_local bool tl_pdl;
 // Opt-in shared-memory sizes of the kernels, set once per device (by typhoon_mla_prepare_shared, with that
 // device current) instead of before every launch.
 cudaError_t set_attrs_naive_sm100();
+cudaError_t set_attrs_naive_pair_sm100();
 cudaError_t set_attrs_absorb_sm100();
 cudaError_t set_attrs_absorb_pair_sm100();
 cudaError_t set_attrs_expand_sm100();
@@ -136,13 +137,20 @@ struct NaiveAttnSm100 {
     // 8-bit cache: device [2][H] power-of-two scales of K_nope and V (tm_kn / tm_vt then describe the code arrays,
     // see make_naive_fp8_tmaps); null for the 16-bit cache
     const float* fp8_mult = nullptr;
+    const CUtensorMap* tm_vt_half = nullptr;   // more than 128 rows of the 16-bit cache: from make_naive_pair_tmap
 };
 int naive_sm100_tile_tokens(int B, bool fp8 = false);   // KV tile width the kernel uses for this batch size (64 or 128)
-// CTAs (at most n_sm, each with an equal contiguous share of all (head, row group, tile) work) and
-// partial slots for a problem size; a pure function of its arguments.
+// Tile ranges (with stream-K at most `places` over the number of row groups, each with an equal contiguous share of the work) and
+// partial slots for a problem size; a pure function of its arguments.  `places` = work items that run at once: SMs, or pairs of
+// SMs for more than 128 rows of the 16-bit cache (naive_uses_pairs).
 // schedule: 0 = chosen by the plan, 1 = column split, 2 = stream-K
-void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8 = false);
+inline bool naive_uses_pairs(int B, bool fp8) { return !fp8 && B > 128; }
+inline int naive_places(int B, int n_sm, bool fp8) { return naive_uses_pairs(B, fp8) ? n_sm / 2 : n_sm; }
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8 = false);
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s);
+// ... its form for more than 128 rows of the 16-bit cache: 256 rows per pair of CTAs
+cudaError_t launch_naive_pair_sm100(const NaiveAttnSm100& a, cudaStream_t s);
+cudaError_t make_naive_pair_tmap(const void* v_t, int H, int64_t Ls_pad, CUtensorMap* tm_vt_half);
 // Up to kNaiveJobsPerLaunch prefixes of the 16-bit cache, each with at most 128 query rows, in one launch: ranges and
 // slots (per prefix) come from naive_sm100_plan_multi over the same prefixes in the same order; the jobs' n_ranges is
 // that plan's.

@@ -3,27 +3,23 @@
 // Per head h the step is a dense contraction over all B query rows:
 //     S = Q_h [B,192] * [K_nope_h | k_pe]^T [192, L_s],  O = softmax(S) * V_h [L_s,128].
 //
-// Work decomposition.  The KV tiles of all heads form one sequence of T = H * n_tiles tiles, which
-// is cut into R equal contiguous ranges.  A CTA owns one range and one group of query rows (128
-// rows for B <= 128, else 256; CTAs of the same range are adjacent in the grid, so the row groups
-// of a head walk the same KV tiles at about the same time and share them through L2).  A CTA works
-// through its range as a few "segments" (head, tile range), each a complete flash-attention pass
-// with its own Q tile that ends in a normalised fp32 partial plus LSE; the combine step merges the
-// partials of a (request, head).  The host picks R: a multiple of H (every range inside one head,
+// This kernel takes up to 128 query rows, and row groups of 128 of the 8-bit cache; naive_pair_sm100.cu takes more rows of the
+// 16-bit cache.
+//
+// Work decomposition.  The KV tiles (64 tokens) of all heads form one sequence of T = H * n_tiles tiles, which
+// is cut into R equal contiguous ranges.  A CTA owns one range and one group of query rows (CTAs of the same
+// range are adjacent in the grid, so the row groups of a head walk the same KV tiles at about the same time and
+// share them through L2).  A CTA works through its range as a few "segments" (head, tile range), each a complete
+// flash-attention pass with its own Q tile that ends in a normalised fp32 partial plus LSE; the combine step merges
+// the partials of a (request, head).  The host picks R: a multiple of H (every range inside one head,
 // "column split") or the number of SMs over the number of row groups ("stream-K": one resident CTA
 // per SM, every SM gets the same number of tiles whatever H and L_s are).
 //
-// Inside a segment two independent attention "streams" share the TMA/MMA machinery:
-//   * B > 128  (mode X, 128-token KV tiles): stream i = query rows [256g + 128i, +128); both
-//     streams consume every KV tile (tiles are loaded once).  Compute-bound regime: N = 128 per
-//     S MMA halves the re-reads of Q from shared memory, the streams ping-pong between tensor
-//     core and softmax.
-//   * B <= 128 (mode Y, 64-token KV tiles): both streams use the same 128 query rows; stream i
-//     takes every second KV tile with its own softmax state, and at the end of the segment
-//     stream 0 merges the two accumulators (same tensor-memory lanes) into one partial.
-//     HBM-bound regime: small tiles give deep K and V rings.
-//     With B <= 64 the MMAs are issued with M = 64 (template flag M64): accumulator row r then
-//     sits in lane 32 (r / 16) + r % 16 and half of the softmax lanes hold no row.
+// Inside a segment two independent attention "streams" share the TMA/MMA machinery: both use the same 128 query
+// rows; stream i takes every second KV tile with its own softmax state, and at the end of the segment
+// stream 0 merges the two accumulators (same tensor-memory lanes) into one partial.  HBM-bound regime: small tiles
+// give deep K and V rings.  With B <= 64 the MMAs are issued with M = 64 (template flag M64): accumulator row r then
+// sits in lane 32 (r / 16) + r % 16 and half of the softmax lanes hold no row.
 //
 // Warp roles (384 threads): warp 0 = TMA producer for Q and the K ring, warp 2 = TMA producer
 // for the V ring, warp 1 = issuer of the S = Q K^T MMAs and TMEM owner, warp 3 = issuer of the
@@ -32,9 +28,8 @@
 // elected lane.  Ring positions, S-buffer uses and accumulator completions are counted across
 // segments, so the pipeline never drains inside a CTA except for the Q tile of a new segment.
 //
-// Tensor memory (512 columns).  64-token tiles: S[i][buf] (64 fp32 columns, double buffered; P
-// in bf16 overwrites the first 32) at (2i+buf)*64, O[i] at 256 + 128 i.  128-token tiles: S[i]
-// (128 columns, P overwrites the first 64) at 128 i, O[i] at 256 + 128 i.
+// Tensor memory (512 columns): S[i][buf] (64 fp32 columns, double buffered; P in bf16 overwrites the first 32) at
+// (2i+buf)*64, O[i] at 256 + 128 i.
 //
 // The expanded cache is stored in 64-token blocks: K_nope [H, L/64, 2 slabs, 64, 64],
 // V^T [H, L/64, 128, 64], rope keys [L, 64]; every TMA box is a contiguous 8 or 16 KB.
@@ -107,10 +102,8 @@ struct Barriers {
     uint64_t q_full, q_free;
     uint64_t k_full[MAX_STAGES], k_empty[MAX_STAGES];
     uint64_t v_full[MAX_STAGES], v_empty[MAX_STAGES];
-    // p_half (128-token tiles): the first 64 tokens' probabilities of a tile are in place, so the PV product can start
-    // on them while the softmax warpgroup is still working on the second 64
-    uint64_t s_ready[2][2], p_ready[2][2], p_half[2], sbuf_free[2][2], o_free[2];
-    // 64-token tiles: stream 1 has published its softmax state (merge_m / merge_l) and its accumulator is
+    uint64_t s_ready[2][2], p_ready[2][2], sbuf_free[2][2], o_free[2];
+    // stream 1 has published its softmax state (merge_m / merge_l) and its accumulator is
     // complete; stream 0 then merges the two streams' results into one partial (128 arrivals per segment)
     uint64_t merge_ready;
     // completion of PV product u of stream i goes to o_done[i][u & 1]: a waiter that knows product
@@ -135,10 +128,9 @@ struct Segment {
     int n_str0, n_str1;    // tiles per stream
 };
 
-// TOK = tokens per KV tile: 64 (mode Y, B <= 128) or 128 (mode X, B > 128).
 // PAIRS > 0 (FP8): the expanded cache is stored as E4M3 codes (see the conversion warps below).
-// NJ: largest number of prefixes per launch (several: 64-token tiles of the 16-bit cache).
-template <int TOK, bool M64, int PAIRS, int NJ>
+// NJ: largest number of prefixes per launch (several: 16-bit cache).
+template <bool M64, int PAIRS, int NJ>
 __global__ void __launch_bounds__(naive_threads(PAIRS), 1)
 naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_constant__ CUtensorMap tm_qp,
                         const __grid_constant__ CUtensorMap tm_kn, const __grid_constant__ CUtensorMap tm_kp,
@@ -161,28 +153,21 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
     TMLA_JOB_MEMBER(const CUtensorMap&, kp_of, tm_kp, tm_kp)
     TMLA_JOB_MEMBER(const CUtensorMap&, vt_of, tm_vt, tm_vt)
 #undef TMLA_JOB_MEMBER
-    constexpr bool MODE_Y = TOK == 64, FP8 = PAIRS > 0;
-    // 128-token tiles (compute-bound regime): pairs of exponentials computed on the FMA pipe instead of the
-    // special-function unit, by position of the pair within a group of eight (bit set = polynomial).  Measured at
-    // B = 512: one pair in four is the best mix (-4 % kernel time); one in eight and three in eight gain 1-2 %, every
-    // second pair changes the compiler's register allocation for the worse (+5 %).
-    constexpr unsigned kPolyExpMask = TOK == 128 ? 0x88u : 0u;
-    constexpr int NB = MODE_Y ? 2 : 1;                  // S buffers per stream
-    constexpr int BLK = TOK / 64;                       // 64-token blocks per tile
+    constexpr bool FP8 = PAIRS > 0;
+    constexpr int TOK = 64;                             // tokens per KV tile
+    constexpr int NB = 2;                               // S buffers per stream
     constexpr int K_SLAB = TOK * 128;                   // bytes of one [TOK][64] K slab
     constexpr int K_TILE_BYTES = (FP8 ? 2 : 3) * K_SLAB;   // (8-bit cache: the rope slab stays in the staging ring)
-    constexpr int V_TILE_BYTES = BLK * 16384;           // BLK slabs [128 dims][64 tokens]
-    constexpr int ROWS = FP8 ? (M64 ? 64 : 128) : (MODE_Y ? 128 : 256);   // query rows per column
-    static_assert(!FP8 || TOK == 64, "the 8-bit cache path is built for 64-token tiles");
+    constexpr int V_TILE_BYTES = 16384;                 // [128 dims][64 tokens]
+    constexpr int ROWS = FP8 && M64 ? 64 : 128;         // query rows per column
     constexpr int Q_SLAB = ((FP8 && M64) ? 64 : 128) * 128;   // bytes of one [rows][64] slab of the query tile
     constexpr int Q_BYTES = 3 * Q_SLAB;
     constexpr int KQ_BYTES = 16384, VQ_BYTES = 8192;    // staging slots: K codes 8 KB + rope keys 8 KB; V codes 8 KB
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    constexpr int n_q_tiles = MODE_Y ? 1 : 2;
     uint8_t* sQ = smem;
-    uint8_t* sK = sQ + n_q_tiles * Q_BYTES;
+    uint8_t* sK = sQ + Q_BYTES;
     uint8_t* sV = sK + p.k_stages * K_TILE_BYTES;
     uint8_t* sKq = sV + p.v_stages * V_TILE_BYTES;      // staging rings (8-bit cache only)
     uint8_t* sVq = sKq + (FP8 ? p.kq_stages : 0) * KQ_BYTES;
@@ -216,13 +201,8 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         const int r_first = first_tile < big ? first_tile / (p.per + 1) : p.rem + (first_tile - big) / p.per;
         s.slot_seg = rng - r_first;
         s.last_of_col = (s.t0 + s.cnt == n_tiles_of(s.job));
-        if (MODE_Y) {
-            s.n_str0 = (s.cnt + 1) >> 1;
-            s.n_str1 = s.cnt >> 1;
-        } else {
-            s.n_str0 = s.cnt;
-            s.n_str1 = (s.row0 + 128 < rows_of(s.job)) ? s.cnt : 0;   // second row tile entirely past B: skip it
-        }
+        s.n_str0 = (s.cnt + 1) >> 1;
+        s.n_str1 = s.cnt >> 1;
         return s;
     };
     // Softmax attention does not depend on the order in which KV tiles are visited.  Segments of
@@ -235,19 +215,15 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         return s.t0 + (t >= s.cnt ? t - s.cnt : t);
     };
     // ring position (within the segment) of the KV tile used by stream i at step j; S columns of use u
-    auto entry_of = [&](int j, int i) { return MODE_Y ? 2 * j + i : j; };
-    auto s_col = [&](int i, int u) { return (uint32_t)(MODE_Y ? (2 * i + (u & 1)) * 64 : i * 128); };
+    auto entry_of = [&](int j, int i) { return 2 * j + i; };
+    auto s_col = [&](int i, int u) { return (uint32_t)((2 * i + (u & 1)) * 64); };
 
     const uint32_t ld0 = (warp == 0 && elect_one()) ? 1u : 0u;
     auto issue_q = [&](const Segment& s) {
-        const int nq = (s.n_str1 > 0 && !MODE_Y) ? 2 : 1;
-        mbar_arrive_expect_tx_if(ld0, &bar->q_full, nq * Q_BYTES);
-        for (int t = 0; t < nq; ++t) {
-            uint8_t* dst = sQ + t * Q_BYTES;
-            tma_load_3d_if(ld0, dst, &qn_of(s.job), &bar->q_full, 0, s.h, s.row0 + t * 128);
-            tma_load_3d_if(ld0, dst + Q_SLAB, &qn_of(s.job), &bar->q_full, 64, s.h, s.row0 + t * 128);
-            tma_load_3d_if(ld0, dst + 2 * Q_SLAB, &qp_of(s.job), &bar->q_full, 0, s.h, s.row0 + t * 128);
-        }
+        mbar_arrive_expect_tx_if(ld0, &bar->q_full, Q_BYTES);
+        tma_load_3d_if(ld0, sQ, &qn_of(s.job), &bar->q_full, 0, s.h, s.row0);
+        tma_load_3d_if(ld0, sQ + Q_SLAB, &qn_of(s.job), &bar->q_full, 64, s.h, s.row0);
+        tma_load_3d_if(ld0, sQ + 2 * Q_SLAB, &qp_of(s.job), &bar->q_full, 0, s.h, s.row0);
     };
     auto issue_k = [&](const Segment& s, int e, int ring_pos) {
         if (FP8) {   // one 64-token block of codes (as 64 rows of 128 bytes) and its rope keys into a staging slot
@@ -261,15 +237,11 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         }
         const int st = ring_pos % p.k_stages;
         uint8_t* dst = sK + st * K_TILE_BYTES;
-        const int blk0 = tile_of(s, e) * BLK;
+        const int blk = tile_of(s, e), gb = s.h * (tokens_pad_of(s.job) / 64) + blk;
         mbar_arrive_expect_tx_if(ld0, &bar->k_full[st], K_TILE_BYTES);
-#pragma unroll
-        for (int bi = 0; bi < BLK; ++bi) {
-            const int gb = s.h * (tokens_pad_of(s.job) / 64) + blk0 + bi;
-            tma_load_3d_if(ld0, dst + bi * 8192, &kn_of(s.job), &bar->k_full[st], 0, 0, gb);
-            tma_load_3d_if(ld0, dst + K_SLAB + bi * 8192, &kn_of(s.job), &bar->k_full[st], 0, 64, gb);
-            tma_load_2d_if(ld0, dst + 2 * K_SLAB + bi * 8192, &kp_of(s.job), &bar->k_full[st], 0, (blk0 + bi) * 64);
-        }
+        tma_load_3d_if(ld0, dst, &kn_of(s.job), &bar->k_full[st], 0, 0, gb);
+        tma_load_3d_if(ld0, dst + K_SLAB, &kn_of(s.job), &bar->k_full[st], 0, 64, gb);
+        tma_load_2d_if(ld0, dst + 2 * K_SLAB, &kp_of(s.job), &bar->k_full[st], 0, blk * 64);
     };
     auto issue_v = [&](const Segment& s, int e, int ring_pos, uint32_t ld) {
         if (FP8) {
@@ -279,11 +251,8 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
             return;
         }
         const int st = ring_pos % p.v_stages;
-        const int blk0 = tile_of(s, e) * BLK;
         mbar_arrive_expect_tx_if(ld, &bar->v_full[st], V_TILE_BYTES);
-#pragma unroll
-        for (int bi = 0; bi < BLK; ++bi)
-            tma_load_4d_if(ld, sV + st * V_TILE_BYTES + bi * 16384, &vt_of(s.job), &bar->v_full[st], 0, 0, blk0 + bi, s.h);
+        tma_load_4d_if(ld, sV + st * V_TILE_BYTES, &vt_of(s.job), &bar->v_full[st], 0, 0, tile_of(s, e), s.h);
     };
 
     // Warp 0 initialises the barriers (one per lane) and at once issues the first segment's Q and
@@ -380,8 +349,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         }
         v_issued = ring;
     } else if (warp == 1) {
-        // ---------------- S = Q K^T issuer.  With two S buffers per stream it runs ahead of the softmax by
-        // up to two steps; with one it follows the PV product of the previous step.
+        // ---------------- S = Q K^T issuer: runs ahead of the softmax by up to two steps
         const uint32_t ld = elect_one() ? 1u : 0u;
         constexpr uint32_t idesc_s = idesc_bf16(M64 ? 64 : 128, TOK, false, false);
         constexpr uint32_t idesc_s_nope = FP8 ? idesc_f16(M64 ? 64 : 128, TOK, false, false) : idesc_s;
@@ -397,31 +365,27 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                     if (j >= (i == 0 ? s.n_str0 : s.n_str1)) continue;
                     const int ring = ring_base + entry_of(j, i);
                     const int st = ring % p.k_stages;
-                    // Awaited: the K tile (mode X: stream 1 reuses stream 0's), with the 8-bit cache also the staging slot
-                    // whose rope keys the product reads, and, from the NB-th use on, the PV product that read P from this
+                    // Awaited: the K tile, with the 8-bit cache also the staging slot whose rope keys the product reads, and, from the NB-th use on, the PV product that read P from this
                     // S buffer NB uses ago.  The barriers are tested together: each test of a barrier costs about 200
                     // clocks even when its phase is complete, and this warp's loop is the pace of the 64-token kernels.
                     const int u = (i == 0 ? used0 : used1) + j;
-                    const bool need_k = MODE_Y || i == 0, need_s = u >= NB;
+                    const bool need_s = u >= NB;
                     uint64_t* const kf = &bar->k_full[st];
                     uint64_t* const kq = &bar->kq_full[FP8 ? ring % p.kq_stages : 0];
                     uint64_t* const sf = &bar->sbuf_free[i][u % NB];
                     const uint32_t kf_par = (ring / p.k_stages) & 1, kq_par = FP8 ? (ring / p.kq_stages) & 1 : 0;
                     const uint32_t sf_par = ((u / NB) - 1) & 1;
-                    if (need_k && need_s)
+                    if (need_s)
                         ok = FP8 ? mbar_wait3_warp(kf, kf_par, kq, kq_par, sf, sf_par, abort_flag)
                                  : mbar_wait2_warp(kf, kf_par, sf, sf_par, abort_flag);
-                    else if (need_k)
+                    else
                         ok = FP8 ? mbar_wait2_warp(kf, kf_par, kq, kq_par, abort_flag) : mbar_wait_warp(kf, kf_par, abort_flag);
-                    else if (need_s)
-                        ok = mbar_wait_warp(sf, sf_par, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t qa = smem_u32(sQ + (MODE_Y ? 0 : i) * Q_BYTES);
+                    const uint32_t qa = smem_u32(sQ);
                     const uint32_t ka = smem_u32(sK + st * K_TILE_BYTES);
                     const uint32_t rope = FP8 ? smem_u32(sKq + (ring % p.kq_stages) * KQ_BYTES + 8192) : ka + 2 * K_SLAB;
                     const uint32_t d = tmem_base + s_col(i, u);
-                    const bool last_user = MODE_Y || i == 1 || s.n_str1 == 0;
 #pragma unroll
                     for (int slab = 0; slab < 3; ++slab) {
                         const uint64_t da = smem_desc_k_sw128(qa + slab * Q_SLAB);
@@ -431,7 +395,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                             umma_ss_if(ld, d, da + 2 * k, db + 2 * k, slab == 2 ? idesc_s : idesc_s_nope, (slab | k) != 0);
                     }
                     umma_commit_if(ld, &bar->s_ready[i][u % NB]);
-                    if (last_user) umma_commit_if(ld, &bar->k_empty[st]);   // last user releases the ring slot
+                    umma_commit_if(ld, &bar->k_empty[st]);                  // releases the ring slot
                     if (FP8) umma_commit_if(ld, &bar->kq_empty[ring % p.kq_stages]);   // ... and the staging slot (rope keys read, codes widened before)
                 }
             }
@@ -457,10 +421,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                     const int st = ring % p.v_stages;
                     // the V tile and the probabilities, tested together (see the S issuer)
                     const int u = (i == 0 ? used0 : used1) + j;
-                    uint64_t* const pf = MODE_Y ? &bar->p_ready[i][u % NB] : &bar->p_half[i];
-                    const uint32_t pf_par = MODE_Y ? (u / NB) & 1 : u & 1;
-                    if (MODE_Y || i == 0) ok = mbar_wait2_warp(&bar->v_full[st], (ring / p.v_stages) & 1, pf, pf_par, abort_flag);
-                    else ok = mbar_wait_warp(pf, pf_par, abort_flag);
+                    ok = mbar_wait2_warp(&bar->v_full[st], (ring / p.v_stages) & 1, &bar->p_ready[i][u % NB], (u / NB) & 1, abort_flag);
                     if (!ok) break;
                     if (j == 0 && seg > 0) {   // the previous segment's epilogue has read this accumulator
                         ok = mbar_wait_warp(&bar->o_free[i], (seg - 1) & 1, abort_flag);
@@ -470,23 +431,12 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                     const uint32_t va = smem_u32(sV + st * V_TILE_BYTES);
                     const uint32_t pa = tmem_base + s_col(i, u);
                     const uint32_t d = tmem_base + 256u + (uint32_t)i * 128u;
-                    const bool last_user = MODE_Y || i == 1 || s.n_str1 == 0;
+                    const uint64_t db = smem_desc_k_sw128(va);
 #pragma unroll
-                    for (int bi = 0; bi < BLK; ++bi) {
-                        if (bi == 1) {   // second 64 tokens of a 128-token tile: the rest of the probabilities
-                            ok = mbar_wait_warp(&bar->p_ready[i][u % NB], (u / NB) & 1, abort_flag);
-                            if (!ok) break;
-                            tc_fence_after();
-                        }
-                        const uint64_t db = smem_desc_k_sw128(va + bi * 16384);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            umma_ts_if(ld, d, pa + 8 * (bi * 4 + k), db + 2 * k, idesc_o, (j | bi | k) != 0);
-                    }
-                    if (!ok) break;
+                    for (int k = 0; k < 4; ++k) umma_ts_if(ld, d, pa + 8 * k, db + 2 * k, idesc_o, (j | k) != 0);
                     umma_commit_if(ld, &bar->o_done[i][u & 1]);
                     umma_commit_if(ld, &bar->sbuf_free[i][u % NB]);
-                    if (last_user) umma_commit_if(ld, &bar->v_empty[st]);
+                    umma_commit_if(ld, &bar->v_empty[st]);
                 }
             }
             used0 += s.n_str0;
@@ -508,7 +458,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         bool ok = true;
         for (int g = g_begin; g < g_end && ok;) {
             const Segment s = segment_at(g);
-            const int tile_row0 = s.row0 + (MODE_Y ? 0 : i * 128);
+            const int tile_row0 = s.row0;
             const int b = lane_has_row ? tile_row0 + row : 0x3fffffff;
             const int nt = i == 0 ? s.n_str0 : s.n_str1;
             const bool warp_has_rows = tile_row0 + (M64 ? (warp & 3) * 16 : lg) < rows_of(s.job);   // warp-uniform: the warp's first row is a real request
@@ -527,7 +477,6 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                     // all 32 rows of this warp are padding past B: their P rows may hold anything (rows of
                     // the MMA are independent and these output rows are never stored); just keep in step
                     tc_fence_before();
-                    if (!MODE_Y) mbar_arrive(&bar->p_half[i]);
                     mbar_arrive(&bar->p_ready[i][buf]);
                     continue;
                 }
@@ -621,21 +570,18 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 // of its dependent instruction chains counts, not only the number of instructions)
                 float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                 uint32_t sr[2][32];
+                tmem_ld32(s_addr, sr[0]);
+                tmem_ld32(s_addr + 32, sr[1]);
+                tmem_ld_wait();
+                if (valid < TOK) {
 #pragma unroll
-                for (int half = 0; half < BLK; ++half) {
-                    tmem_ld32(s_addr + half * 64, sr[0]);
-                    tmem_ld32(s_addr + half * 64 + 32, sr[1]);
-                    tmem_ld_wait();
-                    if (valid < TOK) {
-#pragma unroll
-                        for (int c = 0; c < 64; ++c)
-                            if (half * 64 + c >= valid) sr[c >> 5][c & 31] = 0xff800000u;   // -inf
-                    }
-#pragma unroll
-                    for (int c = 0; c < 64; c += 2)
-                        mx4[(c >> 1) & 3] = max3(mx4[(c >> 1) & 3], __uint_as_float(sr[c >> 5][c & 31]),
-                                                 __uint_as_float(sr[(c + 1) >> 5][(c + 1) & 31]));
+                    for (int c = 0; c < 64; ++c)
+                        if (c >= valid) sr[c >> 5][c & 31] = 0xff800000u;   // -inf
                 }
+#pragma unroll
+                for (int c = 0; c < 64; c += 2)
+                    mx4[(c >> 1) & 3] = max3(mx4[(c >> 1) & 3], __uint_as_float(sr[c >> 5][c & 31]),
+                                             __uint_as_float(sr[(c + 1) >> 5][(c + 1) & 31]));
                 const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_l2;
                 // lazy rescale: only when some row's maximum grew by more than 2^8
                 const bool grow = lane_has_row && mx > m_ref + 8.f;
@@ -664,8 +610,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                     tmem_st_wait();
                 }
                 // pass 2: p = 2^(s * scale - m_ref) (one FMA and one ex2 per element), packed to bf16 over
-                // the S columns (P column c holds tokens 2c, 2c+1); with 128-token tiles the logits are read
-                // again, 64 at a time, to stay within the register budget
+                // the S columns (P column c holds tokens 2c, 2c+1)
                 const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
                 // probabilities of 32 logits held in `src`: 16 packed bf16 pairs, sums into the four partial sums
                 auto probs32 = [&](const uint32_t (&src)[32], uint32_t (&dst)[16]) {
@@ -674,49 +619,18 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                         // two logits per instruction: distance to the reference exponent, probabilities, running sums
                         float x0, x1;
                         unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(src[2 * c]), __uint_as_float(src[2 * c + 1])), scale2, neg_m2), x0, x1);
-                        float p0, p1;
-                        if ((kPolyExpMask >> (c & 7)) & 1) {
-                            exp2_poly_x2(x0, x1, p0, p1);
-                        } else {
-                            p0 = fast_exp2(x0);
-                            p1 = fast_exp2(x1);
-                        }
+                        const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
                         dst[c] = FP8 ? pack_f16(p0, p1) : pack_bf16(p0, p1);
                         if (c & 1) l_sum2b = add_f32x2(l_sum2b, pack_f32x2(p0, p1));
                         else l_sum2 = add_f32x2(l_sum2, pack_f32x2(p0, p1));
                     }
                 };
-                if (BLK == 1) {
-                    // the 64 logits of pass 1 are still in registers
-                    uint32_t pk[2][16];
-                    probs32(sr[0], pk[0]);
-                    tmem_st16(s_addr, pk[0]);
-                    probs32(sr[1], pk[1]);
-                    tmem_st16(s_addr + 16, pk[1]);
-                } else {
-                    // 128-token tiles: the logits are read again, 32 at a time with the next 32 already requested, to stay
-                    // within the register budget.  Quarter q covers S columns [32 q, 32 q + 32) and writes P columns
-                    // [16 q, 16 q + 16): those overlap only S columns that are already in registers or consumed.
-                    tmem_ld32(s_addr, sr[0]);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        tmem_ld_wait();
-                        if (q < 3) tmem_ld32(s_addr + (q + 1) * 32, sr[(q + 1) & 1]);
-                        if (valid < TOK) {
-#pragma unroll
-                            for (int c = 0; c < 32; ++c)
-                                if (q * 32 + c >= valid) sr[q & 1][c] = 0xff800000u;
-                        }
-                        uint32_t pk[16];
-                        probs32(sr[q & 1], pk);
-                        tmem_st16(s_addr + q * 16, pk);
-                        if (q == 1) {   // first half of the tile's probabilities in place
-                            tmem_st_wait();
-                            tc_fence_before();
-                            mbar_arrive(&bar->p_half[i]);
-                        }
-                    }
-                }
+                // the 64 logits of pass 1 are still in registers
+                uint32_t pk[2][16];
+                probs32(sr[0], pk[0]);
+                tmem_st16(s_addr, pk[0]);
+                probs32(sr[1], pk[1]);
+                tmem_st16(s_addr + 16, pk[1]);
                 tmem_st_wait();
                 tc_fence_before();
                 mbar_arrive(&bar->p_ready[i][buf]);
@@ -744,18 +658,17 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 unpack_f32x2(add_f32x2(l_sum2, l_sum2b), a, c);
                 l_sum = a + c;
             }
-            // ---- segment epilogue: normalised partial + LSE into this segment's slot.  With 64-token tiles the two
+            // ---- segment epilogue: normalised partial + LSE into this segment's slot.  The two
             // streams worked on the same query rows: stream 1 publishes its softmax state, stream 0 merges both
             // accumulators (same tensor-memory lanes) and writes one partial.
             const int slot = s.slot_seg;
-            const bool owns_rows = MODE_Y ? i == 0 : (i == 0 || s.row0 + 128 < rows_of(s.job));
             if (nt > 0) {
                 const int u_last = used + nt - 1;
                 ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_done[i][u_last & 1], (u_last >> 1) & 1, abort_flag));
                 if (!ok) break;
                 tc_fence_after();
             }
-            if (MODE_Y && i == 1) {
+            if (i == 1) {
                 if (segi > 0) {   // stream 0 has read what the previous segment published (it frees O1 after that)
                     ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_free[1], (segi - 1) & 1, abort_flag));
                     if (!ok) break;
@@ -765,29 +678,23 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                 tc_fence_before();
                 mbar_arrive(&bar->merge_ready);
             } else {
-                float a0 = 0.f, a1 = 0.f, lse2 = -INFINITY;   // weights of the two accumulators, LSE in base 2
-                if (MODE_Y) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&bar->merge_ready, segi & 1, abort_flag));
-                    if (!ok) break;
-                    tc_fence_after();
-                    const float m1 = bar->merge_m[r], l1 = bar->merge_l[r];
-                    const float m = fmaxf(m_ref, m1);           // stream 0 always has a tile: m_ref is finite
-                    const float e0 = fast_exp2(m_ref - m), e1 = l1 > 0.f ? fast_exp2(m1 - m) : 0.f;
-                    const float l = l_sum * e0 + l1 * e1;
-                    a0 = e0 / l;
-                    a1 = e1 / l;
-                    lse2 = m + log2f(l);
-                } else if (nt > 0) {
-                    a0 = 1.f / l_sum;
-                    lse2 = m_ref + log2f(l_sum);
-                }
+                // weights of the two accumulators, LSE in base 2
+                ok = __all_sync(0xffffffffu, mbar_wait(&bar->merge_ready, segi & 1, abort_flag));
+                if (!ok) break;
+                tc_fence_after();
+                const float m1 = bar->merge_m[r], l1 = bar->merge_l[r];
+                const float m = fmaxf(m_ref, m1);           // stream 0 always has a tile: m_ref is finite
+                const float e0 = fast_exp2(m_ref - m), e1 = l1 > 0.f ? fast_exp2(m1 - m) : 0.f;
+                const float l = l_sum * e0 + l1 * e1;
+                float a0 = e0 / l, a1 = e1 / l;
+                const float lse2 = m + log2f(l);
                 if (FP8) {   // the accumulators hold P times the V codes' values: the true values divided by the scale
                     const float vm = p.mult[p.H + s.h];
                     a0 *= vm;
                     a1 *= vm;
                 }
-                if (nt > 0 && warp_has_rows) {
-                    const uint32_t o_addr = tmem_base + ((uint32_t)lg << 16) + 256u + (uint32_t)(MODE_Y ? 0 : i) * 128u;
+                if (warp_has_rows) {
+                    const uint32_t o_addr = tmem_base + ((uint32_t)lg << 16) + 256u;
                     float* dst = o_part_of(s.job) + (((int64_t)slot * p.part_rows + b) * p.H + s.h) * 128;
 #pragma unroll 1
                     for (int c = 0; c < 4; ++c) {
@@ -797,7 +704,7 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                         float v[32];
 #pragma unroll
                         for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(orr[q]) * a0;
-                        if (MODE_Y && s.n_str1 > 0) {   // uniform over the CTA (the tensor-memory load is warp-collective)
+                        if (s.n_str1 > 0) {   // uniform over the CTA (the tensor-memory load is warp-collective)
                             tmem_ld32(o_addr + 128u + c * 32, orr);
                             tmem_ld_wait();
 #pragma unroll
@@ -810,18 +717,16 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
                         }
                     }
                     if (b < rows_of(s.job)) lse_part_of(s.job)[((int64_t)slot * p.part_rows + b) * p.H + s.h] = lse2 * kLn2;
-                } else if (nt == 0 && owns_rows && b < rows_of(s.job)) {
-                    lse_part_of(s.job)[((int64_t)slot * p.part_rows + b) * p.H + s.h] = -INFINITY;   // this stream had no tile
                 }
                 // the segment that ends a head marks the head's unused slots as empty
-                if (s.last_of_col && owns_rows && b < rows_of(s.job)) {
+                if (s.last_of_col && b < rows_of(s.job)) {
                     for (int ss = s.slot_seg + 1; ss < n_slots_of(s.job); ++ss)
                         lse_part_of(s.job)[((int64_t)ss * p.part_rows + b) * p.H + s.h] = -INFINITY;
                 }
                 // the accumulator(s) just read may be overwritten by the next segment
                 tc_fence_before();
-                mbar_arrive(&bar->o_free[i]);
-                if (MODE_Y) mbar_arrive(&bar->o_free[1]);
+                mbar_arrive(&bar->o_free[0]);
+                mbar_arrive(&bar->o_free[1]);
             }
             ++segi;
             used += nt;
@@ -987,9 +892,9 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // may run in several waves); ns minimises waves x (tiles per CTA + a fixed cost of about six tile
 // times for the Q load and the pipeline fill).  "Stream-K" uses R = SMs / row groups resident
 // CTAs and gives every SM the same number of tiles at the price of a few more segments (each
-// pays the fixed cost and a partial slot; with 64-token tiles a further slot per head is also charged
-// the extra read it causes in the combine).  Stream-K is taken when its modelled cost is lower (by at
-// least 5% in the HBM-bound regime of 64-token tiles).
+// pays the fixed cost and a partial slot; a further slot per head is also charged the extra read it
+// causes in the combine).  Stream-K is taken when its modelled cost is lower by at least 5%.  (With more than
+// 128 rows of the 16-bit cache a place is a pair of SMs, see naive_pair_sm100.cu.)
 //
 // `n` prefixes (at most kNaiveJobsPerLaunch, of Ls[i] tokens): the sequence holds all prefixes' tiles of a head, then the next
 // head's; n_slots[i] are the slots of prefix i.  Runs on every call of a step, so the slots of all prefixes come from one walk
@@ -1033,31 +938,58 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
             }
         return most;
     };
+    // With more than 128 rows of the 16-bit cache ranges may also hold several whole heads (one segment each, one slot per
+    // head), and a choice is charged half its time and half its SM time: places that it leaves free go to the absorb branch.
+    // (700 rows x 32 heads over 2048 tokens + 64: 106 us per step with 48 of 74 pairs, 123 with 72.)  But a few free SMs only help if the
+    // query absorption, about 4 us per head and 128 requests, gets done on them meanwhile; else it had better wait for all
+    // SMs.  (64 pairs / 74, us per step of 128 heads: 140 rows, 3000 + 500 tokens 120 / 132, 200 rows, 2000 + 300 tokens 156 / 128.)
+    const bool pairs = !mode_y;
+    auto charge = [&](double cost, long long items) {   // `cost` of all waves
+        const double waves = (double)((items + n_sm - 1) / n_sm);
+        return pairs ? cost * (0.5 + 0.5 * (double)items / (waves * n_sm)) : cost;
+    };
+    auto absorption_fits = [&](double cost, long long items) { return cost * 0.9 * 2.0 * (double)(n_sm - items) >= 4.0 * H * ((B + 127) / 128); };
     // column split
     const long long base = (long long)H * m_groups;
-    const double fixed = 6.0;
+    // Cost of a range's beginning and of each further segment, in tile times.  (A pair of CTAs requests the next segment's queries
+    // early and goes on with its logits while the last segment's output is written; a further wave of pairs costs a launch, its
+    // set-up and a pipeline fill.  700 rows x 128 heads over 500 tokens, six waves: 103 us, the work of 50.)
+    const double fixed = 6.0, boundary = mode_y ? 6.0 : 3.0;
     // every further partial slot is one more dependent read of B x H x 128 floats in the combine that follows
-    // (about 5 us, i.e. 8 tile times, measured with 64-token tiles; not significant next to 128-token tiles)
-    const double slot_cost = mode_y ? 8.0 : 0.0;
+    // (about 5 us, i.e. 8 tile times, measured with 64-token tiles; with more than 128 rows the bytes count: 512 per row and
+    // head at 5 TB/s, in tiles of 0.9 us)
+    const double slot_cost = mode_y ? 8.0 : 1.1e-4 * B * H;
     int ns_best = 1;
     double cost_best = 1e30, eff_best = 0.0;
     for (int ns = 1; ns <= std::min(n_tiles, 32); ++ns) {
         const int per = (n_tiles + ns - 1) / ns;
         if (n_tiles % ns != 0) continue;   // equal parts only: every range stays inside one head
         const long long waves = (ns * base + n_sm - 1) / n_sm;
-        const double cost = (double)waves * (per + fixed) + slot_cost * (ns - 1);
+        const double cost = charge((double)waves * (per + fixed) + slot_cost * (ns - 1), ns * base);
         if (cost < cost_best - 1e-9) {
             cost_best = cost;
             ns_best = ns;
             eff_best = (double)(T * m_groups) / ((double)waves * per * n_sm);
         }
     }
+    int r_column = H * ns_best;
+    if (pairs && schedule == 0)
+        for (int k = 2; k <= H; ++k) {   // whole heads, k per range, in one wave
+            const long long items = (long long)(H / k) * m_groups;
+            const double time = (double)k * n_tiles + fixed + (k - 1) * boundary;
+            if (H % k != 0 || items > n_sm || !absorption_fits(time, items)) continue;
+            if (charge(time, items) < cost_best - 1e-9) {
+                cost_best = charge(time, items);
+                r_column = H / k;
+            }
+        }
     // stream-K: equal ranges; a CTA meets at most (tiles per range / tiles per head) + 2 segments
     const int r_stream = (int)std::min<long long>(std::max(1, n_sm / m_groups), T);
     const long long per_stream = (T + r_stream - 1) / r_stream;
     const long long waves_stream = ((long long)r_stream * m_groups + n_sm - 1) / n_sm;
     const double segs_stream = (per_stream >= n_tiles) ? (double)per_stream / n_tiles + 1.0 : 2.0;
-    const double cost_stream = (double)waves_stream * (per_stream + segs_stream * fixed) + slot_cost * (fill_slots(r_stream) - 1);
+    const double cost_stream = charge((double)waves_stream * (per_stream + fixed + (segs_stream - 1.0) * boundary) + slot_cost * (fill_slots(r_stream) - 1),
+                                      (long long)r_stream * m_groups);
     bool stream_k;
     if (schedule == 1) stream_k = false;
     else if (schedule == 2) stream_k = true;
@@ -1069,7 +1001,7 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
         // the concurrent absorb branch and writes fewer partials
         stream_k = !hbm_bound_small && cost_stream < (mode_y ? 0.95 : 1.0) * cost_best;
     }
-    const int R = stream_k ? r_stream : H * ns_best;
+    const int R = stream_k ? r_stream : r_column;
     *n_ranges = R;
     if (R != r_stream) fill_slots(R);   // the kernel uses the same partition
 }
@@ -1105,11 +1037,10 @@ cudaError_t query_tmaps(const NaiveAttnSm100& a, CUtensorMap* tm_qn, CUtensorMap
 
 // Launch parameters for `n_tiles` tiles per head and at most `rows` query rows per prefix, and the shared memory.
 cudaError_t fill_params(const NaiveAttnSm100& a, int rows, long long n_tiles, NaiveSm100Params* p, int* smem) {
-    const bool fp8 = a.fp8_mult != nullptr, mode_y = fp8 || rows <= 128;
-    const int tok = mode_y ? 64 : 128;
+    const bool fp8 = a.fp8_mult != nullptr;
     p->B = a.B; p->H = a.H; p->Ls = a.Ls; p->Ls_pad = (a.Ls + 127) / 128 * 128;
     p->part_rows = a.part_rows > 0 ? a.part_rows : a.B;
-    p->m_groups = fp8 ? (rows + 127) / 128 : (mode_y ? 1 : (rows + 255) / 256);
+    p->m_groups = fp8 ? (rows + 127) / 128 : 1;
     p->n_ranges = a.n_ranges;
     const long long T = (long long)a.H * n_tiles;
     if (T >= (1LL << 31) || a.n_ranges > T) return cudaErrorInvalidValue;
@@ -1117,15 +1048,15 @@ cudaError_t fill_params(const NaiveAttnSm100& a, int rows, long long n_tiles, Na
     p->per = (int)(T / a.n_ranges);
     p->rem = (int)(T % a.n_ranges);
     p->n_seg_max = a.n_slots;
-    p->k_stages = fp8 ? (rows <= 64 ? 3 : 2) : (mode_y ? 4 : 2);   // (8-bit cache: the 128-row query tile takes 24 KB more)
-    p->v_stages = fp8 ? (rows <= 64 ? 3 : 2) : (mode_y ? 4 : 1);
+    p->k_stages = fp8 ? (rows <= 64 ? 3 : 2) : 4;   // (8-bit cache: the 128-row query tile takes 24 KB more)
+    p->v_stages = fp8 ? (rows <= 64 ? 3 : 2) : 4;
     p->kq_stages = fp8 ? 4 : 0;
     p->vq_stages = fp8 ? 4 : 0;
     p->mult = a.fp8_mult;
     p->scale_log2 = a.scale * kLog2e;
     p->o_part = a.o_part; p->lse_part = a.lse_part; p->status = a.status;
-    const int k_tile = fp8 ? 16384 : tok * 384, v_tile = mode_y ? 16384 : 32768;
-    *smem = ((fp8 && rows <= 64) ? Q_TILE_BYTES / 2 : (mode_y ? 1 : 2) * Q_TILE_BYTES) + p->k_stages * k_tile + p->v_stages * v_tile +
+    const int k_tile = fp8 ? 16384 : 64 * 384, v_tile = 16384;
+    *smem = ((fp8 && rows <= 64) ? Q_TILE_BYTES / 2 : Q_TILE_BYTES) + p->k_stages * k_tile + p->v_stages * v_tile +
             p->kq_stages * 16384 + p->vq_stages * 8192 + 1024 + (int)sizeof(Barriers) + 64;
     return *smem > kNaiveSmemMax ? cudaErrorInvalidValue : cudaSuccess;
 }
@@ -1135,11 +1066,11 @@ cudaError_t fill_params(const NaiveAttnSm100& a, int rows, long long n_tiles, Na
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s) {
     if (a.B <= 0 || a.Ls <= 0 || a.n_ranges <= 0) return cudaSuccess;
     const bool fp8 = a.fp8_mult != nullptr;
-    const int tok = naive_sm100_tile_tokens(a.B, fp8);
+    if (naive_uses_pairs(a.B, fp8)) return launch_naive_pair_sm100(a, s);
     NaiveSm100Params p{};
     CUtensorMap tm_qn, tm_qp;
     int smem = 0;
-    cudaError_t e = fill_params(a, a.B, (a.Ls + tok - 1) / tok, &p, &smem);
+    cudaError_t e = fill_params(a, a.B, (a.Ls + 63) / 64, &p, &smem);
     if (e == cudaSuccess) e = query_tmaps(a, &tm_qn, &tm_qp);
     if (e != cudaSuccess) return e;
     auto launch = [&](auto* kernel, int threads) {
@@ -1147,12 +1078,11 @@ cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s) {
                           NaiveSm100Jobs<1>{});
     };
     if (fp8 && a.B <= 64)
-        return p.per >= kTwoPairTiles ? launch(naive_attn_sm100_kernel<64, true, 2, 1>, naive_threads(2)) : launch(naive_attn_sm100_kernel<64, true, 1, 1>, naive_threads(1));
-    if (fp8) return launch(naive_attn_sm100_kernel<64, false, 1, 1>, naive_threads(1));
+        return p.per >= kTwoPairTiles ? launch(naive_attn_sm100_kernel<true, 2, 1>, naive_threads(2)) : launch(naive_attn_sm100_kernel<true, 1, 1>, naive_threads(1));
+    if (fp8) return launch(naive_attn_sm100_kernel<false, 1, 1>, naive_threads(1));
     // (up to 64 rows half-height MMAs: the padding rows 64..127 of the query tile cost tensor-pipe time and power)
-    if (a.B <= 64) return launch(naive_attn_sm100_kernel<64, true, 0, 1>, 384);
-    if (a.B <= 128) return launch(naive_attn_sm100_kernel<64, false, 0, 1>, 384);
-    return launch(naive_attn_sm100_kernel<128, false, 0, 1>, 384);
+    if (a.B <= 64) return launch(naive_attn_sm100_kernel<true, 0, 1>, 384);
+    return launch(naive_attn_sm100_kernel<false, 0, 1>, 384);
 }
 
 cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaStream_t s) {
@@ -1187,7 +1117,7 @@ cudaError_t launch_naive_attn_sm100_multi(const NaiveAttnSm100* a, int n, cudaSt
     auto launch = [&](auto* kernel) {
         return launch_pdl(kernel, dim3(p.n_ranges), dim3(384), smem, s, j0.tm_qn, j0.tm_qp, j0.tm_kn, j0.tm_kp, j0.tm_vt, p, jobs);
     };
-    return rows <= 64 ? launch(naive_attn_sm100_kernel<64, true, 0, kJobs>) : launch(naive_attn_sm100_kernel<64, false, 0, kJobs>);
+    return rows <= 64 ? launch(naive_attn_sm100_kernel<true, 0, kJobs>) : launch(naive_attn_sm100_kernel<false, 0, kJobs>);
 }
 
 cudaError_t set_attrs_naive_sm100() {
@@ -1195,14 +1125,13 @@ cudaError_t set_attrs_naive_sm100() {
     auto opt_in = [&](auto* kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNaiveSmemMax);
     };
-    opt_in(naive_attn_sm100_kernel<64, true, 0, 1>);
-    opt_in(naive_attn_sm100_kernel<64, false, 0, 1>);
-    opt_in(naive_attn_sm100_kernel<128, false, 0, 1>);
-    opt_in(naive_attn_sm100_kernel<64, true, 1, 1>);
-    opt_in(naive_attn_sm100_kernel<64, true, 2, 1>);
-    opt_in(naive_attn_sm100_kernel<64, false, 1, 1>);
-    opt_in(naive_attn_sm100_kernel<64, true, 0, kJobs>);
-    opt_in(naive_attn_sm100_kernel<64, false, 0, kJobs>);
+    opt_in(naive_attn_sm100_kernel<true, 0, 1>);
+    opt_in(naive_attn_sm100_kernel<false, 0, 1>);
+    opt_in(naive_attn_sm100_kernel<true, 1, 1>);
+    opt_in(naive_attn_sm100_kernel<true, 2, 1>);
+    opt_in(naive_attn_sm100_kernel<false, 1, 1>);
+    opt_in(naive_attn_sm100_kernel<true, 0, kJobs>);
+    opt_in(naive_attn_sm100_kernel<false, 0, kJobs>);
     return e;
 }
 
