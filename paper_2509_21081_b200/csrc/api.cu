@@ -157,7 +157,7 @@ int naive_splits(int B, int H, int64_t Ls, int n_sm) {
 
 void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int* chunk, int* n_sh,
                    int* n_sf) {
-    const bool pair = tc && absorb_uses_pairs(H);
+    const bool pair = tc && absorb_uses_pairs(B, H, Ls_absorb, cap_suffix);
     const int row_tile = pair ? 128 : 64;
     const int units = B * ((H + row_tile - 1) / row_tile);
     // work items per shared-prefix chunk: row groups of the stacked [B * H] query matrix, or of each request
@@ -906,7 +906,7 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                       o_part_a, lse_part_a, sh->status, forked ? nullptr : sh->w_uv, cfg.stacked_absorb};
         prof_before(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         e = !tc ? launch_absorb_attn_mma(ab, s)
-            : absorb_uses_pairs(H) ? launch_absorb_pair_sm100(ab, sh->Ls_pad, o_lat, lse_a, sh->status, s)
+            : absorb_uses_pairs(B, H, ab.Ls_absorb, (int64_t)max_pages * page_size) ? launch_absorb_pair_sm100(ab, sh->Ls_pad, o_lat, lse_a, sh->status, s)
                                    : launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s);
         prof_after(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         if (e != cudaSuccess) return fail(e);

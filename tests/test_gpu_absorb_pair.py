@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 LENGTHS = [0, 1, 15, 16, 17, 48, 63, 64, 65, 80, 112, 113, 127, 128, 129, 144, 191, 192, 193, 255, 256, 257, 385, 1000]
 
 
-@pytest.mark.parametrize("H,page,Ls,late", [(128, 64, 300, 1), (128, 128, 129, 8), (80, 64, 64, 1), (96, 128, 1, 1), (112, 64, 1153, 8)])
+@pytest.mark.parametrize("H,page,Ls,late", [(128, 64, 300, 1), (128, 128, 129, 8), (80, 64, 64, 1), (96, 128, 1, 1), (112, 64, 1153, 8),
+                                            (16, 64, 1100, 8), (64, 128, 1025, 1)])
 @pytest.mark.parametrize("B", [len(LENGTHS), 1])
 def test_lengths_and_rows(H, page, Ls, late, B):
     from paper_2509_21081_b200 import binding as b
