@@ -271,8 +271,9 @@ naive_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
                     umma_pair_ts(tmem_base, pa + 8 * k, db + (k >> 2) * (SLAB / 16) + 2 * (k & 3), idesc_o, (e_p | k) != 0);
-                umma_pair_commit(&bar->o_done[t & 3]);
+                // o_done last: the odd CTA waits for it before it leaves, not for the v_empty of its last tiles
                 umma_pair_commit(&bar->v_empty[st]);
+                umma_pair_commit(&bar->o_done[t & 3]);
             }
             __syncwarp();
             if (++e_p == sp.cnt) {
