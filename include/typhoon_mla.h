@@ -159,7 +159,9 @@ int typhoon_mla_release_cached(void);
 
 /* Bytes of scratch typhoon_mla_decode needs for this problem size in `mode`
  * (TYPHOON_MLA_MODE_AUTO: the worst case over the modes AUTO may resolve to, so the
- * same workspace serves every step whatever the crossover rule picks).  Host, pure:
+ * same workspace serves every step whatever the crossover rule picks).  A workspace of this
+ * size also serves every step of fewer requests or a narrower page table (a step whose own
+ * choice of partials is larger takes fewer).  Host, pure:
  * it reads the handle and touches no process-wide state, so it may be called from
  * any thread at any time.  Returns 0 on invalid arguments. */
 size_t typhoon_mla_workspace_bytes(const typhoon_mla_shared_t* shared, int32_t B,

@@ -147,16 +147,17 @@ struct Plan {
 constexpr int kDefaultNumSM = 148;        // a B200; used where no device is at hand (pure planning queries)
 constexpr int kMaxAbsorbChunks = 1024;   // chunks per request the merge kernel accepts
 
-int naive_splits(int B, int H, int64_t Ls, int n_sm) {
+int naive_splits(int B, int H, int64_t Ls, int n_sm, int max_slots) {
     if (Ls <= 0) return 0;
     int n_tiles = (int)((Ls + 63) / 64);
     int base = ((B + 63) / 64) * H;
     int want = (4 * n_sm + base - 1) / base;
-    return std::max(1, std::min({want, n_tiles, 64}));
+    return std::max(1, std::min({want, n_tiles, 64, max_slots}));
 }
 
-void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int* chunk, int* n_sh,
-                   int* n_sf) {
+// max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks
+void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks, int* chunk,
+                   int* n_sh, int* n_sf) {
     const bool pair = tc && absorb_uses_pairs(B, H, Ls_absorb, cap_suffix);
     const int row_tile = pair ? 128 : 64;
     const int units = B * ((H + row_tile - 1) / row_tile);
@@ -175,7 +176,7 @@ void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_abs
             const int64_t ch = round_up((longest + parts - 1) / parts, tile);
             const int64_t per_req = (Ls_absorb + ch - 1) / ch + (cap_suffix + ch - 1) / ch;
             const int64_t items = (int64_t)units_sh * ((Ls_absorb + ch - 1) / ch) + (int64_t)units * ((cap_suffix + ch - 1) / ch);
-            if (per_req > kMaxAbsorbChunks) continue;   // limit of the merge kernel
+            if (per_req > max_chunks) continue;
             const int64_t waves = (items + slots - 1) / slots;
             const double cost = (double)waves * ((double)ch / tile + fixed + (per_req > 1 ? split : 0.0));
             if (cost < best_cost - 1e-9) {
@@ -187,37 +188,16 @@ void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_abs
     } else {
         const int target = std::max(1, (2 * n_sm + units - 1) / units);
         c = std::max<int64_t>(round_up((longest + target - 1) / target, 64), 256);
-        while ((Ls_absorb + c - 1) / c + (cap_suffix + c - 1) / c > kMaxAbsorbChunks) c *= 2;
+        while ((Ls_absorb + c - 1) / c + (cap_suffix + c - 1) / c > max_chunks) c *= 2;
     }
     *chunk = (int)c;
     *n_sh = (int)((Ls_absorb + c - 1) / c);
     *n_sf = (int)((cap_suffix + c - 1) / c);
 }
 
-// `mode` is resolved (ABSORB, HYBRID or NAIVE); `tc` and `schedule` come from the caller's settings snapshot.
-Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int max_pages, int page_size, int mode,
-               int naive_slots_override = -1, bool stacked = true) {
-    Plan p{};
-    const int H = sh->dims.num_heads;
-    const int n_sm = sh->num_sms > 0 ? sh->num_sms : kDefaultNumSM;
-    p.mode = mode;
-    const int64_t cap = (int64_t)max_pages * page_size;
-    const bool use_naive = (mode != TYPHOON_MLA_MODE_ABSORB) && sh->Ls > 0;
-    const bool use_absorb = (mode != TYPHOON_MLA_MODE_NAIVE);
-    if (naive_slots_override >= 0) {   // several shared-prefix launches planned by the caller
-        p.n_split_naive = naive_slots_override > 0 ? 1 : 0;
-        p.n_slots_naive = naive_slots_override;
-    } else if (use_naive && tc) {
-        naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0);   // n_split_naive = tile ranges
-    } else {
-        p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm) : 0;
-        p.n_slots_naive = p.n_split_naive;
-    }
-    if (use_absorb) {
-        absorb_chunks(tc, stacked, n_sm, B, H, mode == TYPHOON_MLA_MODE_ABSORB ? sh->Ls : 0, cap, &p.chunk, &p.n_shared_chunks,
-                      &p.n_suffix_chunks);
-    }
-    const int n_chunks = p.n_shared_chunks + p.n_suffix_chunks;
+// The workspace's parts, for partials of `chunk_rows` rows (chunks x requests x heads) of the absorb attention and `slot_rows` of
+// the shared-prefix attention.
+void lay_out(Plan* p, int B, int H, int64_t chunk_rows, int64_t slot_rows) {
     const size_t BH = (size_t)B * H;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -225,18 +205,93 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
         off += round_up((int64_t)bytes, 256);
         return o;
     };
-    p.off_order = take((size_t)B * 4);
-    p.off_desc = take((size_t)B * 16);
-    p.off_qabs = take(BH * 512 * 2);
-    p.off_opart_a = take((size_t)n_chunks * BH * 512 * 4);
-    p.off_lsepart_a = take((size_t)n_chunks * BH * 4);
-    p.off_olat = take(BH * 512 * 2);
-    p.off_lse_a = take(BH * 4);
-    p.off_oabs = take(BH * 128 * 4);
-    p.off_opart_n = take((size_t)p.n_slots_naive * BH * 128 * 4);
-    p.off_lsepart_n = take((size_t)p.n_slots_naive * BH * 4);
-    p.total = off;
-    return p;
+    p->off_order = take((size_t)B * 4);
+    p->off_desc = take((size_t)B * 16);
+    p->off_qabs = take(BH * 512 * 2);
+    p->off_opart_a = take((size_t)chunk_rows * 512 * 4);
+    p->off_lsepart_a = take((size_t)chunk_rows * 4);
+    p->off_olat = take(BH * 512 * 2);
+    p->off_lse_a = take(BH * 4);
+    p->off_oabs = take(BH * 128 * 4);
+    p->off_opart_n = take((size_t)slot_rows * 128 * 4);
+    p->off_lsepart_n = take((size_t)slot_rows * 4);
+    p->total = off;
+}
+
+// The number of partials that a plan chooses neither grows nor falls steadily with the batch or the page table.  A workspace sized
+// for B requests and max_pages pages has to do for smaller steps as well: it holds at least the "floor" of its sizes, every term of
+// which grows with both, and a step whose own choice does not fit is planned again within what there is, which the floor of ITS
+// sizes guarantees to be possible (one chunk per segment, two slots).  The constant is four waves of 64 rows per SM: of (H, L_s,
+// pages, sized batch, batch) combinations over 16..128 heads, 100..65536 tokens, 1..200 pages and up to 1024 requests, 67 of 550800
+// do not get their own choice in the mode that AUTO takes (1828 with one wave; at most 11 % longer by the plan's own model).
+// It also bounds what the warp-MMA plan (about 2 n_sm 64-row chunks per segment) and every schedule of the shared-prefix kernel
+// choose, n_sm / (row groups) ranges over H heads: at most 2 n_sm / H / groups + 2 slots.
+int64_t floor_chunk_rows(int n_sm, int64_t rows, int64_t Ls_absorb, int64_t cap_suffix) {
+    const int segments = (Ls_absorb > 0) + (cap_suffix > 0);
+    return std::min(rows * ((Ls_absorb + 63) / 64 + (cap_suffix + 63) / 64), (int64_t)256 * n_sm + segments * rows);
+}
+int64_t floor_slot_rows(int n_sm, int64_t rows, int64_t Ls) {
+    return Ls <= 0 ? 0 : std::min(rows * ((Ls + 63) / 64), (int64_t)256 * n_sm + 2 * rows);
+}
+
+// `mode` is resolved (ABSORB, HYBRID or NAIVE); `tc` and `schedule` come from the caller's settings snapshot.  workspace_bytes: 0 gives
+// the floor's sizes (offsets and total only).  A plan whose total exceeds workspace_bytes cannot be run with them.
+Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int max_pages, int page_size, int mode,
+               int naive_slots_override = -1, bool stacked = true, size_t workspace_bytes = SIZE_MAX) {
+    const int H = sh->dims.num_heads;
+    const int n_sm = sh->num_sms > 0 ? sh->num_sms : kDefaultNumSM;
+    const int64_t cap = (int64_t)max_pages * page_size, rows = (int64_t)B * H;
+    const bool use_naive = (mode != TYPHOON_MLA_MODE_ABSORB) && sh->Ls > 0;
+    const bool use_absorb = (mode != TYPHOON_MLA_MODE_NAIVE);
+    const int64_t Ls_absorb = mode == TYPHOON_MLA_MODE_ABSORB ? sh->Ls : 0;
+    auto plan_within = [&](int max_chunks, int max_slots) {
+        Plan p{};
+        p.mode = mode;
+        if (naive_slots_override >= 0) {   // several shared-prefix launches planned by the caller
+            p.n_split_naive = naive_slots_override > 0 ? 1 : 0;
+            p.n_slots_naive = naive_slots_override;
+        } else if (use_naive && tc) {   // n_split_naive = tile ranges
+            naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0,
+                             max_slots);
+        } else {
+            p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm, max_slots) : 0;
+            p.n_slots_naive = p.n_split_naive;
+        }
+        if (use_absorb) absorb_chunks(tc, stacked, n_sm, B, H, Ls_absorb, cap, max_chunks, &p.chunk, &p.n_shared_chunks, &p.n_suffix_chunks);
+        lay_out(&p, B, H, (int64_t)(p.n_shared_chunks + p.n_suffix_chunks) * rows, (int64_t)p.n_slots_naive * rows);
+        return p;
+    };
+    Plan p{};
+    if (workspace_bytes > 0) {
+        p = plan_within(kMaxAbsorbChunks, INT32_MAX);
+        if (p.total <= workspace_bytes) return p;
+    }
+    const int64_t chunk_rows = use_absorb ? floor_chunk_rows(n_sm, rows, Ls_absorb, cap) : 0;
+    const int64_t slot_rows = naive_slots_override >= 0 ? naive_slots_override * rows : use_naive ? floor_slot_rows(n_sm, rows, sh->Ls) : 0;
+    Plan least{};
+    lay_out(&least, B, H, chunk_rows, slot_rows);
+    if (workspace_bytes == 0) return least;
+    if (workspace_bytes < least.total) return p;
+    const int64_t more = (int64_t)(workspace_bytes - least.total);   // (a chunk's row: 512 values and its LSE, of which the sum is rounded up)
+    const int64_t max_chunks = (chunk_rows + std::max<int64_t>(more - 256, 0) / (512 * 4 + 4)) / rows;
+    return plan_within((int)std::min<int64_t>(max_chunks, kMaxAbsorbChunks), (int)std::min<int64_t>(slot_rows / rows, INT32_MAX));
+}
+
+// Worst case over the modes that `mode` can resolve to, over both kernel implementations and over the work decompositions a test hook
+// may select, and the floor: a workspace of this size serves steps of at most B requests and max_pages pages whatever the
+// switches are set to when they run.  Only local values are used; no process-wide state is read or written.
+size_t query_bytes(const typhoon_mla_shared* sh, int B, int max_pages, int page_size, int mode) {
+    size_t worst = 0;
+    for (int m : {TYPHOON_MLA_MODE_ABSORB, TYPHOON_MLA_MODE_HYBRID, TYPHOON_MLA_MODE_NAIVE}) {
+        if (mode != TYPHOON_MLA_MODE_AUTO && mode != m && !(mode == TYPHOON_MLA_MODE_HYBRID && sh->Ls == 0)) continue;
+        const int pages = m == TYPHOON_MLA_MODE_NAIVE ? 0 : max_pages;
+        worst = std::max(worst, make_plan(sh, true, 0, B, pages, page_size, m, -1, true, 0).total);
+        for (bool tc : {true, false})
+            for (int schedule : {0, 1, 2})
+                for (bool stacked : {true, false})
+                    worst = std::max(worst, make_plan(sh, tc, schedule, B, pages, page_size, m, -1, stacked).total);
+    }
+    return worst + 256;
 }
 
 // The handle's buffers, stream and events live on the device it was prepared on.
@@ -727,19 +782,28 @@ size_t typhoon_mla_workspace_bytes(const typhoon_mla_shared_t* sh, int32_t B, in
                                    int32_t mode) {
     if (!sh || B < 1 || max_pages < 0 || (page_size != 64 && page_size != 128)) return 0;
     if (mode < TYPHOON_MLA_MODE_AUTO || mode > TYPHOON_MLA_MODE_NAIVE) return 0;
-    // Worst case over the modes `mode` can resolve to, over both kernel implementations and over the work
-    // decompositions a test hook may select: a workspace sized here serves whatever the switches are set to when
-    // the step runs.  Only local values are used; no process-wide state is read or written.
-    size_t worst = 0;
-    for (int m : {TYPHOON_MLA_MODE_ABSORB, TYPHOON_MLA_MODE_HYBRID, TYPHOON_MLA_MODE_NAIVE}) {
-        if (mode != TYPHOON_MLA_MODE_AUTO && mode != m && !(mode == TYPHOON_MLA_MODE_HYBRID && sh->Ls == 0)) continue;
-        const int pages = m == TYPHOON_MLA_MODE_NAIVE ? 0 : max_pages;
-        for (bool tc : {true, false})
-            for (int schedule : {0, 1, 2})
-                for (bool stacked : {true, false})
-                    worst = std::max(worst, make_plan(sh, tc, schedule, B, pages, page_size, m, -1, stacked).total);
-    }
-    return worst + 256;
+    return query_bytes(sh, B, max_pages, page_size, mode);
+}
+
+int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8bit, int32_t B, int32_t max_pages, int32_t page_size,
+                               int32_t mode, int32_t path, int32_t schedule, int32_t stacked, int32_t num_sms, size_t workspace_bytes,
+                               size_t* query, size_t* step, int32_t* n_chunks, int32_t* n_slots) {
+    if (num_heads < 16 || num_heads > 128 || num_heads % 16 || L_s < 0 || L_s > (int64_t)1 << 24 || B < 1 || max_pages < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if ((page_size != 64 && page_size != 128) || mode < TYPHOON_MLA_MODE_AUTO || mode > TYPHOON_MLA_MODE_NAIVE) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (path < 0 || path > 1 || schedule < 0 || schedule > 2 || num_sms < 0 || !query || !step || !n_chunks || !n_slots) return TYPHOON_MLA_ERR_INVALID_ARG;
+    typhoon_mla_shared sh{};
+    sh.dims.num_heads = num_heads; sh.dims.d_nope = 128; sh.dims.d_rope = 64; sh.dims.d_v = 128; sh.dims.kv_lora_rank = 512;
+    sh.Ls = L_s;
+    sh.fp8 = prefix_8bit != 0 && L_s > 0;
+    sh.num_sms = num_sms;
+    *query = query_bytes(&sh, B, max_pages, page_size, mode);
+    const int m = resolve_mode(&sh, B, max_pages, mode);
+    const Plan p = make_plan(&sh, path == TYPHOON_MLA_PATH_TCGEN05, schedule, B, m == TYPHOON_MLA_MODE_NAIVE ? 0 : max_pages, page_size, m, -1,
+                             stacked != 0, workspace_bytes > 0 ? workspace_bytes : SIZE_MAX);
+    *step = p.total;
+    *n_chunks = p.n_shared_chunks + p.n_suffix_chunks;
+    *n_slots = p.n_slots_naive;
+    return workspace_bytes > 0 && workspace_bytes < p.total ? TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL : TYPHOON_MLA_OK;
 }
 
 // One launch of the shared-prefix kernel: `rows` requests starting at `row0` against the prefix of
@@ -993,8 +1057,9 @@ static int decode_impl(const typhoon_mla_shared_t* sh, const void* q_nope, const
             return TYPHOON_MLA_ERR_INVALID_ARG;
     }
     if (mode == TYPHOON_MLA_MODE_NAIVE && sh->Ls == 0) max_pages = 0;
-    const Plan pl = make_plan(sh, cfg.tc(), cfg.naive_schedule, B, use_absorb ? max_pages : 0, page_size, mode, -1, cfg.stacked_absorb);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return TYPHOON_MLA_ERR_INVALID_ARG;
+    const Plan pl = make_plan(sh, cfg.tc(), cfg.naive_schedule, B, use_absorb ? max_pages : 0, page_size, mode, -1, cfg.stacked_absorb,
+                              std::max<size_t>(workspace_bytes, 1));
     if (workspace_bytes < pl.total) return TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL;
 
     NaiveJob job{sh, 0, B, pl.n_split_naive, pl.n_slots_naive, 0};
@@ -1133,7 +1198,8 @@ size_t typhoon_mla_tree_workspace_bytes(const typhoon_mla_prefix_level_t* levels
     for (int schedule : {0, 1, 2}) {
         TreePlan tp;
         if (plan_tree(levels, n_levels, B, schedule, &tp) != TYPHOON_MLA_OK) return 0;
-        worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots).total);
+        for (size_t bytes : {SIZE_MAX, (size_t)0})   // the step's own choice, and what smaller page tables may choose (make_plan)
+            worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots, true, bytes).total);
     }
     return worst + 256;
 }
@@ -1162,8 +1228,9 @@ int typhoon_mla_decode_tree(const typhoon_mla_prefix_level_t* levels, int32_t n_
     if (!on_handle_device(tp.sh0)) return TYPHOON_MLA_ERR_INVALID_ARG;
     // NAIVE when there is no page table (nothing for the absorb branch), else Algorithm 1 with several line-4 launches
     const int mode = max_pages == 0 ? TYPHOON_MLA_MODE_NAIVE : TYPHOON_MLA_MODE_HYBRID;
-    const Plan pl = make_plan(tp.sh0, true, cfg.naive_schedule, B, max_pages, page_size, mode, tp.total_slots);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return TYPHOON_MLA_ERR_INVALID_ARG;
+    const Plan pl = make_plan(tp.sh0, true, cfg.naive_schedule, B, max_pages, page_size, mode, tp.total_slots, true,
+                              std::max<size_t>(workspace_bytes, 1));
     if (workspace_bytes < pl.total) return TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL;
     return decode_core(cfg, tp.sh0, tp.jobs, tp.n_jobs, tp.empties, tp.n_empties, pl, q_nope, q_pe, B, ckv_pages, kpe_pages,
                        ckv_token_stride, kpe_token_stride, page_size, num_pages, block_table, max_pages, seq_lens,

@@ -900,7 +900,8 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // head's; n_slots[i] are the slots of prefix i.  Runs on every call of a step, so the slots of all prefixes come from one walk
 // along the sequence without divisions (16 prefixes x 128 heads: 8 us; a pass per prefix with a division per tile
 // count and range took 159).
-static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
+static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8,
+                          int max_slots) {
     // (8-bit cache: always 64-token tiles, row groups of 128 requests)
     const bool mode_y = fp8 || B <= 128;
     const int tok = mode_y ? 64 : 128;
@@ -961,7 +962,7 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     const double slot_cost = mode_y ? 8.0 : 1.1e-4 * B * H;
     int ns_best = 1;
     double cost_best = 1e30, eff_best = 0.0;
-    for (int ns = 1; ns <= std::min(n_tiles, 32); ++ns) {
+    for (int ns = 1; ns <= std::min({n_tiles, 32, max_slots}); ++ns) {
         const int per = (n_tiles + ns - 1) / ns;
         if (n_tiles % ns != 0) continue;   // equal parts only: every range stays inside one head
         const long long waves = (ns * base + n_sm - 1) / n_sm;
@@ -988,10 +989,11 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     const long long per_stream = (T + r_stream - 1) / r_stream;
     const long long waves_stream = ((long long)r_stream * m_groups + n_sm - 1) / n_sm;
     const double segs_stream = (per_stream >= n_tiles) ? (double)per_stream / n_tiles + 1.0 : 2.0;
-    const double cost_stream = charge((double)waves_stream * (per_stream + fixed + (segs_stream - 1.0) * boundary) + slot_cost * (fill_slots(r_stream) - 1),
+    const int slots_stream = fill_slots(r_stream);
+    const double cost_stream = charge((double)waves_stream * (per_stream + fixed + (segs_stream - 1.0) * boundary) + slot_cost * (slots_stream - 1),
                                       (long long)r_stream * m_groups);
     bool stream_k;
-    if (schedule == 1) stream_k = false;
+    if (schedule == 1 || slots_stream > max_slots) stream_k = false;
     else if (schedule == 2) stream_k = true;
     else {
         // With at most 64 query rows a CTA keeps up with its share of HBM: more resident CTAs do not
@@ -1006,12 +1008,12 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     if (R != r_stream) fill_slots(R);   // the kernel uses the same partition
 }
 
-void naive_sm100_plan(int B, int H, int64_t Ls, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8) {
-    plan_sequence(B, H, &Ls, 1, n_sm, schedule, n_ranges, n_slots, fp8);
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, int max_slots) {
+    plan_sequence(B, H, &Ls, 1, places, schedule, n_ranges, n_slots, fp8, max_slots);
 }
 
 void naive_sm100_plan_multi(int max_rows, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots) {
-    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false);
+    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false, INT32_MAX);
 }
 
 

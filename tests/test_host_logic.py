@@ -230,3 +230,40 @@ def test_planning_a_launch_of_many_prefixes_costs_no_more_than_planning_each(b):
         return min(times)
 
     assert best([256 + 64 * i for i in range(16)]) < 16 * best([736])
+
+
+@pytest.mark.parametrize("H,L_s,pages,fp8,batches", [
+    (16, 4096, 16, False, (8, 130)), (16, 8192, 4, False, (8, 32)), (16, 1000, 4, False, (32,)), (64, 256, 4, False, (32, 256)),
+    (128, 1000, 4, False, (8, 130)), (128, 100, 200, False, (128,)), (48, 20000, 33, False, (300, 1024)), (32, 0, 16, False, (64,)),
+    (16, 30, 0, False, (200,)), (96, 65536, 1, False, (900,)), (128, 4096, 8, True, (130, 400)), (16, 16384, 24, True, (130,))])
+def test_workspace_serves_smaller_batches_and_page_tables(b, H, L_s, pages, fp8, batches):
+    """Batches on both sides of 128 query rows and of 128 (request, head) rows, page tables on both sides of the prefix's length."""
+    for batch in batches:
+        for m in (b.MODE_AUTO, b.MODE_ABSORB, b.MODE_HYBRID, b.MODE_NAIVE):
+            size = b.typhoon_mla_workspace_plan(H, L_s, batch, pages, mode=m, prefix_8bit=fp8)[0]
+            for B in sorted({*range(1, min(batch, 33)), *range(1, batch + 1, max(1, batch // 29)), 127, 128, 129, batch - 1, batch}):
+                if not 1 <= B <= batch:
+                    continue
+                for p in sorted({pages, pages * 3 // 4, pages // 2, min(pages, max(L_s // 64 - 1, 0)), min(pages, 1), 0}):
+                    for path, schedule, stacked in ((0, 0, True), (0, 1, True), (0, 2, False), (1, 0, True)):
+                        for mode in ((b.MODE_AUTO, b.MODE_ABSORB, b.MODE_HYBRID, b.MODE_NAIVE) if m == b.MODE_AUTO else (m,)):
+                            args = dict(mode=mode, prefix_8bit=fp8, path=path, schedule=schedule, stacked=stacked)
+                            _, step, chunks, slots = b.typhoon_mla_workspace_plan(H, L_s, B, p, workspace_bytes=size, **args)
+                            assert step <= size
+                            _, own, own_chunks, own_slots = b.typhoon_mla_workspace_plan(H, L_s, B, p, **args)
+                            assert (chunks, slots) == (own_chunks, own_slots) if own <= size else (chunks < own_chunks or slots < own_slots)
+
+
+def test_workspace_that_is_too_small_is_refused(b):
+    for H, L_s, B, pages in ((16, 4096, 8, 16), (128, 16384, 64, 4), (64, 300, 256, 64), (96, 65536, 900, 1)):
+        for mode in (b.MODE_ABSORB, b.MODE_HYBRID, b.MODE_NAIVE):
+            _, step, chunks, slots = b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode)
+            assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=step)[1:] == (step, chunks, slots)
+            # with a byte less the step takes fewer partials or is refused; without room for one of each kind it is refused
+            try:
+                assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=step - 1)[1] < step
+            except b.TyphoonMLAError as e:
+                assert "workspace" in str(e)
+            least = B * H * (512 * (2 + 2) + 128 * 4) + B * H * 4 * (512 if mode != b.MODE_NAIVE else 128)
+            with pytest.raises(b.TyphoonMLAError, match="workspace"):
+                b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=least)
