@@ -20,7 +20,8 @@ extern "C" {
 /* Work decomposition the tcgen05 shared-prefix kernel (Algorithm 1 line 4) would use for a problem
  * size on a GPU with `num_sms` multiprocessors (0: 148, a B200): tokens per KV tile (64 for B <= 128,
  * else 128), number of contiguous tile ranges the H * n_tiles tiles are cut into, query-row groups
- * per range (CTAs = ranges * row_groups) and partial slots written per (request, head).  schedule:
+ * per range (B <= 128: one; else of 256 rows, each worked on by a pair of CTAs, so that CTAs =
+ * 2 * ranges * row_groups) and partial slots written per (request, head).  schedule:
  * 0 = the library's choice, 1 = every range inside one head ("column split"), 2 = ranges of equal
  * size over all heads ("stream-K").  Host, pure (a function of the sizes only, so the decomposition
  * and with it the summation order are reproducible).  INVALID_ARG for B < 1, L_s < 1, unsupported H

@@ -342,7 +342,7 @@ int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t sc
     if (num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (!tile_tokens || !n_ranges || !row_groups || !n_slots) return TYPHOON_MLA_ERR_INVALID_ARG;
     int r = 0, sl = 0;
-    naive_sm100_plan(B, num_heads, L_s, num_sms > 0 ? num_sms : kDefaultNumSM, schedule, &r, &sl);
+    naive_sm100_plan(B, num_heads, L_s, naive_places(B, num_sms > 0 ? num_sms : kDefaultNumSM, false), schedule, &r, &sl);
     *tile_tokens = naive_sm100_tile_tokens(B);
     *n_ranges = r;
     *row_groups = B <= 128 ? 1 : (B + 255) / 256;

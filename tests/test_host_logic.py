@@ -162,11 +162,16 @@ def test_naive_plan_invariants(b):
             if schedule == 1:
                 assert R % H == 0 and n_tiles % (R // H) == 0 and seg_max == R // H
             if schedule == 2:
-                assert R == min(max(1, 148 // groups), T)
-    # benchmark configs: config 1 one range per head; config 2 and config 4 at B = 512 one CTA per SM
+                assert R == min(max(1, (148 if B <= 128 else 74) // groups), T)   # one range per SM, or per pair of SMs
+            if schedule == 0 and B > 128:
+                assert R % H == 0 or H % R == 0 or R == min(max(1, 74 // groups), T)
+    # benchmark configs: config 1 one range per head; config 2 one CTA per SM; config 4 at B = 512 one CTA pair per pair of SMs
     assert b.typhoon_mla_naive_plan(128, 64, 4096)[1:] == (128, 1, 1)
     assert b.typhoon_mla_naive_plan(128, 128, 26624)[1] == 148
-    assert b.typhoon_mla_naive_plan(128, 512, 16384)[1:3] == (74, 2)
+    assert b.typhoon_mla_naive_plan(128, 512, 16384)[1:3] == (37, 2)
+    # what a step launches and sizes its partials for
+    for H, B, Ls in ((128, 512, 16384), (64, 256, 8192), (16, 166, 7069), (32, 700, 2048), (128, 64, 4096), (16, 129, 1)):
+        assert b.typhoon_mla_naive_plan(H, B, Ls)[3] == b.typhoon_mla_workspace_plan(H, Ls, B, 4, mode=b.MODE_HYBRID)[3]
     # every further partial slot is charged with 64-token tiles: shapes where equal ranges over all heads would
     # need three or more slots per head keep one or two ranges per head (measured to be the faster choice)
     assert b.typhoon_mla_naive_plan(128, 128, 16384)[1:] == (128, 1, 1)
