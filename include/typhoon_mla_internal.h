@@ -37,13 +37,15 @@ int typhoon_mla_naive_plan_multi(int32_t num_heads, int32_t max_rows, const int6
 
 /* Workspace planning without a handle, on a GPU with `num_sms` multiprocessors (0: 148): `query` = what typhoon_mla_workspace_bytes
  * returns for a prefix of L_s tokens, B requests, page-table width max_pages and `mode`; `step`, `n_chunks` (absorb partials per
- * row) and `n_slots` (shared-prefix partials per row) = the bytes and partials of the plan that typhoon_mla_decode takes with a
- * workspace of `workspace_bytes` (0: unlimited), with the given kernel path, schedule and stacked-absorb switch.  Host; reads the
+ * row), `n_slots` (shared-prefix partials per row) and `absorb_pairs` (1: the absorb attention takes 128 query rows per pair of
+ * CTAs, 0: 64 per CTA) = bytes, partials and kernel of the plan that typhoon_mla_decode takes with a workspace
+ * of `workspace_bytes` (0: unlimited), with the given kernel path, schedule and stacked-absorb switch.  Host; reads the
  * crossover rule's model (AUTO) and nothing else.  WORKSPACE_TOO_SMALL where decode returns it (the outputs are written),
  * INVALID_ARG for arguments outside the ranges above. */
 int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8bit, int32_t B, int32_t max_pages, int32_t page_size,
                                int32_t mode, int32_t path, int32_t schedule, int32_t stacked, int32_t num_sms, size_t workspace_bytes,
-                               size_t* query /* host */, size_t* step /* host */, int32_t* n_chunks /* host */, int32_t* n_slots /* host */);
+                               size_t* query /* host */, size_t* step /* host */, int32_t* n_chunks /* host */, int32_t* n_slots /* host */,
+                               int32_t* absorb_pairs /* host */);
 
 /* How the tcgen05 output projection (Algorithm 1 lines 7 and 8) of B requests with `n_slots` partial slots, of which some
  * come from a prefix with 8-bit storage (or none), is cut on a GPU with `num_sms` multiprocessors (0: 148): items of one head, 128 requests and `columns` output columns, the CTAs they run

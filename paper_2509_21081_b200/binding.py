@@ -61,7 +61,7 @@ def _load():
     lib.typhoon_mla_naive_plan_multi.restype = C.c_int
     lib.typhoon_mla_naive_plan_multi.argtypes = [i32, i32, C.POINTER(i64), i32, i32, i32, C.POINTER(i32), C.POINTER(i32)]
     lib.typhoon_mla_workspace_plan.restype = C.c_int
-    lib.typhoon_mla_workspace_plan.argtypes = [i32, i64] + [i32] * 9 + [sz, C.POINTER(sz), C.POINTER(sz), C.POINTER(i32), C.POINTER(i32)]
+    lib.typhoon_mla_workspace_plan.argtypes = [i32, i64] + [i32] * 9 + [sz, C.POINTER(sz), C.POINTER(sz)] + [C.POINTER(i32)] * 3
     lib.typhoon_mla_project_plan.restype = C.c_int
     lib.typhoon_mla_project_plan.argtypes = [i32, i32, i32, i32, i32] + [C.POINTER(i32)] * 4
     lib.typhoon_mla_release_cached.restype = C.c_int
@@ -383,12 +383,12 @@ def typhoon_mla_naive_plan_multi(num_heads: int, max_rows: int, L_s, schedule: i
 def typhoon_mla_workspace_plan(num_heads: int, L_s: int, B: int, max_pages: int, page_size: int = 64, mode: int = MODE_AUTO,
                                workspace_bytes: int = 0, prefix_8bit: bool = False, path: int = 0, schedule: int = 0,
                                stacked: bool = True, num_sms: int = 0):
-    """(size query, bytes of a step's plan, absorb chunks, prefix slots); raises where a step with `workspace_bytes` would."""
-    q, s, c, n = C.c_size_t(), C.c_size_t(), C.c_int32(), C.c_int32()
+    """(size query, bytes of a step's plan, absorb chunks, prefix slots, absorb kernel takes CTA pairs); raises where a step with
+    `workspace_bytes` would."""
+    out = [C.c_size_t(), C.c_size_t(), C.c_int32(), C.c_int32(), C.c_int32()]
     _check(_lib.typhoon_mla_workspace_plan(num_heads, L_s, int(prefix_8bit), B, max_pages, page_size, mode, path, schedule, int(stacked),
-                                           num_sms, workspace_bytes, C.byref(q), C.byref(s), C.byref(c), C.byref(n)),
-           "typhoon_mla_workspace_plan")
-    return q.value, s.value, c.value, n.value
+                                           num_sms, workspace_bytes, *[C.byref(x) for x in out]), "typhoon_mla_workspace_plan")
+    return tuple(x.value for x in out)
 
 
 def typhoon_mla_project_plan(num_heads: int, B: int, n_slots: int, prefix_8bit: bool = False, num_sms: int = 0):

@@ -137,6 +137,7 @@ struct Plan {
     int mode;
     int n_split_naive;       // KV splits of the warp-MMA naive kernel / tile ranges of the tcgen05 one
     int n_slots_naive;       // partial slots the naive kernel writes (>= n_split_naive)
+    bool absorb_pairs;       // absorb attention by the kernel of 128 rows per CTA pair
     int chunk;               // tokens per absorb chunk
     int n_shared_chunks;     // absorb chunks over the shared prefix (ABSORB mode)
     int n_suffix_chunks;
@@ -155,23 +156,20 @@ int naive_splits(int B, int H, int64_t Ls, int n_sm, int max_slots) {
     return std::max(1, std::min({want, n_tiles, 64, max_slots}));
 }
 
-// max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks
-void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks, int* chunk,
-                   int* n_sh, int* n_sf) {
-    const bool pair = tc && absorb_uses_pairs(B, H, Ls_absorb, cap_suffix);
-    const int row_tile = pair ? 128 : 64;
-    const int units = B * ((H + row_tile - 1) / row_tile);
-    // work items per shared-prefix chunk: row groups of the stacked [B * H] query matrix, or of each request
-    const int units_sh = (tc && stacked) ? (int)(((int64_t)B * H + row_tile - 1) / row_tile) : units;
+// Kernel and chunk length of the absorb attention.  max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks.
+void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks,
+                   bool* pairs, int* chunk, int* n_sh, int* n_sf) {
     const int64_t longest = std::max<int64_t>(std::max(Ls_absorb, cap_suffix), 1);
-    int64_t c;
-    if (tc) {
-        // One CTA (pair) per SM (pair of SMs): minimise waves x (tiles per chunk + fixed cost in tile units) over the number of
-        // chunks the longest segment is cut into.  A split segment writes and re-reads fp32 partials, 2 KB per row both ways.
-        const int tile = pair ? 128 : 64, slots = pair ? n_sm / 2 : n_sm;
+    // One CTA (pair) per SM (pair of SMs): minimise waves x (tiles per chunk + fixed cost in tile units) over the number of
+    // chunks the longest segment is cut into.  A split segment writes and re-reads fp32 partials, 2 KB per row both ways.
+    auto cut = [&](bool pair) {
+        const int tile = pair ? 128 : 64, slots = pair ? n_sm / 2 : n_sm;   // (tile: tokens, and rows of an item)
         const double fixed = pair ? 4.0 : 3.0, split = pair ? 3.0 : 3.5;
+        // items per chunk of a suffix; of the prefix, cut from the stacked [B * H] query matrix or from each request's rows
+        const int units = B * ((H + tile - 1) / tile);
+        const int units_sh = stacked ? (int)(((int64_t)B * H + tile - 1) / tile) : units;
         double best_cost = 1e30;
-        c = round_up(longest, tile);
+        int64_t c = round_up(longest, tile);
         for (int parts = 1; parts <= 512; ++parts) {
             const int64_t ch = round_up((longest + parts - 1) / parts, tile);
             const int64_t per_req = (Ls_absorb + ch - 1) / ch + (cap_suffix + ch - 1) / ch;
@@ -185,7 +183,41 @@ void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_abs
             }
             if (ch <= tile) break;
         }
+        return c;
+    };
+    // Estimate of the kernel's time with chunks of `c` tokens, in SM clocks: the items' work spread over all places and half an item more.
+    // (2580 and 2416 clocks per tile, as measured in the two kernels.)
+    auto clocks = [&](bool pair, int64_t c) {
+        const int tile = pair ? 128 : 64;
+        const double n_sh = (double)((Ls_absorb + c - 1) / c), n_sf = (double)((cap_suffix + c - 1) / c);
+        const double extra = (pair ? 6.0 : 5.0) + (n_sh + n_sf > 1 ? (pair ? 3.0 : 3.5) : 0.0);
+        const double t_sh = (double)std::min(c, Ls_absorb) / tile + extra, t_sf = (double)((std::min(c, cap_suffix) + tile - 1) / tile) + extra;
+        const double items_sh = (double)(((int64_t)B * H + tile - 1) / tile) * n_sh, items_sf = (double)B * ((H + tile - 1) / tile) * n_sf;
+        const double longest_item = n_sh > 0 ? t_sh : t_sf;
+        const double tiles = std::max(longest_item, (items_sh * t_sh + items_sf * t_sf) / (pair ? n_sm / 2 : n_sm) + 0.5 * longest_item);
+        return tiles * (pair ? 2416.0 : 2580.0);
+    };
+    int64_t c;
+    *pairs = false;
+    if (tc && H > 64) {
+        *pairs = true;
+        c = cut(true);
+    } else if (tc) {
+        // Up to 64 heads the pair kernel is for the prefix of an absorb-only step, whose rows are stacked and fill its 128; a suffix item
+        // has rows of nobody and still takes two SMs.  (B200, us per step, 64-row / pair: 64 heads, 12 requests, 22865 + 567 tokens
+        // 71.9 / 51.5; 32 heads, 31, 4399 + 389 35.1 / 30.4; 16 heads, 60, 1426 + 39 28.0 / 33.8; 48 heads, 67, 131 + 11 27.0 / 35.3;
+        // 32 heads, 185, 3378 + 17 110 / 134.  Over 184 such steps this choice is on average 0.5 % behind the better of the two, and in
+        // four more than 3 % behind the 64-row kernel; pairs throughout 3.6 % and 42, comparing the costs above 1.0 % and 16.)
+        c = cut(false);
+        if (stacked && (int64_t)B * H >= 128 && Ls_absorb > 0 && Ls_absorb >= cap_suffix) {
+            const int64_t c_pair = cut(true);
+            if (clocks(true, c_pair) < 0.95 * clocks(false, c)) {
+                *pairs = true;
+                c = c_pair;
+            }
+        }
     } else {
+        const int units = B * ((H + 63) / 64);
         const int target = std::max(1, (2 * n_sm + units - 1) / units);
         c = std::max<int64_t>(round_up((longest + target - 1) / target, 64), 256);
         while ((Ls_absorb + c - 1) / c + (cap_suffix + c - 1) / c > max_chunks) c *= 2;
@@ -257,7 +289,9 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
             p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm, max_slots) : 0;
             p.n_slots_naive = p.n_split_naive;
         }
-        if (use_absorb) absorb_chunks(tc, stacked, n_sm, B, H, Ls_absorb, cap, max_chunks, &p.chunk, &p.n_shared_chunks, &p.n_suffix_chunks);
+        if (use_absorb)
+            absorb_chunks(tc, stacked, n_sm, B, H, Ls_absorb, cap, max_chunks, &p.absorb_pairs, &p.chunk,
+                          &p.n_shared_chunks, &p.n_suffix_chunks);
         lay_out(&p, B, H, (int64_t)(p.n_shared_chunks + p.n_suffix_chunks) * rows, (int64_t)p.n_slots_naive * rows);
         return p;
     };
@@ -787,10 +821,11 @@ size_t typhoon_mla_workspace_bytes(const typhoon_mla_shared_t* sh, int32_t B, in
 
 int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8bit, int32_t B, int32_t max_pages, int32_t page_size,
                                int32_t mode, int32_t path, int32_t schedule, int32_t stacked, int32_t num_sms, size_t workspace_bytes,
-                               size_t* query, size_t* step, int32_t* n_chunks, int32_t* n_slots) {
+                               size_t* query, size_t* step, int32_t* n_chunks, int32_t* n_slots, int32_t* absorb_pairs) {
     if (num_heads < 16 || num_heads > 128 || num_heads % 16 || L_s < 0 || L_s > (int64_t)1 << 24 || B < 1 || max_pages < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
     if ((page_size != 64 && page_size != 128) || mode < TYPHOON_MLA_MODE_AUTO || mode > TYPHOON_MLA_MODE_NAIVE) return TYPHOON_MLA_ERR_INVALID_ARG;
-    if (path < 0 || path > 1 || schedule < 0 || schedule > 2 || num_sms < 0 || !query || !step || !n_chunks || !n_slots) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (path < 0 || path > 1 || schedule < 0 || schedule > 2 || num_sms < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (!query || !step || !n_chunks || !n_slots || !absorb_pairs) return TYPHOON_MLA_ERR_INVALID_ARG;
     typhoon_mla_shared sh{};
     sh.dims.num_heads = num_heads; sh.dims.d_nope = 128; sh.dims.d_rope = 64; sh.dims.d_v = 128; sh.dims.kv_lora_rank = 512;
     sh.Ls = L_s;
@@ -803,6 +838,7 @@ int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8b
     *step = p.total;
     *n_chunks = p.n_shared_chunks + p.n_suffix_chunks;
     *n_slots = p.n_slots_naive;
+    *absorb_pairs = p.absorb_pairs ? 1 : 0;
     return workspace_bytes > 0 && workspace_bytes < p.total ? TYPHOON_MLA_ERR_WORKSPACE_TOO_SMALL : TYPHOON_MLA_OK;
 }
 
@@ -969,9 +1005,9 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                       seq_lens, order, desc, B, H, pl.chunk, pl.n_shared_chunks, pl.n_suffix_chunks, softmax_scale,
                       o_part_a, lse_part_a, sh->status, forked ? nullptr : sh->w_uv, cfg.stacked_absorb};
         prof_before(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
-        e = !tc ? launch_absorb_attn_mma(ab, s)
-            : absorb_uses_pairs(B, H, ab.Ls_absorb, (int64_t)max_pages * page_size) ? launch_absorb_pair_sm100(ab, sh->Ls_pad, o_lat, lse_a, sh->status, s)
-                                   : launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s);
+        if (!tc) e = launch_absorb_attn_mma(ab, s);
+        else if (pl.absorb_pairs) e = launch_absorb_pair_sm100(ab, sh->Ls_pad, o_lat, lse_a, sh->status, s);
+        else e = launch_absorb_attn_sm100(ab, &sh->tm_ckv, &sh->tm_kpe_tok, o_lat, lse_a, sh->status, s);
         prof_after(TYPHOON_MLA_KERNEL_ABSORB_ATTN, s);
         if (e != cudaSuccess) return fail(e);
         ++launches;

@@ -201,14 +201,7 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
 cudaError_t make_absorb_shared_tmaps(const void* ckv, const void* kpe, int64_t Ls_pad, CUtensorMap* tm_ckv,
                                      CUtensorMap* tm_kpe);
 
-// The same for 128 query rows per pair of CTAs (chunk must be a multiple of 128).
-// ... which also takes absorb-only steps of fewer heads with at least 128 (request, head) rows, if the prefix is no shorter than the
-// longest suffix: the prefix's rows are stacked and fill the pair, while a suffix item has rows of nobody (it costs as much as in the
-// 64-row kernel).  B200, us per step, 64-row kernel / pairs: 64 heads, 16 requests over 16384 tokens 68.5 / 48.3, 28 over 8192 66.9 /
-// 51.9; 16 heads, 16 requests over 16384 35.6 / 31.1.  Beside a shared-prefix kernel it loses (64 heads, 100 requests 81 / 96).
-inline bool absorb_uses_pairs(int B, int H, int64_t Ls_absorb, int64_t cap_suffix) {
-    return H > 64 || ((int64_t)B * H >= 128 && Ls_absorb > 0 && Ls_absorb >= cap_suffix);
-}
+// The same for 128 query rows per pair of CTAs and at most 128 heads (chunk must be a multiple of 128).
 cudaError_t launch_absorb_pair_sm100(const AbsorbAttn& a, int64_t Ls_pad, void* o_lat_direct, float* lse_direct, int* status,
                                      cudaStream_t s);
 

@@ -253,17 +253,17 @@ def test_workspace_serves_smaller_batches_and_page_tables(b, H, L_s, pages, fp8,
                     for path, schedule, stacked in ((0, 0, True), (0, 1, True), (0, 2, False), (1, 0, True)):
                         for mode in ((b.MODE_AUTO, b.MODE_ABSORB, b.MODE_HYBRID, b.MODE_NAIVE) if m == b.MODE_AUTO else (m,)):
                             args = dict(mode=mode, prefix_8bit=fp8, path=path, schedule=schedule, stacked=stacked)
-                            _, step, chunks, slots = b.typhoon_mla_workspace_plan(H, L_s, B, p, workspace_bytes=size, **args)
+                            _, step, chunks, slots, _ = b.typhoon_mla_workspace_plan(H, L_s, B, p, workspace_bytes=size, **args)
                             assert step <= size
-                            _, own, own_chunks, own_slots = b.typhoon_mla_workspace_plan(H, L_s, B, p, **args)
+                            _, own, own_chunks, own_slots, _ = b.typhoon_mla_workspace_plan(H, L_s, B, p, **args)
                             assert (chunks, slots) == (own_chunks, own_slots) if own <= size else (chunks < own_chunks or slots < own_slots)
 
 
 def test_workspace_that_is_too_small_is_refused(b):
     for H, L_s, B, pages in ((16, 4096, 8, 16), (128, 16384, 64, 4), (64, 300, 256, 64), (96, 65536, 900, 1)):
         for mode in (b.MODE_ABSORB, b.MODE_HYBRID, b.MODE_NAIVE):
-            _, step, chunks, slots = b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode)
-            assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=step)[1:] == (step, chunks, slots)
+            _, step, chunks, slots, _ = b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode)
+            assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=step)[1:4] == (step, chunks, slots)
             # with a byte less the step takes fewer partials or is refused; without room for one of each kind it is refused
             try:
                 assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=step - 1)[1] < step
@@ -272,3 +272,13 @@ def test_workspace_that_is_too_small_is_refused(b):
             least = B * H * (512 * (2 + 2) + 128 * 4) + B * H * 4 * (512 if mode != b.MODE_NAIVE else 128)
             with pytest.raises(b.TyphoonMLAError, match="workspace"):
                 b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=mode, workspace_bytes=least)
+
+
+@pytest.mark.parametrize("H,B,L_s,pages,pairs", [
+    # measured on B200 in both kernels, us per absorb-only step (64 rows per CTA, 128 per pair)
+    (64, 12, 22865, 9, 1), (64, 44, 23213, 21, 1), (32, 31, 4399, 7, 1), (64, 2, 23872, 1, 1), (48, 73, 1816, 1, 1),   # 71.9 / 51.5 .. 56.3 / 44.4
+    (16, 60, 1426, 1, 0), (48, 67, 131, 1, 0), (16, 187, 193, 1, 0), (16, 214, 199, 1, 0), (48, 465, 343, 1, 0), (32, 185, 3378, 1, 0),   # 28.0 / 33.8 .. 127 / 157
+    (16, 7, 4096, 1, 0), (64, 16, 256, 8, 0)])   # fewer than 128 rows; a table wider than the prefix
+def test_absorb_only_steps_take_the_kernel_that_is_faster_for_them(b, H, B, L_s, pages, pairs):
+    assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_ABSORB)[4] == pairs
+    assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_ABSORB, stacked=False)[4] == 0
