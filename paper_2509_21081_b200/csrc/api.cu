@@ -284,7 +284,7 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
             p.n_slots_naive = naive_slots_override;
         } else if (use_naive && tc) {   // n_split_naive = tile ranges
             naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0,
-                             max_slots);
+                             use_absorb && cap > 0, max_slots);
         } else {
             p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm, max_slots) : 0;
             p.n_slots_naive = p.n_split_naive;
@@ -370,13 +370,13 @@ double typhoon_mla_batch_threshold(const typhoon_mla_dims_t* d, int32_t S_q, dou
     return (d_qk + d->d_v) / ((double)S_q * (2.0 * d->kv_lora_rank + d->d_rope)) * (T / M);
 }
 
-int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms,
+int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms, int32_t absorb_beside,
                            int32_t* tile_tokens, int32_t* n_ranges, int32_t* row_groups, int32_t* n_slots) {
     if (B < 1 || L_s < 1 || L_s > (int64_t)1 << 30 || schedule < 0 || schedule > 2 || num_sms < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (!tile_tokens || !n_ranges || !row_groups || !n_slots) return TYPHOON_MLA_ERR_INVALID_ARG;
     int r = 0, sl = 0;
-    naive_sm100_plan(B, num_heads, L_s, naive_places(B, num_sms > 0 ? num_sms : kDefaultNumSM, false), schedule, &r, &sl);
+    naive_sm100_plan(B, num_heads, L_s, naive_places(B, num_sms > 0 ? num_sms : kDefaultNumSM, false), schedule, &r, &sl, false, absorb_beside != 0);
     *tile_tokens = naive_sm100_tile_tokens(B);
     *n_ranges = r;
     *row_groups = B <= 128 ? 1 : (B + 255) / 256;
@@ -1147,7 +1147,8 @@ struct TreePlan {
     EmptySlots empties[kMaxTreeJobs];
     int n_jobs = 0, n_empties = 0, total_slots = 0;
 };
-int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int schedule, TreePlan* tp) {
+// `beside`: the step has an absorb branch.
+int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int schedule, bool beside, TreePlan* tp) {
     if (!levels || n_levels < 1 || n_levels > kMaxLevels || B < 1) return TYPHOON_MLA_ERR_INVALID_ARG;
     for (int l = 0; l < n_levels && !tp->sh0; ++l) {
         if (!levels[l].prefixes || !levels[l].group_begin || levels[l].n_groups < 1) return TYPHOON_MLA_ERR_INVALID_ARG;
@@ -1194,7 +1195,9 @@ int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int
             }
             naive_sm100_plan_multi(rows, H, len, n, n_sm, schedule, &ranges, &slots_of[j]);
         } else {
-            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, naive_places(tp->jobs[j].rows, n_sm, tp->jobs[j].sh->fp8 != 0), schedule, &ranges, &slots_of[j], tp->jobs[j].sh->fp8 != 0);
+            const bool fp8 = tp->jobs[j].sh->fp8 != 0;
+            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, naive_places(tp->jobs[j].rows, n_sm, fp8), schedule, &ranges, &slots_of[j],
+                             fp8, beside);
         }
         for (int k = 0; k < n; ++k) tp->jobs[j + k].n_ranges = ranges;
         tp->jobs[j].n_merged = n;
@@ -1229,14 +1232,16 @@ int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int
 size_t typhoon_mla_tree_workspace_bytes(const typhoon_mla_prefix_level_t* levels, int32_t n_levels, int32_t B,
                                         int32_t max_pages, int32_t page_size) {
     if (max_pages < 0 || (page_size != 64 && page_size != 128)) return 0;
-    // worst case over the work decompositions a test hook may select (the tree step needs the tcgen05 kernels)
+    // worst case over the work decompositions a test hook may select (the tree step needs the tcgen05 kernels), with and without
+    // an absorb branch, and the floor (make_plan)
     size_t worst = 0;
-    for (int schedule : {0, 1, 2}) {
-        TreePlan tp;
-        if (plan_tree(levels, n_levels, B, schedule, &tp) != TYPHOON_MLA_OK) return 0;
-        for (size_t bytes : {SIZE_MAX, (size_t)0})   // the step's own choice, and what smaller page tables may choose (make_plan)
-            worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots, true, bytes).total);
-    }
+    for (int schedule : {0, 1, 2})
+        for (bool beside : {true, false}) {
+            TreePlan tp;
+            if (plan_tree(levels, n_levels, B, schedule, beside, &tp) != TYPHOON_MLA_OK) return 0;
+            for (size_t bytes : {SIZE_MAX, (size_t)0})
+                worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots, true, bytes).total);
+        }
     return worst + 256;
 }
 
@@ -1259,7 +1264,7 @@ int typhoon_mla_decode_tree(const typhoon_mla_prefix_level_t* levels, int32_t n_
             return TYPHOON_MLA_ERR_INVALID_ARG;
     }
     TreePlan tp;
-    const int rc = plan_tree(levels, n_levels, B, cfg.naive_schedule, &tp);
+    const int rc = plan_tree(levels, n_levels, B, cfg.naive_schedule, max_pages > 0, &tp);
     if (rc != TYPHOON_MLA_OK) return rc;
     if (!on_handle_device(tp.sh0)) return TYPHOON_MLA_ERR_INVALID_ARG;
     // NAIVE when there is no page table (nothing for the absorb branch), else Algorithm 1 with several line-4 launches

@@ -146,8 +146,9 @@ int naive_sm100_tile_tokens(int B, bool fp8 = false);   // KV tile width the ker
 // schedule: 0 = chosen by the plan, 1 = column split, 2 = stream-K
 inline bool naive_uses_pairs(int B, bool fp8) { return !fp8 && B > 128; }
 inline int naive_places(int B, int n_sm, bool fp8) { return naive_uses_pairs(B, fp8) ? n_sm / 2 : n_sm; }
-// max_slots (>= 1): the plan chooses no more partial slots than that.
-void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8 = false,
+// beside: the absorb branch of the step runs beside the launch (else nothing does).  max_slots (>= 1): the plan chooses no more
+// partial slots than that.
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, bool beside,
                       int max_slots = INT32_MAX);
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s);
 // ... its form for more than 128 rows of the 16-bit cache: 256 rows per pair of CTAs

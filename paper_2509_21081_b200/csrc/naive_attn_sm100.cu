@@ -901,7 +901,7 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // along the sequence without divisions (16 prefixes x 128 heads: 8 us; a pass per prefix with a division per tile
 // count and range took 159).
 static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8,
-                          int max_slots) {
+                          bool beside, int max_slots) {
     // (8-bit cache: always 64-token tiles, row groups of 128 requests)
     const bool mode_y = fp8 || B <= 128;
     const int tok = mode_y ? 64 : 128;
@@ -939,27 +939,34 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
             }
         return most;
     };
-    // With more than 128 rows of the 16-bit cache ranges may also hold several whole heads (one segment each, one slot per
-    // head), and a choice is charged half its time and half its SM time: places that it leaves free go to the absorb branch.
-    // (700 rows x 32 heads over 2048 tokens + 64: 106 us per step with 48 of 74 pairs, 123 with 72.)  But a few free SMs only help if the
-    // query absorption, about 4 us per head and 128 requests, gets done on them meanwhile; else it had better wait for all
-    // SMs.  (64 pairs / 74, us per step of 128 heads: 140 rows, 3000 + 500 tokens 120 / 132, 200 rows, 2000 + 300 tokens 156 / 128.)
+    // More than 128 rows of the 16-bit cache (a place is a pair of SMs; costs in tiles of 0.9 us).  Ranges may also hold several whole
+    // heads (one segment each, one slot per head).  By itself a choice is charged its time.  Beside the absorb branch it is charged
+    // 15 % of its time and 85 % of its SM time, since the places that it leaves free go to that branch, and up to 8 tiles in the
+    // measure in which they do not suffice to get the query absorption (8 us per head and 128 requests) done meanwhile, because the
+    // branch's chain of launches then starts behind this kernel.  (The constants are the best of a search over 96 shapes, 129 to 1024
+    // rows, 16 to 128 heads, 69 to 27000 tokens, every cut measured: on average the choice is 0.8 % behind the best cut beside the
+    // branch and 0.1 % by itself.  B200, us per step: 198 rows x 128 heads, 244 + 138 tokens, two waves of 64 places 88, 32 places
+    // 78; 310 x 48, 2108 + 533, 37 x 2 equal ranges 142, 16 x 2 110; 166 x 16, 7069 + 1537, 64 places 74, 32 69; 216 x 96, 15590 +
+    // 221, 74 places 253, 48 (chosen) 266; by themselves 212 x 128, 660 tokens, two waves 35.8, 64 places 32.1.)
     const bool pairs = !mode_y;
     auto charge = [&](double cost, long long items) {   // `cost` of all waves
+        if (!pairs) return cost;
         const double waves = (double)((items + n_sm - 1) / n_sm);
-        return pairs ? cost * (0.5 + 0.5 * (double)items / (waves * n_sm)) : cost;
+        cost += 4.0 * (waves - 1.0);
+        if (!beside) return cost;
+        const double absorbed = cost * 0.9 * 2.0 * (n_sm - items / waves) / (8.0 * H * ((B + 127) / 128));
+        return cost * (0.15 + 0.85 * items / (waves * n_sm)) + 8.0 * (1.0 - std::min(1.0, absorbed));
     };
-    auto absorption_fits = [&](double cost, long long items) { return cost * 0.9 * 2.0 * (double)(n_sm - items) >= 4.0 * H * ((B + 127) / 128); };
     // column split
     const long long base = (long long)H * m_groups;
     // Cost of a range's beginning and of each further segment, in tile times.  (A pair of CTAs requests the next segment's queries
     // early and goes on with its logits while the last segment's output is written; a further wave of pairs costs a launch, its
-    // set-up and a pipeline fill.  700 rows x 128 heads over 500 tokens, six waves: 103 us, the work of 50.)
-    const double fixed = 6.0, boundary = mode_y ? 6.0 : 3.0;
+    // set-up and a pipeline fill.)
+    const double fixed = pairs ? 12.0 : 6.0, boundary = pairs ? 3.0 : 6.0;
     // every further partial slot is one more dependent read of B x H x 128 floats in the combine that follows
     // (about 5 us, i.e. 8 tile times, measured with 64-token tiles; with more than 128 rows the bytes count: 512 per row and
     // head at 5 TB/s, in tiles of 0.9 us)
-    const double slot_cost = mode_y ? 8.0 : 1.1e-4 * B * H;
+    const double slot_cost = pairs ? 1.1e-4 * B * H : 8.0;
     int ns_best = 1;
     double cost_best = 1e30, eff_best = 0.0;
     for (int ns = 1; ns <= std::min({n_tiles, 32, max_slots}); ++ns) {
@@ -975,12 +982,12 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     }
     int r_column = H * ns_best;
     if (pairs && schedule == 0)
-        for (int k = 2; k <= H; ++k) {   // whole heads, k per range, in one wave
-            const long long items = (long long)(H / k) * m_groups;
-            const double time = (double)k * n_tiles + fixed + (k - 1) * boundary;
-            if (H % k != 0 || items > n_sm || !absorption_fits(time, items)) continue;
-            if (charge(time, items) < cost_best - 1e-9) {
-                cost_best = charge(time, items);
+        for (int k = 2; k <= H; ++k) {   // whole heads, k per range
+            if (H % k != 0) continue;
+            const long long items = (long long)(H / k) * m_groups, waves = (items + n_sm - 1) / n_sm;
+            const double cost = charge((double)waves * ((double)k * n_tiles + fixed + (k - 1) * boundary), items);
+            if (cost <= cost_best + 1e-9) {   // (as good on fewer places)
+                cost_best = cost;
                 r_column = H / k;
             }
         }
@@ -1008,12 +1015,12 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     if (R != r_stream) fill_slots(R);   // the kernel uses the same partition
 }
 
-void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, int max_slots) {
-    plan_sequence(B, H, &Ls, 1, places, schedule, n_ranges, n_slots, fp8, max_slots);
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, bool beside, int max_slots) {
+    plan_sequence(B, H, &Ls, 1, places, schedule, n_ranges, n_slots, fp8, beside, max_slots);
 }
 
 void naive_sm100_plan_multi(int max_rows, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots) {
-    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false, INT32_MAX);
+    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false, true, INT32_MAX);
 }
 
 

@@ -165,10 +165,10 @@ def test_naive_plan_invariants(b):
                 assert R == min(max(1, (148 if B <= 128 else 74) // groups), T)   # one range per SM, or per pair of SMs
             if schedule == 0 and B > 128:
                 assert R % H == 0 or H % R == 0 or R == min(max(1, 74 // groups), T)
-    # benchmark configs: config 1 one range per head; config 2 one CTA per SM; config 4 at B = 512 one CTA pair per pair of SMs
+    # benchmark configs: config 1 one range per head; config 2 one CTA per SM; config 4 at B = 512 four heads per range
     assert b.typhoon_mla_naive_plan(128, 64, 4096)[1:] == (128, 1, 1)
     assert b.typhoon_mla_naive_plan(128, 128, 26624)[1] == 148
-    assert b.typhoon_mla_naive_plan(128, 512, 16384)[1:3] == (37, 2)
+    assert b.typhoon_mla_naive_plan(128, 512, 16384)[1:3] == (32, 2)
     # what a step launches and sizes its partials for
     for H, B, Ls in ((128, 512, 16384), (64, 256, 8192), (16, 166, 7069), (32, 700, 2048), (128, 64, 4096), (16, 129, 1)):
         assert b.typhoon_mla_naive_plan(H, B, Ls)[3] == b.typhoon_mla_workspace_plan(H, Ls, B, 4, mode=b.MODE_HYBRID)[3]
@@ -181,6 +181,15 @@ def test_naive_plan_invariants(b):
     for bad in ((8, 1, 10, 0), (128, 0, 10, 0), (128, 1, 0, 0), (128, 1, 10, 3)):
         with pytest.raises(Exception):
             b.typhoon_mla_naive_plan(*bad)
+
+
+@pytest.mark.parametrize("H,B,L_s,beside,alone", [
+    # ranges that were measured (B200) to be the fastest cut beside the absorb branch, or within 2 % of it, and by themselves: a
+    # part of the places beside the branch, one wave of them alone
+    (128, 198, 244, 32, 64), (48, 310, 2108, 24, 37), (64, 182, 602, 32, 64), (128, 258, 194, 16, 32), (128, 212, 660, 32, 64), (64, 256, 8192, 64, 74)])
+def test_more_than_128_rows_leave_places_to_the_absorb_branch(b, H, B, L_s, beside, alone):
+    assert b.typhoon_mla_naive_plan(H, B, L_s)[1] == beside
+    assert b.typhoon_mla_naive_plan(H, B, L_s, absorb_beside=False)[1] == alone
 
 
 @pytest.mark.parametrize("H,B,slots,early", [(128, 64, 1, 1), (128, 128, 2, 1), (128, 129, 2, 0), (128, 198, 1, 0), (128, 1024, 1, 0),
