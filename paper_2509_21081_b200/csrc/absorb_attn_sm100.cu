@@ -1,7 +1,7 @@
-// Absorb attention over latent tokens (Algorithm 1 line 6) on tcgen05 / TMEM / TMA, for at most 64 heads (more go to
-// absorb_pair_sm100.cu).
+// Absorb attention over latent tokens (Algorithm 1 line 6) on tcgen05 / TMEM / TMA, 64 query rows at a time (absorb_pair_sm100.cu takes
+// 128; the step's plan chooses).
 //
-// Work item (CTA) = (64 query rows, KV chunk).  Over a request's own suffix the rows are the heads of that
+// Work item (CTA) = (64 query rows, KV chunk).  Over a request's own suffix the rows are 64 heads of that
 // request.  Over the shared prefix (absorb-only steps) every request attends to the same tokens, so the rows are
 // 64 consecutive rows of the stacked [B * H] query matrix: with fewer than 64 heads per request (a head-sharded
 // model) several requests fill one tile instead of each padding its own.  The problem is run
@@ -142,7 +142,7 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         if (lane == 5) prefetch_tmap(&tm_kpe_pg);
     }
     // Work items in launch order: the shared-prefix items (chunk fastest, then row group), then the suffix items
-    // (chunk fastest, then request position in longest-first order).
+    // (chunk fastest, then head group, then request position in longest-first order).
     const int n_shared_items = p.n_shared_chunks * p.shared_groups;
     const bool shared_seg = (int)blockIdx.x < n_shared_items;
     // The preceding kernel writes Q_A and the descriptors, the caller's kernels the page table and the lengths: the wait.  The
@@ -155,15 +155,16 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         if (p.stacked) {                       // 64 consecutive rows of the stacked query matrix
             row0 = g * 64;
             n_rows = min(64, p.B * p.H - row0);
-        } else {                               // the heads of one request
-            b = g;
-            row0 = b * p.H;
-            n_rows = p.H;
+        } else {                               // 64 heads of one request
+            const int hg = (p.H + 63) / 64;
+            b = g / hg;
+            row0 = b * p.H + (g % hg) * 64;
+            n_rows = min(64, p.H - (g % hg) * 64);
         }
     } else {
-        const int i = blockIdx.x - n_shared_items;
+        const int i = blockIdx.x - n_shared_items, hg = (p.H + 63) / 64;
         chunk = p.n_shared_chunks + i % p.n_suffix_chunks;
-        const int z = i / p.n_suffix_chunks;
+        const int y = (i / p.n_suffix_chunks) % hg, z = i / (p.n_suffix_chunks * hg);
         // one 16-byte load gives the request, its suffix length and its first two pages (else three
         // dependent loads stand between the kernel's start and its first copy)
         if (p.desc != nullptr) {
@@ -172,8 +173,8 @@ absorb_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
         } else {
             b = p.order ? p.order[z] : z;
         }
-        row0 = b * p.H;
-        n_rows = p.H;
+        row0 = b * p.H + y * 64;
+        n_rows = min(64, p.H - y * 64);
     }
 
     // token range of this chunk
@@ -626,7 +627,7 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
                                      void* o_lat_direct, float* lse_direct, int* status, cudaStream_t s) {
     const int n_chunks = a.n_shared_chunks + a.n_suffix_chunks;
     if (a.B <= 0 || n_chunks <= 0) return cudaSuccess;
-    if (a.chunk % TOK != 0 || a.H > 64) return cudaErrorInvalidValue;
+    if (a.chunk % TOK != 0) return cudaErrorInvalidValue;
     CUtensorMap tm_qa, tm_qp, tm_ckv_pg, tm_kpe_pg;
     {   // the queries as one [B * H, 512] matrix: a box is 64 consecutive rows (of one request or across requests);
         // rows past the end read as zeros
@@ -655,8 +656,9 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
     AbsorbSm100Params p{};
     p.B = a.B; p.H = a.H;
     p.chunk = a.chunk; p.n_shared_chunks = a.n_shared_chunks; p.n_suffix_chunks = a.n_suffix_chunks;
+    const int head_groups = (a.H + 63) / 64;
     p.stacked = a.stacked ? 1 : 0;
-    p.shared_groups = a.stacked ? (int)(((int64_t)a.B * a.H + 63) / 64) : a.B;
+    p.shared_groups = a.stacked ? (int)(((int64_t)a.B * a.H + 63) / 64) : a.B * head_groups;
     p.Ls_absorb = a.Ls_absorb;
     p.page_size = a.page_size; p.max_pages = a.max_pages; p.num_pages = a.num_pages;
     p.block_table = a.block_table; p.seq_lens = a.seq_lens; p.order = a.order;
@@ -666,7 +668,7 @@ cudaError_t launch_absorb_attn_sm100(const AbsorbAttn& a, const CUtensorMap* tm_
     p.o_lat_direct = n_chunks == 1 ? reinterpret_cast<__nv_bfloat16*>(o_lat_direct) : nullptr;
     p.lse_direct = lse_direct;
     const int smem = kAbsorbSmem;
-    dim3 grid(a.n_shared_chunks * p.shared_groups + a.n_suffix_chunks * a.B, 1, 1);
+    dim3 grid(a.n_shared_chunks * p.shared_groups + a.n_suffix_chunks * head_groups * a.B, 1, 1);
     p.l2_base = reinterpret_cast<const char*>(a.w_uv);
     p.l2_total = a.w_uv ? (uint32_t)a.H * 128u * 512u * 2u : 0u;
     p.l2_bytes = (p.l2_total / (grid.x * 32u) / 16u + 1u) * 16u;

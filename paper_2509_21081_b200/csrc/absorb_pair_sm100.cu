@@ -1,7 +1,7 @@
 // Absorb attention over latent tokens (Algorithm 1 line 6) for 128 query rows at a time: a pair of CTAs on one product.
 //
-// Work item (CTA pair) = (128 query rows, KV chunk).  Over a request's own suffix the rows are the heads of that request (more
-// than 64 of them; fewer go to the 64-row kernel), over the shared prefix 128 consecutive rows of the stacked [B * H] matrix.
+// Work item (CTA pair) = (128 query rows, KV chunk).  Over a request's own suffix the rows are the heads of that request (with
+// fewer than 128 some rows are nobody's), over the shared prefix 128 consecutive rows of the stacked [B * H] matrix.
 //     S [128 rows, 128 tokens] = Q [128, 576] * K_tile [128, 576]^T       (K_tile = latent 512 | rope 64 of 128 tokens)
 //     O [128 rows, 512]       += P [128, 128 tokens] * C_tile [128, 512]
 // Each CTA holds 64 query rows; with M = 128 over two CTAs the accumulators of its 64 rows fold into all 128 lanes of its tensor
@@ -580,7 +580,7 @@ cudaError_t launch_absorb_pair_sm100(const AbsorbAttn& a, int64_t Ls_pad, void* 
                                      cudaStream_t s) {
     const int n_chunks = a.n_shared_chunks + a.n_suffix_chunks;
     if (a.B <= 0 || n_chunks <= 0) return cudaSuccess;
-    if (a.chunk % TOK != 0) return cudaErrorInvalidValue;
+    if (a.chunk % TOK != 0 || a.H > 128) return cudaErrorInvalidValue;
     const int64_t rows = (int64_t)a.B * a.H;
     CUtensorMap tm_qa, tm_qp, tm_ckv_sh, tm_kpe_sh, tm_ckv_pg, tm_kpe_pg, tm_o_sh, tm_o_sf;
     {   // the queries as one [B * H, 512] matrix; rows past the end read as zeros

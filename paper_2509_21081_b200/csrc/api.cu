@@ -156,8 +156,20 @@ int naive_splits(int B, int H, int64_t Ls, int n_sm, int max_slots) {
     return std::max(1, std::min({want, n_tiles, 64, max_slots}));
 }
 
+// Whether the absorb attention of a step of more than 64 heads goes to the kernel of 128 rows per CTA pair: yes, except where the table
+// holds few tokens per request and the step runs beside a shared-prefix launch of at most 128 rows.  Those CTAs leave single SMs free,
+// not the two neighbouring ones that a pair needs, and with suffixes this short what the 64-row kernel gets done on them counts
+// for more than the pair's faster tiles.  (B200, us per step, 64-row / pair: 96 heads, 24 requests, 2301 tokens and one page of 64
+// 36.5 / 40.6, 128 heads, 100 requests, 1277 and one page 63.7 / 66.4, 1280 and four pages 63.3 / 66.1; 128 heads, 8 requests, 809
+// and four pages 43.8 / 39.4; 54 requests, 1267 and two pages 52.6 / 51.9.  Over 119 such steps this line loses 0.5 % to the better of
+// the two, one kernel for all 1.4 and 2.4 %.)
+bool many_heads_use_pairs(int B, int64_t cap_suffix, bool beside_prefix) {
+    return !(beside_prefix && B <= 128 && (cap_suffix <= 64 || (cap_suffix <= 256 && B > 64)));
+}
+
 // Kernel and chunk length of the absorb attention.  max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks.
-void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks,
+// `beside_prefix`: a shared-prefix launch runs beside it.
+void absorb_chunks(bool tc, bool stacked, bool beside_prefix, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks,
                    bool* pairs, int* chunk, int* n_sh, int* n_sf) {
     const int64_t longest = std::max<int64_t>(std::max(Ls_absorb, cap_suffix), 1);
     // One CTA (pair) per SM (pair of SMs): minimise waves x (tiles per chunk + fixed cost in tile units) over the number of
@@ -200,8 +212,8 @@ void absorb_chunks(bool tc, bool stacked, int n_sm, int B, int H, int64_t Ls_abs
     int64_t c;
     *pairs = false;
     if (tc && H > 64) {
-        *pairs = true;
-        c = cut(true);
+        *pairs = many_heads_use_pairs(B, cap_suffix, beside_prefix);
+        c = cut(*pairs);
     } else if (tc) {
         // Up to 64 heads the pair kernel is for the prefix of an absorb-only step, whose rows are stacked and fill its 128; a suffix item
         // has rows of nobody and still takes two SMs.  (B200, us per step, 64-row / pair: 64 heads, 12 requests, 22865 + 567 tokens
@@ -290,7 +302,7 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
             p.n_slots_naive = p.n_split_naive;
         }
         if (use_absorb)
-            absorb_chunks(tc, stacked, n_sm, B, H, Ls_absorb, cap, max_chunks, &p.absorb_pairs, &p.chunk,
+            absorb_chunks(tc, stacked, p.n_slots_naive > 0, n_sm, B, H, Ls_absorb, cap, max_chunks, &p.absorb_pairs, &p.chunk,
                           &p.n_shared_chunks, &p.n_suffix_chunks);
         lay_out(&p, B, H, (int64_t)(p.n_shared_chunks + p.n_suffix_chunks) * rows, (int64_t)p.n_slots_naive * rows);
         return p;

@@ -291,3 +291,11 @@ def test_workspace_that_is_too_small_is_refused(b):
 def test_absorb_only_steps_take_the_kernel_that_is_faster_for_them(b, H, B, L_s, pages, pairs):
     assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_ABSORB)[4] == pairs
     assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_ABSORB, stacked=False)[4] == 0
+
+
+@pytest.mark.parametrize("H,B,L_s,pages,pairs", [
+    (96, 24, 2301, 1, 0), (128, 100, 1277, 1, 0), (128, 100, 1280, 4, 0), (96, 128, 508, 1, 0),   # 36.5 / 40.6, 63.7 / 66.4, 63.3 / 66.1, 48.9 / 51.5
+    (128, 8, 809, 4, 1), (96, 24, 544, 4, 1), (128, 64, 4096, 8, 1), (128, 128, 26624, 32, 1), (128, 129, 1000, 1, 1)])   # 43.8 / 39.4, 40.3 / 37.4
+def test_many_heads_beside_a_prefix_of_few_rows_take_the_kernel_that_is_faster_for_them(b, H, B, L_s, pages, pairs):
+    assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_HYBRID)[4] == pairs
+    assert b.typhoon_mla_workspace_plan(H, L_s, B, pages, mode=b.MODE_ABSORB)[4] == 1    # nothing runs beside
