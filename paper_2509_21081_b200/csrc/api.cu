@@ -968,15 +968,11 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
             if (order) desc = reinterpret_cast<int32_t*>(ws + pl.off_desc);
             // Beside the shared-prefix kernel the absorb branch has the SMs that kernel's CTAs leave free: if those are few,
             // that many CTAs walk through the heads (each resident for the whole launch) instead of one CTA per head
-            // queueing for them.
+            // queueing for them.  (With one tile of 128 requests per head; a launch then has one CTA per range.)
             int walk_ctas = 0;
-            if (forked) {
+            if (forked && B <= 128) {
                 int naive_ctas = 0;
-                for (int j = 0; j < n_jobs; ++j) {
-                    const int rows = jobs[j].rows;
-                    const int groups = jobs[j].sh->fp8 ? (rows + 127) / 128 : (rows <= 128 ? 1 : 2 * ((rows + 255) / 256));   // CTAs per range
-                    naive_ctas = std::max(naive_ctas, jobs[j].n_ranges * groups);
-                }
+                for (int j = 0; j < n_jobs; ++j) naive_ctas = std::max(naive_ctas, jobs[j].n_ranges);
                 const int free_sms = sh->num_sms - naive_ctas;
                 if (jobs[0].n_merged == n_jobs && free_sms >= 8 && free_sms < H) {
                     // ... but only if the shared-prefix kernel lasts about as long as the walk (measured: about 5 us per head
@@ -985,12 +981,11 @@ static int decode_core(const Settings& cfg, const typhoon_mla_shared* sh, const 
                     // which spreads over the whole GPU as soon as that kernel ends, is faster.  A 64-token tile of the 8-bit
                     // cache takes 1.0 us, with more than 64 rows 1.3 (H = 128, us per step, one CTA per head / walk: 64
                     // requests over 1900 tokens 65.4 / 53.2, over 2400 69.7 / 59.6, 100 over 1500 74.3 / 65.5).
-                    const int64_t tok = jobs[0].rows <= 128 || jobs[0].sh->fp8 ? 64 : 128;
                     int64_t head_tiles = 0;
-                    for (int j = 0; j < n_jobs; ++j) head_tiles += (jobs[j].sh->Ls + tok - 1) / tok;
+                    for (int j = 0; j < n_jobs; ++j) head_tiles += (jobs[j].sh->Ls + 63) / 64;
                     const int64_t tiles_per_cta = (head_tiles * H + jobs[0].n_ranges - 1) / jobs[0].n_ranges;
                     const int heads_per_cta = (H + free_sms - 1) / free_sms;
-                    const double tile_us = jobs[0].sh->fp8 ? (jobs[0].rows <= 64 ? 1.0 : 1.3) : tok == 64 ? 0.7 : 3.0;
+                    const double tile_us = jobs[0].sh->fp8 ? (jobs[0].rows <= 64 ? 1.0 : 1.3) : 0.7;
                     if ((double)tiles_per_cta * tile_us >= 4.0 * heads_per_cta) walk_ctas = free_sms;
                 }
             }
