@@ -319,14 +319,16 @@ absorb_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
                             const uint64_t da0 = smem_desc_k_sw128(pa);
                             const uint64_t db0 = smem_desc_mn_sw128(va + (4 * nb) * SLAB, SLAB, 1024);
                             const uint32_t d = tmem_base + (uint32_t)nb * 128u;
+                            auto product = [&](int k) {   // 16 tokens (descriptor addresses count 16-byte units)
+                                umma_pair_ss(d, da0 + (k >> 2) * (SLAB / 16) + 2 * (k & 3), db0 + (k >> 2) * (2 * SLAB / 16) + (k & 3) * 128,
+                                             idesc_o, (t | k) != 0);
+                            };
                             if (n_k == 8) {
 #pragma unroll
-                                for (int k = 0; k < 8; ++k)   // descriptor addresses count 16-byte units
-                                    umma_pair_ss(d, da0 + (k >> 2) * (SLAB / 16) + 2 * (k & 3), db0 + (k >> 2) * (2 * SLAB / 16) + (k & 3) * 128, idesc_o, (t | k) != 0);
+                                for (int k = 0; k < 8; ++k) product(k);
                             } else {
 #pragma unroll 1
-                                for (int k = 0; k < n_k; ++k)
-                                    umma_pair_ss(d, da0 + (k >> 2) * (SLAB / 16) + 2 * (k & 3), db0 + (k >> 2) * (2 * SLAB / 16) + (k & 3) * 128, idesc_o, (t | k) != 0);
+                                for (int k = 0; k < n_k; ++k) product(k);
                             }
                             umma_pair_commit(&sh->v_empty[nb]);
                             if (nb == 1) umma_pair_commit(&sh->o_done[t & 1]);
@@ -470,8 +472,10 @@ absorb_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_qa, const __grid
                                 uint4 v;
                                 uint32_t* vv = reinterpret_cast<uint32_t*>(&v);
 #pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    vv[e] = pack_bf16(__uint_as_float(orr[8 * c + 2 * e]) * inv, __uint_as_float(orr[8 * c + 2 * e + 1]) * inv);
+                                for (int e = 0; e < 4; ++e) {
+                                    const uint32_t* x = orr + 8 * c + 2 * e;
+                                    vv[e] = pack_bf16(__uint_as_float(x[0]) * inv, __uint_as_float(x[1]) * inv);
+                                }
                                 *reinterpret_cast<uint4*>(box + (((4 * (i & 1) + c) ^ (row & 7)) * 16)) = v;
                             }
                         } else {

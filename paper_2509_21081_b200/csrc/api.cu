@@ -181,9 +181,11 @@ void absorb_chunks(bool tc, bool stacked, bool beside_prefix, int n_sm, int B, i
         const int units = B * ((H + tile - 1) / tile);
         const int units_sh = stacked ? (int)(((int64_t)B * H + tile - 1) / tile) : units;
         double best_cost = 1e30;
-        int64_t c = round_up(longest, tile);
+        int64_t c = round_up(longest, tile), weighed = 0;
         for (int parts = 1; parts <= 512; ++parts) {
             const int64_t ch = round_up((longest + parts - 1) / parts, tile);
+            if (ch == weighed) continue;
+            weighed = ch;
             const int64_t per_req = (Ls_absorb + ch - 1) / ch + (cap_suffix + ch - 1) / ch;
             const int64_t items = (int64_t)units_sh * ((Ls_absorb + ch - 1) / ch) + (int64_t)units * ((cap_suffix + ch - 1) / ch);
             if (per_req > max_chunks) continue;
@@ -203,8 +205,10 @@ void absorb_chunks(bool tc, bool stacked, bool beside_prefix, int n_sm, int B, i
         const int tile = pair ? 128 : 64;
         const double n_sh = (double)((Ls_absorb + c - 1) / c), n_sf = (double)((cap_suffix + c - 1) / c);
         const double extra = (pair ? 6.0 : 5.0) + (n_sh + n_sf > 1 ? (pair ? 3.0 : 3.5) : 0.0);
-        const double t_sh = (double)std::min(c, Ls_absorb) / tile + extra, t_sf = (double)((std::min(c, cap_suffix) + tile - 1) / tile) + extra;
-        const double items_sh = (double)(((int64_t)B * H + tile - 1) / tile) * n_sh, items_sf = (double)B * ((H + tile - 1) / tile) * n_sf;
+        const double t_sh = (double)std::min(c, Ls_absorb) / tile + extra;
+        const double t_sf = (double)((std::min(c, cap_suffix) + tile - 1) / tile) + extra;
+        const double items_sh = (double)(((int64_t)B * H + tile - 1) / tile) * n_sh;
+        const double items_sf = (double)B * ((H + tile - 1) / tile) * n_sf;
         const double longest_item = n_sh > 0 ? t_sh : t_sf;
         const double tiles = std::max(longest_item, (items_sh * t_sh + items_sf * t_sf) / (pair ? n_sm / 2 : n_sm) + 0.5 * longest_item);
         return tiles * (pair ? 2416.0 : 2580.0);
@@ -318,7 +322,8 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
     lay_out(&least, B, H, chunk_rows, slot_rows);
     if (workspace_bytes == 0) return least;
     if (workspace_bytes < least.total) return p;
-    const int64_t more = (int64_t)(workspace_bytes - least.total);   // (a chunk's row: 512 values and its LSE, of which the sum is rounded up)
+    // (a chunk's row: 512 values and its LSE; the LSEs' bytes are rounded up to 256)
+    const int64_t more = (int64_t)(workspace_bytes - least.total);
     const int64_t max_chunks = (chunk_rows + std::max<int64_t>(more - 256, 0) / (512 * 4 + 4)) / rows;
     return plan_within((int)std::min<int64_t>(max_chunks, kMaxAbsorbChunks), (int)std::min<int64_t>(slot_rows / rows, INT32_MAX));
 }
@@ -476,14 +481,16 @@ static int choose_mode_impl(const typhoon_mla_dims_t* dims, int64_t Ls, int32_t 
     const typhoon_mla_dims_t& d = *dims;
     const double H = d.num_heads, L = (double)Ls;
     const double f_naive = 2.0 * B * H * L * (d.d_nope + d.d_rope + d.d_v);
-    // (the absorb kernel works on groups of 64 rows of the stacked [B * H] query matrix: a partial group costs as
-    // much as a full one)
+    // (the absorb kernels work on groups of 64 or 128 rows of the stacked [B * H] query matrix: a partial group costs as
+    // much as a full one; counted in groups of 64)
     const double rows_abs = std::ceil(B * H / 64.0) * 64.0;
     const double f_absorb = 2.0 * rows_abs * L * (2.0 * d.kv_lora_rank + d.d_rope);
     const double by_naive = 2.0 * L * (H * (d.d_nope + d.d_v) + d.d_rope);
     const double by_absorb = 2.0 * L * (d.kv_lora_rank + d.d_rope);
-    // The absorb kernel re-reads the prefix per request and runs M = 64 tiles: measured on B200 it
-    // reaches about half of the tensor throughput the naive kernel does, hence the factor.
+    // The factor: the 64-row absorb kernel reaches about half of the tensor throughput that the naive kernel does (B200).  The
+    // pair kernel reaches more, and for 21 to 36 requests of 128 heads the latent form would be the faster one (24 over 16384
+    // tokens 135 us, hybrid 185); the line stays, because that form's 16-bit absorbed queries and latent outputs put the result
+    // further from the 64-bit one (3.0e-3 against 2.2e-3).  A caller can ask for it.
     const double T = g_tensor_flops.load(), M = g_hbm_bytes.load();
     const double t_hybrid = naive_time_factor * std::max(f_naive / T, by_naive / M) + g_hybrid_fixed_s.load();
     const double t_absorb = std::max(f_absorb / (g_absorb_efficiency.load() * T), by_absorb / M);

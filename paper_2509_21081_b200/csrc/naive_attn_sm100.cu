@@ -883,7 +883,6 @@ naive_attn_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
 
 }  // namespace
 
-
 int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 128; }
 
 // Host-side plan (pure function of the sizes): number of tile ranges R and of partial slots.
@@ -997,8 +996,8 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     const long long waves_stream = ((long long)r_stream * m_groups + n_sm - 1) / n_sm;
     const double segs_stream = (per_stream >= n_tiles) ? (double)per_stream / n_tiles + 1.0 : 2.0;
     const int slots_stream = fill_slots(r_stream);
-    const double cost_stream = charge((double)waves_stream * (per_stream + fixed + (segs_stream - 1.0) * boundary) + slot_cost * (slots_stream - 1),
-                                      (long long)r_stream * m_groups);
+    const double time_stream = (double)waves_stream * (per_stream + fixed + (segs_stream - 1.0) * boundary);
+    const double cost_stream = charge(time_stream + slot_cost * (slots_stream - 1), (long long)r_stream * m_groups);
     bool stream_k;
     if (schedule == 1 || slots_stream > max_slots) stream_k = false;
     else if (schedule == 2) stream_k = true;

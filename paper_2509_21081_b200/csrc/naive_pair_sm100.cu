@@ -104,7 +104,8 @@ naive_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
         constexpr int n_bars = (int)(offsetof(Barriers, tmem_base) / sizeof(uint64_t));
         for (int i = lane; i < n_bars; i += 32) {
             uint64_t* m = all + i;
-            mbar_init(m, m == &bar->o_free ? 16 : (m >= &bar->p_ready[0] && m < &bar->o_free) ? 8 : (m >= &bar->q_free[0] && m < &bar->k_empty[0]) ? 3 : 1);
+            const bool probabilities = m >= &bar->p_ready[0] && m < &bar->o_free, queries = m >= &bar->q_free[0] && m < &bar->k_empty[0];
+            mbar_init(m, m == &bar->o_free ? 16 : probabilities ? 8 : queries ? 3 : 1);
         }
         if (lane == 0) bar->abort_flag = 0;
         fence_mbar_init();
@@ -334,7 +335,8 @@ naive_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_qn, const __grid_
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         float x0, x1, p0, p1;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(src[2 * c]), __uint_as_float(src[2 * c + 1])), scale2, neg_m2), x0, x1);
+                        const uint64_t logits = pack_f32x2(__uint_as_float(src[2 * c]), __uint_as_float(src[2 * c + 1]));
+                        unpack_f32x2(fma_f32x2(logits, scale2, neg_m2), x0, x1);
                         if ((kPolyExpMask >> (c & 7)) & 1) {
                             exp2_poly_x2(x0, x1, p0, p1);
                         } else {
