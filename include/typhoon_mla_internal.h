@@ -18,8 +18,8 @@ extern "C" {
 #endif
 
 /* Work decomposition the tcgen05 shared-prefix kernel (Algorithm 1 line 4) would use for a problem
- * size on a GPU with `num_sms` multiprocessors (0: 148, a B200), beside an absorb branch (`absorb_beside`
- * 1: HYBRID steps and trees with a page table) or by itself: tokens per KV tile (64 for B <= 128,
+ * size on a GPU with `num_sms` multiprocessors (0: 148, a B200), beside an absorb branch of requests whose
+ * page table holds `suffix_tokens` each (HYBRID steps; more than 128 rows) or, with 0, by itself: tokens per KV tile (64 for B <= 128,
  * else 128), number of contiguous tile ranges the H * n_tiles tiles are cut into, query-row groups
  * per range (B <= 128: one; else of 256 rows, each worked on by a pair of CTAs, so that CTAs =
  * 2 * ranges * row_groups) and partial slots written per (request, head).  schedule:
@@ -27,7 +27,7 @@ extern "C" {
  * size over all heads ("stream-K").  Host, pure (a function of the sizes only, so the decomposition
  * and with it the summation order are reproducible).  INVALID_ARG for B < 1, L_s < 1, unsupported H
  * or schedule outside 0..2; no output is written then. */
-int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms, int32_t absorb_beside,
+int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms, int32_t suffix_tokens,
                            int32_t* tile_tokens /* host */, int32_t* n_ranges /* host */,
                            int32_t* row_groups /* host */, int32_t* n_slots /* host */);
 

@@ -363,10 +363,10 @@ def typhoon_mla_cost_model(dims: Dims, kind: int, B: int, S_q: int, L_s: int, L_
     return m.value, w.value
 
 
-def typhoon_mla_naive_plan(num_heads: int, B: int, L_s: int, schedule: int = 0, num_sms: int = 0, absorb_beside: bool = True):
+def typhoon_mla_naive_plan(num_heads: int, B: int, L_s: int, schedule: int = 0, num_sms: int = 0, suffix_tokens: int = 256):
     """(tile_tokens, n_ranges, row_groups, n_slots) of the shared-prefix kernel's work decomposition."""
     t, r, g, sl = C.c_int32(), C.c_int32(), C.c_int32(), C.c_int32()
-    _check(_lib.typhoon_mla_naive_plan(num_heads, B, L_s, schedule, num_sms, int(absorb_beside), C.byref(t), C.byref(r), C.byref(g),
+    _check(_lib.typhoon_mla_naive_plan(num_heads, B, L_s, schedule, num_sms, suffix_tokens, C.byref(t), C.byref(r), C.byref(g),
                                        C.byref(sl)),
            "typhoon_mla_naive_plan")
     return t.value, r.value, g.value, sl.value

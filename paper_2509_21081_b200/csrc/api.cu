@@ -300,7 +300,7 @@ Plan make_plan(const typhoon_mla_shared* sh, bool tc, int schedule, int B, int m
             p.n_slots_naive = naive_slots_override;
         } else if (use_naive && tc) {   // n_split_naive = tile ranges
             naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), schedule, &p.n_split_naive, &p.n_slots_naive, sh->fp8 != 0,
-                             use_absorb && cap > 0, max_slots);
+                             use_absorb ? absorb_branch_us(B, H, cap) : 0.0, max_slots);
         } else {
             p.n_split_naive = use_naive ? naive_splits(B, H, sh->Ls, n_sm, max_slots) : 0;
             p.n_slots_naive = p.n_split_naive;
@@ -387,13 +387,15 @@ double typhoon_mla_batch_threshold(const typhoon_mla_dims_t* d, int32_t S_q, dou
     return (d_qk + d->d_v) / ((double)S_q * (2.0 * d->kv_lora_rank + d->d_rope)) * (T / M);
 }
 
-int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms, int32_t absorb_beside,
+int typhoon_mla_naive_plan(int32_t num_heads, int32_t B, int64_t L_s, int32_t schedule, int32_t num_sms, int32_t suffix_tokens,
                            int32_t* tile_tokens, int32_t* n_ranges, int32_t* row_groups, int32_t* n_slots) {
-    if (B < 1 || L_s < 1 || L_s > (int64_t)1 << 30 || schedule < 0 || schedule > 2 || num_sms < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (B < 1 || L_s < 1 || L_s > (int64_t)1 << 30 || schedule < 0 || schedule > 2 || num_sms < 0 || suffix_tokens < 0)
+        return TYPHOON_MLA_ERR_INVALID_ARG;
     if (num_heads < 16 || num_heads > 128 || num_heads % 16) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (!tile_tokens || !n_ranges || !row_groups || !n_slots) return TYPHOON_MLA_ERR_INVALID_ARG;
     int r = 0, sl = 0;
-    naive_sm100_plan(B, num_heads, L_s, naive_places(B, num_sms > 0 ? num_sms : kDefaultNumSM, false), schedule, &r, &sl, false, absorb_beside != 0);
+    const int places = naive_places(B, num_sms > 0 ? num_sms : kDefaultNumSM, false);
+    naive_sm100_plan(B, num_heads, L_s, places, schedule, &r, &sl, false, absorb_branch_us(B, num_heads, suffix_tokens));
     *tile_tokens = naive_sm100_tile_tokens(B);
     *n_ranges = r;
     *row_groups = B <= 128 ? 1 : (B + 255) / 256;
@@ -1161,7 +1163,9 @@ struct TreePlan {
     EmptySlots empties[kMaxTreeJobs];
     int n_jobs = 0, n_empties = 0, total_slots = 0;
 };
-// `beside`: the step has an absorb branch.
+// `beside`: the step has an absorb branch.  (It is taken to have kTreeSuffix tokens per request whatever the table holds: the slots
+// must not depend on the width, or a narrower table could need more of them than the workspace was sized for.)
+constexpr int64_t kTreeSuffix = 512;
 int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int schedule, bool beside, TreePlan* tp) {
     if (!levels || n_levels < 1 || n_levels > kMaxLevels || B < 1) return TYPHOON_MLA_ERR_INVALID_ARG;
     for (int l = 0; l < n_levels && !tp->sh0; ++l) {
@@ -1210,8 +1214,9 @@ int plan_tree(const typhoon_mla_prefix_level_t* levels, int n_levels, int B, int
             naive_sm100_plan_multi(rows, H, len, n, n_sm, schedule, &ranges, &slots_of[j]);
         } else {
             const bool fp8 = tp->jobs[j].sh->fp8 != 0;
-            naive_sm100_plan(tp->jobs[j].rows, H, tp->jobs[j].sh->Ls, naive_places(tp->jobs[j].rows, n_sm, fp8), schedule, &ranges, &slots_of[j],
-                             fp8, beside);
+            const int rows = tp->jobs[j].rows, places = naive_places(rows, n_sm, fp8);
+            naive_sm100_plan(rows, H, tp->jobs[j].sh->Ls, places, schedule, &ranges, &slots_of[j], fp8,
+                             beside ? absorb_branch_us(B, H, kTreeSuffix) : 0.0);
         }
         for (int k = 0; k < n; ++k) tp->jobs[j + k].n_ranges = ranges;
         tp->jobs[j].n_merged = n;

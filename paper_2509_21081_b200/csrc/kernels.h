@@ -146,10 +146,18 @@ int naive_sm100_tile_tokens(int B, bool fp8 = false);   // KV tile width the ker
 // schedule: 0 = chosen by the plan, 1 = column split, 2 = stream-K
 inline bool naive_uses_pairs(int B, bool fp8) { return !fp8 && B > 128; }
 inline int naive_places(int B, int n_sm, bool fp8) { return naive_uses_pairs(B, fp8) ? n_sm / 2 : n_sm; }
-// beside: the absorb branch of the step runs beside the launch (else nothing does).  max_slots (>= 1): the plan chooses no more
-// partial slots than that.
-void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, bool beside,
+// absorb_us: SM time of the absorb branch that runs beside the launch (absorb_branch_us; 0: nothing does; only more than 128 rows of
+// the 16-bit cache ask for it).  max_slots (>= 1): the plan chooses no more partial slots than that.
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, double absorb_us,
                       int max_slots = INT32_MAX);
+// An upper estimate of the SM time (us) that query absorption and absorb attention of a hybrid step take, for suffixes as long as the
+// page table holds (the lengths are on the device): 4 us per head and 128 requests; per request 10 us and 1.25 us per 128-token tile on
+// a pair of SMs, or 7.5 us and 1.35 us per 64-token tile on one (launch, set-up, merge and projection in the constant part).
+inline double absorb_branch_us(int B, int H, int64_t cap_suffix) {
+    if (cap_suffix <= 0) return 0.0;
+    const double item = H > 64 ? 2.0 * (10.0 + 1.25 * (double)((cap_suffix + 127) / 128)) : 7.5 + 1.35 * (double)cap_suffix / 64.0;
+    return 4.0 * H * ((B + 127) / 128) + B * item;
+}
 cudaError_t launch_naive_attn_sm100(const NaiveAttnSm100& a, cudaStream_t s);
 // ... its form for more than 128 rows of the 16-bit cache: 256 rows per pair of CTAs
 cudaError_t launch_naive_pair_sm100(const NaiveAttnSm100& a, cudaStream_t s);

@@ -900,7 +900,7 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // along the sequence without divisions (16 prefixes x 128 heads: 8 us; a pass per prefix with a division per tile
 // count and range took 159).
 static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots, bool fp8,
-                          bool beside, int max_slots) {
+                          double absorb_us, int max_slots) {
     // (8-bit cache: always 64-token tiles, row groups of 128 requests)
     const bool mode_y = fp8 || B <= 128;
     const int tok = mode_y ? 64 : 128;
@@ -939,29 +939,31 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
         return most;
     };
     // More than 128 rows of the 16-bit cache (a place is a pair of SMs; costs in tiles of 0.9 us).  Ranges may also hold several whole
-    // heads (one segment each, one slot per head).  By itself a choice is charged its time.  Beside the absorb branch it is charged
-    // 15 % of its time and 85 % of its SM time, since the places that it leaves free go to that branch, and up to 8 tiles in the
-    // measure in which they do not suffice to get the query absorption (8 us per head and 128 requests) done meanwhile, because the
-    // branch's chain of launches then starts behind this kernel.  (The constants are the best of a search over 96 shapes, 129 to 1024
-    // rows, 16 to 128 heads, 69 to 27000 tokens, every cut measured: on average the choice is 0.8 % behind the best cut beside the
-    // branch and 0.1 % by itself.  B200, us per step: 198 rows x 128 heads, 244 + 138 tokens, two waves of 64 places 88, 32 places
-    // 78; 310 x 48, 2108 + 533, 37 x 2 equal ranges 142, 16 x 2 110; 166 x 16, 7069 + 1537, 64 places 74, 32 69; 216 x 96, 15590 +
-    // 221, 74 places 253, 48 (chosen) 266; by themselves 212 x 128, 660 tokens, two waves 35.8, 64 places 32.1.)
+    // heads (one segment each, one slot per head).  By itself a choice is charged its time.  Beside the absorb branch it is charged the
+    // time of both (all SM time over all SMs, or its own if that is longer; and 7 % of its own, for ties), and up to 16 tiles in the
+    // measure in which its free places do not suffice to get the query absorption (7 us per head and 128 requests) done meanwhile,
+    // because the branch's chain of launches then starts behind this kernel.  (The constants are from a search over 285 shapes, 129
+    // to 1024 rows, 16 to 128 heads, 69 to 27000 tokens, every cut measured: on average the choice is 0.5 % behind the best cut
+    // beside the branch, over 96 of the shapes 0.1 % by itself.  B200, us per step: 198 rows x 128 heads, 244 + 138 tokens, two waves
+    // of 64 places 88, 32 places 78; 310 x 48, 2108 + 533, 37 x 2 equal ranges 142, 16 x 2 109; 134 x 16, 26345
+    // + 35, 32 places 115, 74 equal ranges 85; 142 x 32, 563 + 832, 16 (chosen) 60, 32 places 54, the largest loss; by themselves 212
+    // x 128, 660 tokens, two waves 35.8, 64 places 32.1.)
     const bool pairs = !mode_y;
-    auto charge = [&](double cost, long long items) {   // `cost` of all waves
-        if (!pairs) return cost;
-        const double waves = (double)((items + n_sm - 1) / n_sm);
-        cost += 4.0 * (waves - 1.0);
-        if (!beside) return cost;
-        const double absorbed = cost * 0.9 * 2.0 * (n_sm - items / waves) / (8.0 * H * ((B + 127) / 128));
-        return cost * (0.15 + 0.85 * items / (waves * n_sm)) + 8.0 * (1.0 - std::min(1.0, absorbed));
+    auto charge = [&](double time, long long items) {   // `time` of all waves
+        if (!pairs) return time;
+        const double waves = (double)((items + n_sm - 1) / n_sm), used = items / waves;
+        time += 4.0 * (waves - 1.0);
+        if (absorb_us <= 0.0) return time;
+        const double both = std::max(time, (2.0 * used * time + absorb_us / 0.9) / (2.0 * n_sm));
+        const double absorbed = time * 0.9 * 2.0 * (n_sm - used) / (7.0 * H * ((B + 127) / 128));
+        return 0.07 * time + 0.93 * both + 16.0 * (1.0 - std::min(1.0, absorbed));
     };
     // column split
     const long long base = (long long)H * m_groups;
     // Cost of a range's beginning and of each further segment, in tile times.  (A pair of CTAs requests the next segment's queries
     // early and goes on with its logits while the last segment's output is written; a further wave of pairs costs a launch, its
     // set-up and a pipeline fill.)
-    const double fixed = pairs ? 12.0 : 6.0, boundary = pairs ? 3.0 : 6.0;
+    const double fixed = pairs ? 12.0 : 6.0, boundary = pairs ? 4.5 : 6.0;
     // every further partial slot is one more dependent read of B x H x 128 floats in the combine that follows
     // (about 5 us, i.e. 8 tile times, measured with 64-token tiles; with more than 128 rows the bytes count: 512 per row and
     // head at 5 TB/s, in tiles of 0.9 us)
@@ -1014,12 +1016,13 @@ static void plan_sequence(int B, int H, const int64_t* Ls, int n, int n_sm, int 
     if (R != r_stream) fill_slots(R);   // the kernel uses the same partition
 }
 
-void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, bool beside, int max_slots) {
-    plan_sequence(B, H, &Ls, 1, places, schedule, n_ranges, n_slots, fp8, beside, max_slots);
+void naive_sm100_plan(int B, int H, int64_t Ls, int places, int schedule, int* n_ranges, int* n_slots, bool fp8, double absorb_us,
+                      int max_slots) {
+    plan_sequence(B, H, &Ls, 1, places, schedule, n_ranges, n_slots, fp8, absorb_us, max_slots);
 }
 
 void naive_sm100_plan_multi(int max_rows, int H, const int64_t* Ls, int n, int n_sm, int schedule, int* n_ranges, int* n_slots) {
-    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false, true, INT32_MAX);
+    plan_sequence(max_rows, H, Ls, n, n_sm, schedule, n_ranges, n_slots, false, 0.0, INT32_MAX);
 }
 
 

@@ -87,7 +87,7 @@ extern "C" int typhoon_mla_naive_shared_noalloc(const typhoon_mla_shared_t* sh, 
     const int n_sm = sh->num_sms > 0 ? sh->num_sms : 148;
     int n_ranges = 0, n_slots = 0;
     if (sh->Ls > 0) {
-        naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), 0, &n_ranges, &n_slots, sh->fp8 != 0, false);
+        naive_sm100_plan(B, H, sh->Ls, naive_places(B, n_sm, sh->fp8 != 0), 0, &n_ranges, &n_slots, sh->fp8 != 0, 0.0);
         if ((size_t)n_slots * per_split > kScratchBytes) {
             n_ranges = H;
             n_slots = 1;

@@ -183,13 +183,14 @@ def test_naive_plan_invariants(b):
             b.typhoon_mla_naive_plan(*bad)
 
 
-@pytest.mark.parametrize("H,B,L_s,beside,alone", [
+@pytest.mark.parametrize("H,B,L_s,suffix,beside,alone", [
     # ranges that were measured (B200) to be the fastest cut beside the absorb branch, or within 2 % of it, and by themselves: a
-    # part of the places beside the branch, one wave of them alone
-    (128, 198, 244, 32, 64), (48, 310, 2108, 24, 37), (64, 182, 602, 32, 64), (128, 258, 194, 16, 32), (128, 212, 660, 32, 64), (64, 256, 8192, 64, 74)])
-def test_more_than_128_rows_leave_places_to_the_absorb_branch(b, H, B, L_s, beside, alone):
-    assert b.typhoon_mla_naive_plan(H, B, L_s)[1] == beside
-    assert b.typhoon_mla_naive_plan(H, B, L_s, absorb_beside=False)[1] == alone
+    # part of the places beside the branch, one wave of them alone; but all of them where the branch is short
+    (128, 198, 244, 192, 32, 64), (128, 258, 194, 256, 16, 32), (128, 212, 660, 64, 32, 64), (64, 256, 8192, 4096, 64, 64), (16, 166, 7069, 1664, 16, 64), (48, 310, 2108, 576, 16, 37),
+    (16, 134, 26345, 64, 74, 74), (48, 243, 17898, 128, 74, 74), (128, 1024, 16384, 256, 16, 18)])
+def test_more_than_128_rows_leave_places_to_the_absorb_branch(b, H, B, L_s, suffix, beside, alone):
+    assert b.typhoon_mla_naive_plan(H, B, L_s, suffix_tokens=suffix)[1] == beside
+    assert b.typhoon_mla_naive_plan(H, B, L_s, suffix_tokens=0)[1] == alone
 
 
 @pytest.mark.parametrize("H,B,slots,early", [(128, 64, 1, 1), (128, 128, 2, 1), (128, 129, 2, 0), (128, 198, 1, 0), (128, 1024, 1, 0),
