@@ -167,7 +167,8 @@ bool many_heads_use_pairs(int B, int64_t cap_suffix, bool beside_prefix) {
     return !(beside_prefix && B <= 128 && (cap_suffix <= 64 || (cap_suffix <= 256 && B > 64)));
 }
 
-// Kernel and chunk length of the absorb attention.  max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks.
+// Kernel and chunk length of the absorb attention.  cap_suffix: the page table's width in tokens (the suffixes' lengths are on the device).
+// max_chunks: at least one per non-empty segment, at most kMaxAbsorbChunks.
 // `beside_prefix`: a shared-prefix launch runs beside it.
 void absorb_chunks(bool tc, bool stacked, bool beside_prefix, int n_sm, int B, int H, int64_t Ls_absorb, int64_t cap_suffix, int max_chunks,
                    bool* pairs, int* chunk, int* n_sh, int* n_sf) {
@@ -843,8 +844,10 @@ size_t typhoon_mla_workspace_bytes(const typhoon_mla_shared_t* sh, int32_t B, in
 int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8bit, int32_t B, int32_t max_pages, int32_t page_size,
                                int32_t mode, int32_t path, int32_t schedule, int32_t stacked, int32_t num_sms, size_t workspace_bytes,
                                size_t* query, size_t* step, int32_t* n_chunks, int32_t* n_slots, int32_t* absorb_pairs) {
-    if (num_heads < 16 || num_heads > 128 || num_heads % 16 || L_s < 0 || L_s > (int64_t)1 << 24 || B < 1 || max_pages < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
-    if ((page_size != 64 && page_size != 128) || mode < TYPHOON_MLA_MODE_AUTO || mode > TYPHOON_MLA_MODE_NAIVE) return TYPHOON_MLA_ERR_INVALID_ARG;
+    if (num_heads < 16 || num_heads > 128 || num_heads % 16 || L_s < 0 || L_s > (int64_t)1 << 24 || B < 1 || max_pages < 0)
+        return TYPHOON_MLA_ERR_INVALID_ARG;
+    if ((page_size != 64 && page_size != 128) || mode < TYPHOON_MLA_MODE_AUTO || mode > TYPHOON_MLA_MODE_NAIVE)
+        return TYPHOON_MLA_ERR_INVALID_ARG;
     if (path < 0 || path > 1 || schedule < 0 || schedule > 2 || num_sms < 0) return TYPHOON_MLA_ERR_INVALID_ARG;
     if (!query || !step || !n_chunks || !n_slots || !absorb_pairs) return TYPHOON_MLA_ERR_INVALID_ARG;
     typhoon_mla_shared sh{};
@@ -854,8 +857,9 @@ int typhoon_mla_workspace_plan(int32_t num_heads, int64_t L_s, int32_t prefix_8b
     sh.num_sms = num_sms;
     *query = query_bytes(&sh, B, max_pages, page_size, mode);
     const int m = resolve_mode(&sh, B, max_pages, mode);
-    const Plan p = make_plan(&sh, path == TYPHOON_MLA_PATH_TCGEN05, schedule, B, m == TYPHOON_MLA_MODE_NAIVE ? 0 : max_pages, page_size, m, -1,
-                             stacked != 0, workspace_bytes > 0 ? workspace_bytes : SIZE_MAX);
+    const int pages = m == TYPHOON_MLA_MODE_NAIVE ? 0 : max_pages;
+    const Plan p = make_plan(&sh, path == TYPHOON_MLA_PATH_TCGEN05, schedule, B, pages, page_size, m, -1, stacked != 0,
+                             workspace_bytes > 0 ? workspace_bytes : SIZE_MAX);
     *step = p.total;
     *n_chunks = p.n_shared_chunks + p.n_suffix_chunks;
     *n_slots = p.n_slots_naive;
@@ -1259,7 +1263,8 @@ size_t typhoon_mla_tree_workspace_bytes(const typhoon_mla_prefix_level_t* levels
             TreePlan tp;
             if (plan_tree(levels, n_levels, B, schedule, beside, &tp) != TYPHOON_MLA_OK) return 0;
             for (size_t bytes : {SIZE_MAX, (size_t)0})
-                worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots, true, bytes).total);
+                worst = std::max(worst, make_plan(tp.sh0, true, schedule, B, max_pages, page_size, TYPHOON_MLA_MODE_HYBRID, tp.total_slots, true,
+                                                  bytes).total);
         }
     return worst + 256;
 }
