@@ -892,8 +892,9 @@ int naive_sm100_tile_tokens(int B, bool fp8) { return (fp8 || B <= 128) ? 64 : 1
 // times for the Q load and the pipeline fill).  "Stream-K" uses R = SMs / row groups resident
 // CTAs and gives every SM the same number of tiles at the price of a few more segments (each
 // pays the fixed cost and a partial slot; a further slot per head is also charged the extra read it
-// causes in the combine).  Stream-K is taken when its modelled cost is lower by at least 5%.  (With more than
-// 128 rows of the 16-bit cache a place is a pair of SMs, see naive_pair_sm100.cu.)
+// causes in the combine).  Stream-K is taken when its modelled cost is lower by at least 5%.  With more than 128 rows
+// of the 16-bit cache a place is a pair of SMs (naive_pair_sm100.cu), ranges of several whole heads are weighed too, the
+// absorb branch beside the launch enters the costs, and the lowest one is taken.
 //
 // `n` prefixes (at most kNaiveJobsPerLaunch, of Ls[i] tokens): the sequence holds all prefixes' tiles of a head, then the next
 // head's; n_slots[i] are the slots of prefix i.  Runs on every call of a step, so the slots of all prefixes come from one walk
